@@ -88,6 +88,7 @@ def measured_peaks():
 # The sources of the bulk sweep kernel: a recorded ncu traffic figure is used
 # only while their hash equals the one recorded with it.
 KERNEL_SOURCES = ("paper_1305_3440_gb300/csrc/lgt_sweep.cuh", "paper_1305_3440_gb300/csrc/lgt_sweep_f32.cu",
+                  "paper_1305_3440_gb300/csrc/lgt_fixed.cuh", "paper_1305_3440_gb300/csrc/lgt_sweep_fixed.cu",
                   "paper_1305_3440_gb300/csrc/lgt_device.cuh", "paper_1305_3440_gb300/csrc/lgt_anchor.cuh",
                   "paper_1305_3440_gb300/csrc/lgt_pair.cuh", "paper_1305_3440_gb300/csrc/lgt_internal.h")
 
@@ -182,16 +183,19 @@ class ClockSampler:
 
 
 def algorithmic_bytes_per_site(kind: str) -> int:
-    """Bytes one site update must move.  Bulk: its 8 links in and out plus G(x) in
-    and out (FP32-12 links 48 B, FP32-18 72 B, G stored as 2 rows: 48 B).
-    FP32-pair and FP64 polish: 8 links of 144 B in and out.  Anchored polish:
-    K0(x) (144 B) and the 8 links' FP32-12 copies (384 B) in, its own D (96 B:
-    rows 0, 1 as pairs) in and out, and the other parity's D high parts (48 B
-    per site: each is read by 8 neighbours, compulsory once)."""
+    """Bytes one site update must move.  Bulk (the links stay as loaded): its 8 links
+    in (FP32-12 48 B, FP32-18 72 B; Coulomb gauge 6), G(x) in and out (2 rows: 48
+    B) and the other parity's G (48 B per site: each is read by 8 neighbours,
+    compulsory once).  FP32-pair and FP64 polish: 8 links of 144 B in and out.
+    Anchored polish: K0(x) (144 B) and the 8 links' FP32-12 copies (384 B) in, its
+    own D (96 B: rows 0, 1 as pairs) in and out, and the other parity's D high parts
+    (48 B per site)."""
     if kind == "fp32_12":
-        return 16 * 48 + 2 * 48
+        return 8 * 48 + 3 * 48
+    if kind == "fp32_12_coulomb":
+        return 6 * 48 + 3 * 48
     if kind == "fp32_18":
-        return 16 * 72 + 2 * 48
+        return 8 * 72 + 3 * 48
     if kind == "anchor":
         return 144 + 8 * 48 + 48 + 2 * 96
     if kind == "anchor_coulomb":  # spatial directions only
@@ -417,7 +421,7 @@ def run_ours(args):
     d = kernels[dom]
     roofline = {"bound": "hbm", "achieved": d["achieved_gbs"], "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": d["achieved_gbs"] / peaks["hbm_gbs"],
-                "traffic": recorded_traffic("k_sweep_f32" if dom == "fp32_12" else "k_sweep_anchor",
+                "traffic": recorded_traffic("k_sweep_fixed" if dom == "fp32_12" else "k_sweep_anchor",
                                             d["launch_config"]),
                 "kernel": f"half-sweep {dom}", "peak_source": src,
                 "bytes_per_site_update": algorithmic_bytes_per_site(dom), "units_per_launch": vol // 2}
@@ -592,7 +596,7 @@ def run_coulomb(args):
     t = float(np.median(times))
     updates = stats.site_updates[0] + stats.site_updates[1]
     peaks, src = measured_peaks()
-    kern = _kernel_summary(stats, 12 * 48 + 2 * 48 + 4 * 48, algorithmic_bytes_per_site("anchor_coulomb"), vol)
+    kern = _kernel_summary(stats, algorithmic_bytes_per_site("fp32_12_coulomb"), algorithmic_bytes_per_site("anchor_coulomb"), vol)
     line = {"workload": "coulomb", "metric": "time to max_t theta_t<1e-14 (s)", "value": t, "unit": "s",
             "higher_is_better": False, "steps": args.steps, "warmup": args.warmup,
             "config": {"workload": "SU(3) Coulomb 48^3x96, eps=0.5, seed 3, OR omega=1.7, FP32-12 bulk + "
@@ -625,7 +629,7 @@ def run_landau64(args):
         lgt.lgt_destroy(ctx)
         out[name] = {"status": st, "seconds": t, "sweeps_bulk": res.sweeps_bulk, "sweeps_polish": res.sweeps_fp64,
                      "F": res.F, "theta": res.theta, "site_updates_per_s": (res.sweeps_bulk + res.sweeps_fp64) * vol / t,
-                     "kernels": _kernel_summary(stats, 16 * 48 + 2 * 48, algorithmic_bytes_per_site("anchor"), vol)}
+                     "kernels": _kernel_summary(stats, algorithmic_bytes_per_site("fp32_12"), algorithmic_bytes_per_site("anchor"), vol)}
     p = lgt.lgt_params_default(dims=dims, bulk=lgt.LGT_FP64, omega=1.8)
     ctx = lgt.lgt_create(p, dev, stream=stream)
     lgt.lgt_sweep(ctx, 2)
@@ -660,8 +664,8 @@ def run_landau64(args):
 def run_mag(args):
     """Maximally Abelian gauge.  The bulk sweep rate on the 32^4 field of the headline
     workload (FP32-12 links, OR omega 1.7; 20 sweeps untimed, then 200 sweeps timed by
-    the sweep kernels' CUDA events; algorithmic bytes per site as the Landau bulk
-    kernel: the 8 links and G read and written once, 864 B) and the FP64 sweep rate
+    the sweep kernels' CUDA events; algorithmic bytes per site: the 8 links and G read
+    and written once, 864 B) and the FP64 sweep rate
     of the same field; then a 16^4 field (eps 0.5, seed 3) fixed to theta_MAG < 1e-12
     through the ladder, and an 8^4 gauge-transformed Abelian field fixed back to
     F_MAG = 1."""
@@ -673,7 +677,7 @@ def run_mag(args):
     dims = (32, 32, 32, 32)
     vol = int(np.prod(dims))
     dev = torch.from_numpy(synth.field(dims, 0.5, 2)).cuda()
-    for name, bulk, bytes_per_site in [("bulk_fp32_12", lgt.LGT_FP32_12, algorithmic_bytes_per_site("fp32_12")),
+    for name, bulk, bytes_per_site in [("bulk_fp32_12", lgt.LGT_FP32_12, 16 * 48 + 2 * 48),
                                        ("fp64", lgt.LGT_FP64, 2304)]:
         p = lgt.lgt_params_default(dims=dims, gauge=lgt.LGT_MAG, bulk=bulk, omega=1.7)
         ctx = lgt.lgt_create(p, dev, stream=stream)

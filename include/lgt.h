@@ -214,6 +214,17 @@ typedef struct {
  *                        14: 64 threads, <= 128 registers (8 blocks per SM);
  *                        15: 64 threads, <= 112 registers (9 blocks per SM),
  *                            the links staged and G loaded into registers.
+ * With neither launch_config nor block_size given, FP32 overrelaxation (bulk
+ * and annealing) sweeps in Landau and Coulomb gauge (whole lattices; jobs of a
+ * server always) use none of these: they keep the FP32 links as loaded and update the accumulated
+ * transformation G alone, K(x) = G(x) sum_mu [U_mu(x) G(x+mu)^+ +
+ * U_mu(x-mu)^+ G(x-mu)^+], which is the K(x) of the rewritten links G U G^+;
+ * tuned over the thread and register budgets of 3, 8 and 9.  The working links
+ * are then G U G^+ formed in FP32 when they are asked for or measured.  FP32
+ * rounding leaves such a field at theta ~ 6e-13 (rewritten links: 3e-14) but the
+ * input transformed by G there too (rewritten links: 1e-8, G and the links
+ * drifting apart), so the bulk phase of lgt_fix and of served jobs ends at theta <
+ * max(theta_switch, 2e-12).
  * The anchored polish (the default after promotion) runs in 0-3 and in 11
  * (<= 80 registers, 24 warps per SM).  A configuration that a phase's kernel
  * lacks (4-15 after promotion, except 11 for the anchored polish; 7, 10 and
@@ -304,8 +315,9 @@ LGT_API lgt_status lgt_promote(lgt_ctx *ctx);
  * (out_on_device = 0) or device memory of V*4*9*2 doubles. */
 LGT_API lgt_status lgt_get_links(lgt_ctx *ctx, double *out, int out_on_device);
 
-/* The working links as stored (bulk phase: FP32 widened to FP64, 12-real
- * storage with its third row rebuilt; FP64 phase: as lgt_get_links). */
+/* The working links (bulk phase: FP32 widened to FP64, 12-real storage with its
+ * third row rebuilt -- as stored, or, with fixed-link sweeps, G U G^+ formed in
+ * FP32 from the stored links and G; FP64 phase: as lgt_get_links). */
 LGT_API lgt_status lgt_get_working_links(lgt_ctx *ctx, double *out, int out_on_device);
 
 /* Sweeps run so far (bulk FP32; after promotion) and the phase: 0 bulk

@@ -220,6 +220,8 @@ struct lgt_ctx {
   void *u64;      // FP64 links (the input while in the bulk phase)
   void *u32;      // bulk working links
   void *G;        // accumulated transformation of the bulk phase; D = G - 1 of the anchored polish
+  int fixed;      // the bulk sweeps keep the links in u32 as loaded and update G alone (lgt_fixed_links)
+  int g_dirty;    // fixed: G != 1, the working links are G u32 G^+
   void *k0;       // anchored polish: K0 (pairs)
   int anchored;   // anchored polish: K0, the FP32-12 copy in u32 and D refer to the field in u64
   int d_dirty;    // anchored polish: D != 0 (sweeps since the field in u64 was last formed)
@@ -383,7 +385,7 @@ static lgt_status load_field(lgt_ctx *c, const double *links, int links_on_devic
     return LGT_EINVAL;
   }
   c->phase = c->prm.bulk == LGT_FP64 ? 1 : 0;
-  c->anchored = c->d_dirty = 0;
+  c->anchored = c->d_dirty = c->g_dirty = 0;
   c->sa_pending = c->prm.sa_sweeps > 0;
   c->active_slices = g.nt;
   c->cfg.omega = c->prm.omega;  // omega_late may take over (omega schedule), omega_polish at promotion
@@ -394,8 +396,10 @@ static lgt_status load_field(lgt_ctx *c, const double *links, int links_on_devic
   return LGT_OK;
 }
 
-extern "C" lgt_status lgt_create(const lgt_params *params, const double *links, int links_on_device,
-                                 void *cuda_stream, lgt_ctx **out) {
+// slab: the context of a temporal slab (its bulk sweeps rewrite the links, which
+// slabs exchange)
+static lgt_status create_context(const lgt_params *params, const double *links, int links_on_device, void *cuda_stream,
+                                 bool slab, lgt_ctx **out) {
   if (!out) {
     lgt_set_error("out is NULL");
     return LGT_EINVAL;
@@ -431,6 +435,9 @@ extern "C" lgt_status lgt_create(const lgt_params *params, const double *links, 
   c->cfg.seed = params->seed;
   c->cfg.transform_temporal = params->transform_temporal ? 1 : 0;
   const Geom &g = c->g;
+  // a forced launch configuration or block size names a kernel that rewrites the links
+  c->fixed = !slab && params->launch_config == 0 && params->block_size == 0 && params->bulk != LGT_FP64 &&
+             lgt_fixed_links(c->bulk_fmt, c->cfg.gauge, c->cfg.algo, g);
 #define CTX_CUDA(call)                                                                         \
   do {                                                                                         \
     cudaError_t e_ = (call);                                                                   \
@@ -474,7 +481,9 @@ extern "C" lgt_status lgt_create(const lgt_params *params, const double *links, 
     c->cfg_polish = lgt_cfg_supported_gauge(polish_fmt, c->cfg.gauge, k) ? k : 0;
   } else if (!params->block_size) {
     cudaError_t te = cudaSuccess;
-    if (c->u32) c->cfg_bulk = lgt_tune_sweep(g, c->bulk_fmt, c->cfg, c->u32, c->G, c->ws, c->stream, &te);
+    if (c->u32)
+      c->cfg_bulk = lgt_tune_sweep(g, c->fixed ? lgt_fixed_fmt(c->bulk_fmt) : c->bulk_fmt, c->cfg, c->u32, c->G, c->ws,
+                                   c->stream, &te);
     if (te == cudaSuccess) {
       if (polish_fmt == FMT_ANCHOR)
         c->cfg_polish = lgt_tune_sweep(g, polish_fmt, c->cfg, c->u32, c->G, c->ws, c->stream, &te, c->k0);
@@ -493,6 +502,11 @@ extern "C" lgt_status lgt_create(const lgt_params *params, const double *links, 
   }
   *out = c;
   return LGT_OK;
+}
+
+extern "C" lgt_status lgt_create(const lgt_params *params, const double *links, int links_on_device,
+                                 void *cuda_stream, lgt_ctx **out) {
+  return create_context(params, links, links_on_device, cuda_stream, false, out);
 }
 
 // A slab's local field in public layout in the staging buffer: the two halo
@@ -543,11 +557,19 @@ extern "C" void lgt_destroy(lgt_ctx *ctx) {
 // ------------------------------------------------------------------ sweeps
 // half-sweeps [first_parity .. first_parity + n_half) (parity alternating);
 // the sweep counter advances after each odd half
-// storage format (and kernel) of the working field in the current phase
 // storage format of the working field (the anchored polish measures the
 // formed field in u64, FP64)
 static int work_fmt(const lgt_ctx *c) {
   return c->phase == 0 ? c->bulk_fmt : (c->phase == 2 ? (int)FMT_PAIR : (int)FMT_F64);
+}
+// kernel format of the current phase's sweeps
+static int sweep_fmt(const lgt_ctx *c) {
+  return c->phase == 3 ? (int)FMT_ANCHOR : (c->phase == 0 && c->fixed ? lgt_fixed_fmt(c->bulk_fmt) : work_fmt(c));
+}
+// format in which measurements and output read the working field: as stored, or
+// formed from the links and G once fixed-link sweeps have run
+static int read_fmt(const lgt_ctx *c) {
+  return c->phase == 0 && c->fixed && c->g_dirty ? lgt_fixed_fmt(c->bulk_fmt) : work_fmt(c);
 }
 
 static int skip_temporal(const lgt_ctx *c) {
@@ -583,7 +605,7 @@ static lgt_status anchor_refresh(lgt_ctx *c) {
 
 static lgt_status run_halves(lgt_ctx *c, int first_parity, int n_half, int use_mask) {
   const bool anch = c->phase == 3;
-  const int fmt = anch ? (int)FMT_ANCHOR : work_fmt(c);
+  const int fmt = sweep_fmt(c);
   void *links = (c->phase == 0 || anch) ? c->u32 : c->u64;
   void *G = ((c->phase == 0 && !c->slab) || anch) ? c->G : nullptr;  // a slab is never promoted
   const int kind = c->phase == 0 ? 0 : 1;
@@ -593,6 +615,7 @@ static lgt_status run_halves(lgt_ctx *c, int first_parity, int n_half, int use_m
     if (st != LGT_OK) return st;
     c->d_dirty = 1;
   }
+  if (c->phase == 0) c->g_dirty = 1;
   const int bt = batch_begin(c, kind);
   const int lc = c->phase == 0 ? c->cfg_bulk : c->cfg_polish;
   const int reunit_every = c->phase == 0 ? c->prm.reunit_every : 0;
@@ -670,11 +693,10 @@ static void fill_meas(const lgt_ctx *c, const double *t, Meas *m) {
 static lgt_status measure(lgt_ctx *c, int with_plaq, double coulomb_target, Meas *m) {
   lgt_status mst = anchor_materialise(c);
   if (mst != LGT_OK) return mst;
-  const int fmt = work_fmt(c);
   const void *links = c->phase == 0 ? c->u32 : c->u64;
   const int bt = batch_begin(c, 2);
-  LGT_CUDA(launch_measure(fmt, c->g, links, c->ws, with_plaq, coulomb_target, 128, c->stream,
-                          c->prm.gauge == LGT_MAG ? 1 : 0));
+  LGT_CUDA(launch_measure(read_fmt(c), c->g, links, c->ws, with_plaq, coulomb_target, 128, c->stream,
+                          c->prm.gauge == LGT_MAG ? 1 : 0, c->G, skip_temporal(c)));
   batch_end(c, bt);
   c->stats.measure_launches++;
   c->stats.launches++;
@@ -860,7 +882,7 @@ extern "C" lgt_status lgt_slab_create(const lgt_params *params, int32_t nt_globa
     return e == cudaErrorMemoryAllocation ? LGT_ENOMEM : LGT_ECUDA;
   }
   lgt_ctx *c = nullptr;
-  st = lgt_create(&local, buf, 1, cuda_stream, &c);
+  st = create_context(&local, buf, 1, cuda_stream, true, &c);
   cudaFreeAsync(buf, stream);
   cudaStreamSynchronize(stream);
   if (st != LGT_OK) return st;
@@ -975,8 +997,8 @@ extern "C" lgt_status lgt_measure_slice_sums(lgt_ctx *ctx, double *sums) {
   lgt_status st = anchor_materialise(c);
   if (st != LGT_OK) return st;
   const int bt = batch_begin(c, 2);
-  LGT_CUDA(launch_measure(work_fmt(c), c->g, c->phase == 0 ? c->u32 : c->u64, c->ws, 1, -1.0, 128, c->stream,
-                          c->prm.gauge == LGT_MAG ? 1 : 0));
+  LGT_CUDA(launch_measure(read_fmt(c), c->g, c->phase == 0 ? c->u32 : c->u64, c->ws, 1, -1.0, 128, c->stream,
+                          c->prm.gauge == LGT_MAG ? 1 : 0, c->G, skip_temporal(c)));
   batch_end(c, bt);
   c->stats.measure_launches++;
   c->stats.launches++;
@@ -1039,13 +1061,13 @@ extern "C" lgt_status lgt_promote(lgt_ctx *ctx) {
 // change afterwards.
 static lgt_status build_loop(lgt_ctx *c, int slot) {
   const bool anch = c->phase == 3;
-  const int fmt = anch ? (int)FMT_ANCHOR : work_fmt(c);
+  const int fmt = sweep_fmt(c);
   void *links = (c->phase == 0 || anch) ? c->u32 : c->u64;
   void *G = (c->phase == 0 || anch) ? c->G : nullptr;
   const int lc = c->phase == 0 ? c->cfg_bulk : c->cfg_polish;
   const int k = c->prm.check_every;
   const bool coulomb = c->prm.gauge == LGT_COULOMB;
-  const double target = slot == 0 ? c->prm.theta_switch : c->prm.theta_tol;
+  const double target = slot == 0 ? lgt_bulk_target(c->fixed, c->prm.theta_switch) : c->prm.theta_tol;
   cudaGraph_t graph = nullptr;
   cudaGraphConditionalHandle h;
   cudaGraphNodeParams cp = {};
@@ -1101,12 +1123,13 @@ static lgt_status run_loop(lgt_ctx *c, int slot, double *best, int *stall, int64
     if (st != LGT_OK) return st;
     c->d_dirty = 1;
   }
+  if (c->phase == 0) c->g_dirty = 1;
   LoopState &L = *c->h_loop;
   L.sweep = c->sweep_index;
   L.count = kind == 0 ? c->sweeps_bulk : c->sweeps_fp64;
   L.remaining = *remaining;
   L.site_updates = 0;
-  L.target = slot == 0 ? c->prm.theta_switch : c->prm.theta_tol;
+  L.target = slot == 0 ? lgt_bulk_target(c->fixed, c->prm.theta_switch) : c->prm.theta_tol;
   L.best = best ? *best : 0.0;
   L.theta = 0.0;
   L.stall = stall ? *stall : 0;
@@ -1168,16 +1191,18 @@ static double sa_beta(double beta0, double beta1, int n, int i) {
   return beta0 * pow(beta1 / beta0, (double)i / (double)(n - 1));
 }
 
-// The loaded field's annealing sweeps (heat bath, launch configuration 0),
+// The loaded field's annealing sweeps (heat bath, one launch configuration),
 // counted as sweeps of the current phase.
 static lgt_status run_annealing(lgt_ctx *c, int64_t *remaining) {
   const int n = (int)(c->prm.sa_sweeps < *remaining ? c->prm.sa_sweeps : *remaining);
-  const int fmt = work_fmt(c);
+  const int fmt = sweep_fmt(c);
+  const int lc = c->phase == 0 && c->fixed ? LGT_FIXED_SA_CFG : 0;
   void *links = c->phase == 0 ? c->u32 : c->u64;
   void *G = c->phase == 0 ? c->G : nullptr;
   const int kind = c->phase == 0 ? 0 : 1;
   SweepCfg sc = c->cfg;
   sc.algo = ALGO_SA;
+  if (c->phase == 0) c->g_dirty = 1;
   const int bt = batch_begin(c, kind);
   for (int i = 0; i < n; i++) {
     sc.beta = sa_beta(c->prm.sa_beta0, c->prm.sa_beta1, c->prm.sa_sweeps, i);
@@ -1188,13 +1213,13 @@ static lgt_status run_annealing(lgt_ctx *c, int64_t *remaining) {
     // reunitarises what it writes.
     const int reunit = c->phase == 0;
     for (int parity = 0; parity < 2; parity++)
-      LGT_CUDA(launch_half_sweep(fmt, c->g, links, G, c->ws, sc, parity, c->sweep_index, reunit, 0, 0, c->stream));
+      LGT_CUDA(launch_half_sweep(fmt, c->g, links, G, c->ws, sc, parity, c->sweep_index, reunit, 0, lc, c->stream));
     c->sweep_index++;
     if (kind == 0) c->sweeps_bulk++;
     else c->sweeps_fp64++;
   }
   batch_end(c, bt);
-  c->last_sites = lgt_cfg_sites(0);
+  c->last_sites = lgt_cfg_sites(lc);
   c->stats.sweep_launches[kind] += 2 * n;
   c->stats.launches += 2 * n;
   c->stats.site_updates[kind] += 2LL * n * c->g.vs_half * c->g.nt;
@@ -1229,7 +1254,7 @@ extern "C" lgt_status lgt_fix(lgt_ctx *ctx, lgt_result *res) {
   if (c->phase == 0) {
     // bulk FP32 phase: until the working field's theta drops below theta_switch
     // or stops improving (the FP32 rounding floor)
-    const double target = c->prm.theta_switch;
+    const double target = lgt_bulk_target(c->fixed, c->prm.theta_switch);
     st = measure(c, 0, coulomb ? target : -1.0, &m);
     if (st != LGT_OK) return st;
     omega_check(c, m.theta);
@@ -1342,7 +1367,7 @@ static lgt_status to_output(lgt_ctx *c, double *out, int out_on_device, int work
   cudaError_t e;
   if (c->phase == 3 && c->d_dirty) e = launch_apply_D(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->stream);
   else if (c->phase >= 1) e = launch_egress(work_fmt(c), g, c->u64, dst, c->stream);
-  else if (working) e = launch_egress(c->bulk_fmt, g, c->u32, dst, c->stream);
+  else if (working) e = launch_egress(read_fmt(c), g, c->u32, dst, c->stream, c->G, skip_temporal(c));
   else e = launch_apply_G(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->stream);
   c->stats.launches++;
   if (e == cudaSuccess && tmp) e = cudaMemcpyAsync(out, tmp, aos_bytes, cudaMemcpyDeviceToHost, c->stream);

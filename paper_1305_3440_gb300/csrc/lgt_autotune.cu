@@ -83,7 +83,7 @@ int lgt_tune_sweep(const Geom &g, int fmt, const SweepCfg &cfg, void *links, voi
     if (e == cudaSuccess) e = cudaMemsetAsync(aux, 0, k0_bytes(g.vh), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(G, 0, d_bytes(g.vh), st);
   } else {
-    e = launch_fill_unit(fmt, g, links, st);
+    e = launch_fill_unit(fmt == FMT_FIX_18 ? (int)FMT_F32_18 : (fmt == FMT_FIX_12 ? (int)FMT_F32_12 : fmt), g, links, st);
     if (e == cudaSuccess && G) e = launch_g_identity(g, G, st);
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lgt_fixed.cuh"
 #include "lgt_measure.cuh"
 #include "lgt_sweep.cuh"
 
@@ -57,7 +58,22 @@ __global__ void __launch_bounds__(256) k_measure_batch(const BatchMeas *jobs, in
   measure_body<FMT>(J.a, t, p, rem - p * J.nbx, J.nbx);
 }
 
-// FP32-18 bulk sweeps of the batch: the lean one-thread layout (K streamed,
+// FP32 overrelaxation sweeps of the batch: the fixed-link update at launch configuration
+// 8's budget (128 threads, <= 128 registers, 4 blocks per SM).
+template <int LFMT, int GAUGE, int ALGO>
+__global__ void __launch_bounds__(128, 4) k_sweep_batch_fixed(const BatchSweep *jobs, int n, int p, int s) {
+  const int b = batch_block(jobs, p);
+  const int k = batch_row(&jobs[0].block_begin, (int)sizeof(BatchSweep), n, b);
+  const BatchSweep &J = jobs[k];
+  SweepArgs a = J.a;
+  a.sweep += (unsigned long long)s;
+  a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
+  const int local = b - J.block_begin;
+  const int t = local / J.nbx;
+  sweep_body_fixed<LFMT, GAUGE, ALGO, fixed_depth(LFMT, 512)>(a, p, t, local - t * J.nbx);
+}
+
+// FP32-18 stochastic-relaxation sweeps of the batch: the lean one-thread layout (K streamed,
 // links reloaded for the write-back; <= 128 registers, 4 blocks of 128 threads
 // per SM), as launch configuration 8 of the single-lattice kernels.
 template <int FMT, int GAUGE, int ALGO>
@@ -73,7 +89,7 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_lean(const BatchSweep *j
   sweep_body_f32_lean<FMT, GAUGE, ALGO>(a, p, t, local - t * J.nbx);
 }
 
-// FP32-12 bulk sweeps of the batch: the staged one-thread layout (each site's
+// FP32-12 stochastic-relaxation sweeps of the batch: the staged one-thread layout (each site's
 // links and G copied into shared memory by one batch of cp.async, then the
 // lean update from there; 4 blocks of 128 threads per SM), as launch
 // configuration 13 of the single-lattice kernels.
@@ -123,15 +139,9 @@ static cudaError_t staged_smem(batch_fn fn, int block, int *smem) {
   return e;
 }
 
-static batch_fn pick_batch_staged(int gauge, int algo) {
-  if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_batch_staged<GAUGE_LANDAU, ALGO_SR> : k_sweep_batch_staged<GAUGE_LANDAU, ALGO_OR>;
-  return algo == ALGO_SR ? k_sweep_batch_staged<GAUGE_COULOMB, ALGO_SR> : k_sweep_batch_staged<GAUGE_COULOMB, ALGO_OR>;
-}
-
-template <int FMT>
-static batch_fn pick_batch_lean(int gauge, int algo) {
-  if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_batch_lean<FMT, GAUGE_LANDAU, ALGO_SR> : k_sweep_batch_lean<FMT, GAUGE_LANDAU, ALGO_OR>;
-  return algo == ALGO_SR ? k_sweep_batch_lean<FMT, GAUGE_COULOMB, ALGO_SR> : k_sweep_batch_lean<FMT, GAUGE_COULOMB, ALGO_OR>;
+template <int LFMT>
+static batch_fn pick_batch_fixed(int gauge) {
+  return gauge == GAUGE_LANDAU ? k_sweep_batch_fixed<LFMT, GAUGE_LANDAU, ALGO_OR> : k_sweep_batch_fixed<LFMT, GAUGE_COULOMB, ALGO_OR>;
 }
 
 template <int FMT>
@@ -143,22 +153,22 @@ static batch_fn pick_batch_fmt(int gauge, int algo) {
 cudaError_t launch_half_sweep_batch(int fmt, int gauge, int algo, const BatchSweep *jobs, int n, int total_blocks,
                                     int parity, int s, int block, cudaStream_t st) {
   if (n <= 0 || total_blocks <= 0) return cudaSuccess;
+  if (block != 128 || (gauge != GAUGE_LANDAU && gauge != GAUGE_COULOMB) || (algo != ALGO_OR && algo != ALGO_SR))
+    return cudaErrorInvalidValue;
   batch_fn fn = nullptr;
   int smem = 0;
   if (fmt == FMT_F64) fn = pick_batch_fmt<FMT_F64>(gauge, algo);
-  else if (fmt == FMT_F32_18) fn = block == 128 ? pick_batch_lean<FMT_F32_18>(gauge, algo) : pick_batch_fmt<FMT_F32_18>(gauge, algo);
-  else if (fmt == FMT_F32_12 && block == 128 && (gauge == GAUGE_LANDAU || gauge == GAUGE_COULOMB) &&
-           (algo == ALGO_OR || algo == ALGO_SR)) {
-    fn = pick_batch_staged(gauge, algo);
-    cudaError_t e = staged_smem(fn, block, &smem);
+  else if (fmt == FMT_FIX_18 && algo == ALGO_OR) fn = pick_batch_fixed<FMT_F32_18>(gauge);
+  else if (fmt == FMT_FIX_12 && algo == ALGO_OR) fn = pick_batch_fixed<FMT_F32_12>(gauge);
+  else if (fmt == FMT_F32_18 && algo == ALGO_SR)
+    fn = gauge == GAUGE_LANDAU ? k_sweep_batch_lean<FMT_F32_18, GAUGE_LANDAU, ALGO_SR> : k_sweep_batch_lean<FMT_F32_18, GAUGE_COULOMB, ALGO_SR>;
+  else if (fmt == FMT_F32_12 && algo == ALGO_SR) {
+    fn = gauge == GAUGE_LANDAU ? k_sweep_batch_staged<GAUGE_LANDAU, ALGO_SR> : k_sweep_batch_staged<GAUGE_COULOMB, ALGO_SR>;
+    const cudaError_t e = staged_smem(fn, block, &smem);
     if (e != cudaSuccess) return e;
   }
-  else if (fmt == FMT_F32_12) fn = block == 128 ? pick_batch_lean<FMT_F32_12>(gauge, algo) : pick_batch_fmt<FMT_F32_12>(gauge, algo);
   else if (fmt == FMT_PAIR) fn = pick_batch_fmt<FMT_PAIR>(gauge, algo);
-  else if (fmt == FMT_ANCHOR && block == 128 && (gauge == GAUGE_LANDAU || gauge == GAUGE_COULOMB) &&
-           (algo == ALGO_OR || algo == ALGO_SR))
-    fn = pick_batch_anchor(gauge, algo);
-  else if (fmt == FMT_ANCHOR) fn = pick_batch_fmt<FMT_ANCHOR>(gauge, algo);
+  else if (fmt == FMT_ANCHOR) fn = pick_batch_anchor(gauge, algo);
   if (!fn) return cudaErrorInvalidValue;
   fn<<<total_blocks, block, smem, st>>>(jobs, n, parity & 1, s);
   return cudaGetLastError();

@@ -28,6 +28,9 @@ enum { FMT_PAIR = 3 };
 // Anchored polish (lgt_anchor.cuh): not a link format but the sweep over a
 // fixed anchor field (FP32-12 copy + K0 pairs) with D = G - 1 as pairs.
 enum { FMT_ANCHOR = 4 };
+// Fixed-link bulk sweeps (lgt_fixed.cuh): likewise sweeps, over FP32 links that
+// stay as loaded (18- or 12-real storage) with G as the only state.
+enum { FMT_FIX_18 = 5, FMT_FIX_12 = 6 };
 enum { GAUGE_LANDAU = 0, GAUGE_COULOMB = 1, GAUGE_MAG = 2 };  // MAG: maximally Abelian gauge
 enum { ALGO_OR = 0, ALGO_SR = 1, ALGO_SA = 2 };  // SA: simulated-annealing heat bath
 
@@ -80,6 +83,49 @@ __host__ __device__ __forceinline__ int cb_shift(const Geom &g, const Coords &c,
   }
   return cb_index(g, x1, x2, x3, t);
 }
+
+// Index arithmetic without integer division, for the kernels that count
+// instructions: x / d as the high word of x * inv, inv = ceil(2^32 / d), exact
+// while x * d < 2^32; inv = 0 stands for the division itself.
+__host__ __device__ __forceinline__ unsigned index_inverse(long long limit, int d) {
+  if (d < 2 || limit * d >= (1ll << 32)) return 0u;
+  return (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d);
+}
+__host__ __device__ __forceinline__ int index_div(int x, unsigned inv, int d) {
+#ifdef __CUDA_ARCH__
+  return inv ? (int)__umulhi((unsigned)x, inv) : x / d;
+#else
+  return inv ? (int)(((unsigned long long)(unsigned)x * inv) >> 32) : x / d;
+#endif
+}
+
+// Site j of parity p in slice t with its neighbours as offsets in the
+// within-parity index (the other parity's index of x + dir mu-hat is that of x
+// plus offset(mu, dir)): the same sites as coords_in_slice and cb_shift.
+// inv_half1, inv_n2: index_inverse(vs_half, half1), index_inverse(n2 * n3, n2).
+struct SiteNb {
+  int xh, x2, x3, odd, t_;
+  __host__ __device__ __forceinline__ SiteNb(const Geom &g, unsigned inv_half1, unsigned inv_n2, int p, int t, int j) {
+    const int row = index_div(j, inv_half1, g.half1);
+    xh = j - row * g.half1;
+    x3 = index_div(row, inv_n2, g.n2);
+    x2 = row - x3 * g.n2;
+    odd = (p + t + x2 + x3) & 1;  // x1 = 2 xh + odd
+    t_ = t;
+  }
+  __host__ __device__ __forceinline__ Coords coords(int t) const { return Coords{2 * xh + odd, x2, x3, t}; }
+  __host__ __device__ __forceinline__ int offset(const Geom &g, int mu, int dir) const {
+    if (mu == 1) {
+      if (dir > 0) return odd ? (xh == g.half1 - 1 ? 1 - g.half1 : 1) : 0;
+      return odd ? 0 : (xh == 0 ? g.half1 - 1 : -1);
+    }
+    const int x = mu == 0 ? t_ : (mu == 2 ? x2 : x3);
+    const int n = mu == 0 ? g.nt : (mu == 2 ? g.n2 : g.n3);
+    const int step = mu == 0 ? g.vs_half : (mu == 2 ? g.half1 : g.half1 * g.n2);
+    if (dir > 0) return x == n - 1 ? -x * step : step;
+    return x == 0 ? (n - 1) * step : -step;
+  }
+};
 
 // ------------------------------------------------------------- link formats
 __host__ __device__ __forceinline__ size_t link_bytes_per_half_site(int fmt) {

@@ -129,6 +129,7 @@ struct SweepArgs {
   // global timeslice of local slice 0 (a temporal slab's offset): the random
   // streams of stochastic relaxation and annealing are counted by the global site
   int t_offset;
+  unsigned inv_half1, inv_n2;  // index_inverse of the lattice's row and plane extents (SiteNb)
   // the slices the launch covers: t_first .. t_first + t_count - 1 (all by default)
   int t_first, t_count;
 };
@@ -148,6 +149,8 @@ struct MeasArgs {
   double coulomb_target;
   int with_plaq;
   int mag;  // maximally Abelian gauge: slot 0 sums |U_aa|^2, slot 2 tr Delta_MAG^2
+  const void *G;      // FMT_FIX_*: the links are formed as G U G^+
+  int skip_temporal;  // FMT_FIX_*: except the temporal ones
 };
 
 // Arguments of the fused estimate's finishing reduction (one block per slice).
@@ -233,6 +236,8 @@ struct SweepCfg {
 //    14:  64 threads, <= 128 registers, 8 blocks per SM (27 KB shared each)
 //    15:  64 threads, <= 112 registers, 9 blocks per SM: the links only in
 //         shared memory (24 KB), G loaded into registers beside the copies
+// The fixed-link bulk sweeps (FMT_FIX_*, lgt_fixed.cuh) are compiled for 3, 8 and
+// 9 (64 or 128 threads at <= 128 registers, 128 at <= 96).
 // The one-thread and four-thread layouts form K(x) in the same order, the lean
 // ones link by link; every configuration groups the fused estimate by the same
 // 8 sites; results differ only in FP32 rounding (the order of K's sums and
@@ -259,7 +264,8 @@ __host__ __device__ constexpr int lgt_cfg_stage_chunks(int c) { return c == 15 ?
 __host__ __device__ constexpr int lgt_cfg_sites(int c) { return lgt_cfg_quad(c) ? lgt_cfg_threads(c) / 4 : lgt_cfg_threads(c); }
 // whether a storage format has kernels for a configuration
 __host__ __device__ constexpr bool lgt_cfg_supported(int fmt, int c) {
-  return c >= 0 && c < LGT_NCFG &&
+  return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 8 || c == 9
+                                                  : c >= 0 && c < LGT_NCFG &&
          (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && c == 11)) &&
          (!(lgt_cfg_pipe(c) || lgt_cfg_stream(c) || lgt_cfg_staged(c)) || fmt == FMT_F32_12);
 }
@@ -312,6 +318,34 @@ constexpr int LGT_FUSED_GROUP = 8;
 typedef void (*sweep_fn)(SweepArgs, int);
 sweep_fn pick_sweep_f32(int fmt, int gauge, int algo, int cfg);  // FP32-18, FP32-12
 sweep_fn pick_sweep_hi(int fmt, int gauge, int algo, int cfg);   // FP64, FP32-pair
+sweep_fn pick_sweep_fixed(int fmt, int gauge, int algo, int cfg);  // fixed-link FP32 bulk
+constexpr int LGT_FIXED_SA_CFG = 8;  // the fixed-link annealing sweeps' configuration
+// The bulk sweeps of a lattice keep their links fixed (FMT_FIX_*) wherever no
+// launch configuration asks for a kernel that rewrites them: overrelaxation in
+// Landau and Coulomb gauge (the maximally Abelian update is quadratic in g and
+// needs the transformed links), whole lattices (slabs exchange transformed links),
+// and indices that fit the kernel's 32-bit byte offsets (vh < 2^28 sites per
+// parity; the FP64 field of a larger lattice would not fit the device anyway).
+// Stochastic relaxation keeps rewriting its links: its squared steps are nearly
+// microcanonical, so the norm drift of rewritten links (1.3e-5 in 40 sweeps) stays
+// in the trajectory and theta of the two differs by up to 1e-4 there, more than a
+// change of kernel may (overrelaxation: 2e-5), although the fixed links have the
+// smaller error against FP64 (5e-7 against 1.3e-5 on 64^4).
+inline bool lgt_fixed_links(int bulk_fmt, int gauge, int algo, const Geom &g) {
+  return (bulk_fmt == FMT_F32_18 || bulk_fmt == FMT_F32_12) && gauge != GAUGE_MAG && algo == ALGO_OR &&
+         g.vh < (1 << 28);
+}
+// The fixed-link bulk ends at this theta at the latest, theta_switch or not: the
+// FP32 rounding of G (one rotation of ~4e-8 per update, carried by all 8 links of
+// the site) leaves its field at theta ~ 6e-13, where further sweeps change
+// nothing.  The field promoted from there has that theta too (G is applied to
+// the very links it was relaxed on; rewritten links drift from G to ~1e-8), so the
+// polish takes it on at once.
+constexpr double LGT_FIXED_FLOOR = 2e-12;
+inline double lgt_bulk_target(bool fixed, double theta_switch) {
+  return fixed && theta_switch < LGT_FIXED_FLOOR ? LGT_FIXED_FLOOR : theta_switch;
+}
+inline int lgt_fixed_fmt(int bulk_fmt) { return bulk_fmt == FMT_F32_18 ? FMT_FIX_18 : FMT_FIX_12; }
 
 // One half-sweep of parity p on a field of format fmt with launch
 // configuration cfg.  G (nullable) is multiplied by g at every updated site.
@@ -349,15 +383,19 @@ cudaError_t launch_fused_finish_batch(const BatchFused *jobs, int n, int total_b
 // Exact measurement of a field of format fmt (FP64 arithmetic) into
 // w.totals / w.slice_F / w.slice_theta.  If coulomb_target >= 0 the slice
 // mask is set to (theta_t >= coulomb_target).  with_plaq: also plaquettes.
+// FMT_FIX_*: of the working links G U G^+ of the FP32 links (temporal ones as
+// they are if skip_temporal).
 cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Workspace &w, int with_plaq,
-                           double coulomb_target, int block, cudaStream_t st, int mag = 0);
+                           double coulomb_target, int block, cudaStream_t st, int mag = 0, const void *G = nullptr,
+                           int skip_temporal = 0);
 
 // AoS complex128 (device) -> SoA of format fmt, with SU(3) / finiteness check
 // (err bit 1 set on failure).
 cudaError_t launch_ingest(int fmt, const Geom &g, const double *aos, void *soa, int *err, cudaStream_t st);
 
-// SoA of format fmt -> AoS complex128 (device)
-cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st);
+// SoA of format fmt -> AoS complex128 (device); FMT_FIX_*: the working links G U G^+
+cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st,
+                          const void *G = nullptr, int skip_temporal = 0);
 
 // G <- identity
 cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st);

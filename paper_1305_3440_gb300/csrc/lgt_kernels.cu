@@ -9,6 +9,7 @@
 #include <stdlib.h>
 
 #include "lgt_device.cuh"
+#include "lgt_fixed.cuh"
 #include "lgt_internal.h"
 #include "lgt_measure.cuh"
 #include "lgt_pair.cuh"
@@ -114,6 +115,8 @@ void fill_sweep_args(SweepArgs *a, const Geom &g, void *links, void *G, const Wo
   a->stream_skip = c.stream_skip;
   a->stream_order = nullptr;  // half-sweep after half-sweep
   a->stream_shift = 1;
+  a->inv_half1 = index_inverse(g.vs_half, g.half1);
+  a->inv_n2 = index_inverse((long long)g.n2 * g.n3, g.n2);
   a->t_offset = c.t_offset;
   a->t_first = c.t_first;
   a->t_count = c.t_count > 0 ? c.t_count : g.nt;
@@ -198,6 +201,7 @@ static cudaError_t launch_sweep_kernel(sweep_fn fn, int cfg, const Geom &g, Swee
 }
 
 static sweep_fn pick_sweep(int fmt, const SweepCfg &c, int cfg) {
+  if (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) return pick_sweep_fixed(fmt, c.gauge, c.algo, cfg);
   return (fmt == FMT_F32_18 || fmt == FMT_F32_12) ? pick_sweep_f32(fmt, c.gauge, c.algo, cfg)
                                                   : pick_sweep_hi(fmt, c.gauge, c.algo, cfg);
 }
@@ -332,19 +336,26 @@ void fill_meas_args(MeasArgs *a, const Geom &g, const void *links, const Workspa
   a->active = w.active;
   a->coulomb_target = coulomb_target;
   a->with_plaq = with_plaq;
+  a->G = nullptr;
+  a->skip_temporal = 0;
   a->mag = 0;  // the maximally Abelian gauge's measurement is asked for explicitly (launch_measure)
 }
 
 cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Workspace &w, int with_plaq,
-                           double coulomb_target, int block, cudaStream_t st, int mag) {
+                           double coulomb_target, int block, cudaStream_t st, int mag, const void *G,
+                           int skip_temporal) {
   MeasArgs a{};
   fill_meas_args(&a, g, links, w, with_plaq, coulomb_target);
   a.mag = mag;
+  a.G = G;
+  a.skip_temporal = skip_temporal;
   dim3 grid(ceil_div(g.vs_half, block), g.nt, 2);
   if (fmt == FMT_F64) k_measure<FMT_F64><<<grid, block, 0, st>>>(a);
   else if (fmt == FMT_F32_18) k_measure<FMT_F32_18><<<grid, block, 0, st>>>(a);
   else if (fmt == FMT_F32_12) k_measure<FMT_F32_12><<<grid, block, 0, st>>>(a);
   else if (fmt == FMT_PAIR) k_measure<FMT_PAIR><<<grid, block, 0, st>>>(a);
+  else if (fmt == FMT_FIX_18) k_measure<FMT_FIX_18><<<grid, block, 0, st>>>(a);
+  else if (fmt == FMT_FIX_12) k_measure<FMT_FIX_12><<<grid, block, 0, st>>>(a);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
@@ -415,14 +426,14 @@ __global__ void k_ingest(Geom g, const double *aos, void *soa, int *err) {
 }
 
 template <int FMT>
-__global__ void k_egress(Geom g, const void *soa, double *aos) {
+__global__ void k_egress(Geom g, const void *soa, double *aos, const void *G, int skip_temporal) {
   int p, mu, i;
   Coords c;
   long long lex;
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (!link_of_thread(g, gid, p, mu, i, c, lex)) return;
   double u[18];
-  load_d<FMT>(soa, g.vh, p, mu, i, u);
+  load_field_d<FMT>(g, soa, G, skip_temporal, p, mu, i, u);
   double *dst = aos + ((size_t)lex * 4 + mu) * 18;
 #pragma unroll
   for (int k = 0; k < 18; k++) dst[k] = u[k];
@@ -439,14 +450,17 @@ cudaError_t launch_ingest(int fmt, const Geom &g, const double *aos, void *soa, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st) {
+cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st, const void *G,
+                          int skip_temporal) {
   const long long n = (long long)g.vh * 8;
   const int blk = 256;
   const unsigned grid = (unsigned)((n + blk - 1) / blk);
-  if (fmt == FMT_F64) k_egress<FMT_F64><<<grid, blk, 0, st>>>(g, soa, aos);
-  else if (fmt == FMT_F32_18) k_egress<FMT_F32_18><<<grid, blk, 0, st>>>(g, soa, aos);
-  else if (fmt == FMT_F32_12) k_egress<FMT_F32_12><<<grid, blk, 0, st>>>(g, soa, aos);
-  else if (fmt == FMT_PAIR) k_egress<FMT_PAIR><<<grid, blk, 0, st>>>(g, soa, aos);
+  if (fmt == FMT_F64) k_egress<FMT_F64><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
+  else if (fmt == FMT_F32_18) k_egress<FMT_F32_18><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
+  else if (fmt == FMT_F32_12) k_egress<FMT_F32_12><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
+  else if (fmt == FMT_PAIR) k_egress<FMT_PAIR><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
+  else if (fmt == FMT_FIX_18) k_egress<FMT_FIX_18><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
+  else if (fmt == FMT_FIX_12) k_egress<FMT_FIX_12><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "lgt_device.cuh"
+#include "lgt_fixed.cuh"
 #include "lgt_internal.h"
 #include "lgt_pair.cuh"
 
@@ -39,6 +40,20 @@ struct LoadD<FMT_PAIR> {
 template <int FMT>
 __device__ __forceinline__ void load_d(const void *base, int vh, int p, int mu, int i, double m[18]) {
   LoadD<FMT>::run(base, vh, p, mu, i, m);
+}
+
+// the same, the working links of a fixed-link bulk formed from U and G
+template <int FMT>
+__device__ __forceinline__ void load_field_d(const Geom &g, const void *links, const void *G, int skip_temporal, int p,
+                                             int mu, int i, double m[18]) {
+  if constexpr (FMT == FMT_FIX_18 || FMT == FMT_FIX_12) {
+    float w[18];
+    load_working<FMT == FMT_FIX_18 ? FMT_F32_18 : FMT_F32_12>(g, links, G, skip_temporal, p, mu, i, w);
+#pragma unroll
+    for (int k = 0; k < 18; k++) m[k] = (double)w[k];
+  } else {
+    load_d<FMT>(links, g.vh, p, mu, i, m);
+  }
 }
 
 // X += s * (U - U^dagger)
@@ -80,7 +95,7 @@ __device__ __forceinline__ void measure_body(const MeasArgs &a, int t, int p, in
     if (a.mag) {  // maximally Abelian gauge: sum_a |U_aa|^2 and X(x) (see lgt_device.cuh)
       for (int mu = 0; mu < 4; mu++) {
         double u[18], y[18];
-        load_d<FMT>(a.links, a.g.vh, p, mu, i, u);
+        load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, p, mu, i, u);
 #pragma unroll
         for (int x = 0; x < 3; x++) {
           v[0] += u[LGT_RE(x, x)] * u[LGT_RE(x, x)] + u[LGT_IM(x, x)] * u[LGT_IM(x, x)];
@@ -91,7 +106,7 @@ __device__ __forceinline__ void measure_body(const MeasArgs &a, int t, int p, in
           }
         }
         acc_antiherm(XL, y, 1.0);
-        load_d<FMT>(a.links, a.g.vh, q, mu, cb_shift(a.g, c, mu, -1), u);
+        load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, q, mu, cb_shift(a.g, c, mu, -1), u);
 #pragma unroll
         for (int x = 0; x < 3; x++)
 #pragma unroll
@@ -105,7 +120,7 @@ __device__ __forceinline__ void measure_body(const MeasArgs &a, int t, int p, in
     }
     for (int mu = 0; mu < 4 && !a.mag; mu++) {
       double u[18];
-      load_d<FMT>(a.links, a.g.vh, p, mu, i, u);
+      load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, p, mu, i, u);
       const double rt = u[LGT_RE(0, 0)] + u[LGT_RE(1, 1)] + u[LGT_RE(2, 2)];
       v[0] += rt;
       acc_antiherm(XL, u, 1.0);
@@ -113,7 +128,7 @@ __device__ __forceinline__ void measure_body(const MeasArgs &a, int t, int p, in
         v[1] += rt;
         acc_antiherm(XS, u, 1.0);
       }
-      load_d<FMT>(a.links, a.g.vh, q, mu, cb_shift(a.g, c, mu, -1), u);
+      load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, q, mu, cb_shift(a.g, c, mu, -1), u);
       acc_antiherm(XL, u, -1.0);
       if (mu > 0) acc_antiherm(XS, u, -1.0);
     }
@@ -125,10 +140,10 @@ __device__ __forceinline__ void measure_body(const MeasArgs &a, int t, int p, in
       for (int mu = 0; mu < 4; mu++)
         for (int nu = mu + 1; nu < 4; nu++) {
           double ua[18], ub[18], uc[18], ud[18], m1[18], m2[18];
-          load_d<FMT>(a.links, a.g.vh, p, mu, i, ua);
-          load_d<FMT>(a.links, a.g.vh, q, nu, cb_shift(a.g, c, mu, +1), ub);
-          load_d<FMT>(a.links, a.g.vh, q, mu, cb_shift(a.g, c, nu, +1), uc);
-          load_d<FMT>(a.links, a.g.vh, p, nu, i, ud);
+          load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, p, mu, i, ua);
+          load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, q, nu, cb_shift(a.g, c, mu, +1), ub);
+          load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, q, mu, cb_shift(a.g, c, nu, +1), uc);
+          load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, p, nu, i, ud);
           mat_mul(ua, ub, m1);       // U_mu(x) U_nu(x+mu)
           mat_mul(ud, uc, m2);       // U_nu(x) U_mu(x+nu)
           // Re tr[m1 m2^dagger] = sum_ab Re(m1_ab conj(m2_ab))

@@ -89,8 +89,12 @@ struct Job {
   // the formed field in u64)
   int work_fmt() const { return phase == 0 ? bulk_fmt : (phase == 2 ? (int)FMT_PAIR : (int)FMT_F64); }
   void *work_links() const { return phase == 0 ? u32 : u64; }
-  // kernel variant and links of the sweeps
-  int sweep_fmt() const { return phase == 3 ? (int)FMT_ANCHOR : work_fmt(); }
+  // kernel variant and links of the sweeps (fixed: the FP32 bulk updates G alone;
+  // the only bulk field ever measured is the loaded one, with G = 1)
+  bool fixed = false;
+  int sweep_fmt() const {
+    return phase == 3 ? (int)FMT_ANCHOR : (phase == 0 && fixed ? lgt_fixed_fmt(bulk_fmt) : work_fmt());
+  }
   void *sweep_links() const { return (phase == 0 || phase == 3) ? u32 : u64; }
   int skip_temporal() const { return (prm.gauge == LGT_COULOMB && !prm.transform_temporal) ? 1 : 0; }
   double theta_of(const double *tot) const {
@@ -187,6 +191,7 @@ cudaError_t admit(lgt_server *s, Job *j, int *bad_input) {
   j->cfg.sr_thr = sr_thr_of(p.p);
   j->cfg.seed = p.seed;
   j->cfg.transform_temporal = p.transform_temporal ? 1 : 0;
+  j->fixed = lgt_fixed_links(j->bulk_fmt, j->cfg.gauge, j->cfg.algo, g);
   j->sweep_index = p.sweep_offset;
   j->remaining = p.max_sweeps;
   j->nbx = (g.vs_half + kServerBlock - 1) / kServerBlock;
@@ -237,7 +242,7 @@ cudaError_t anchor_setup(lgt_server *s, Job *j) {
 
 double coulomb_target(const Job *j) {
   if (j->prm.gauge != LGT_COULOMB) return -1.0;
-  return j->phase == 0 ? j->prm.theta_switch : j->prm.theta_tol;
+  return j->phase == 0 ? lgt_bulk_target(j->fixed, j->prm.theta_switch) : j->prm.theta_tol;
 }
 
 struct Segment {
@@ -631,7 +636,7 @@ void worker_main(lgt_server *s) {
           } else {
             j->stall = theta < LGT_STALL_CEILING ? j->stall + 1 : 0;
           }
-          if (theta < j->prm.theta_switch || j->remaining <= 0 || j->stall >= LGT_STALL_CHECKS) {
+          if (theta < lgt_bulk_target(j->fixed, j->prm.theta_switch) || j->remaining <= 0 || j->stall >= LGT_STALL_CHECKS) {
             if ((e = promote_job(s, j)) != cudaSuccess) break;
           }
         } else if (theta < j->prm.theta_tol) {
