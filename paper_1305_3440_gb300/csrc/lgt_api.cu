@@ -221,7 +221,7 @@ struct lgt_ctx {
   void *u32;      // bulk working links
   void *G;        // accumulated transformation of the bulk phase; D = G - 1 of the anchored polish
   int fixed;      // the bulk sweeps keep the links in u32 as loaded and update G alone (lgt_fixed_links)
-  int g_dirty;    // fixed: G != 1, the working links are G u32 G^+
+  int g_dirty;    // bulk sweeps have run since the load: G != 1 (fixed: the working links are G u32 G^+)
   void *k0;       // anchored polish: K0 (pairs)
   int anchored;   // anchored polish: K0, the FP32-12 copy in u32 and D refer to the field in u64
   int d_dirty;    // anchored polish: D != 0 (sweeps since the field in u64 was last formed)
@@ -371,12 +371,11 @@ static lgt_status load_field(lgt_ctx *c, const double *links, int links_on_devic
   c->inj_wait_ns = 0;
   c->inj_skip = 0;
   LGT_CUDA(cudaMemsetAsync(c->ws.active, 1, (size_t)g.nt, c->stream));
-  LGT_CUDA(launch_ingest(FMT_F64, g, src, c->u64, c->ws.err, c->stream));
+  LGT_CUDA(launch_ingest(c->bulk_fmt, g, src, c->u64, c->u32, c->ws.err, c->stream));
   c->stats.launches++;
   if (c->u32) {
-    LGT_CUDA(launch_ingest(c->bulk_fmt, g, src, c->u32, c->ws.err, c->stream));
     LGT_CUDA(launch_g_identity(g, c->G, c->stream));
-    c->stats.launches += 2;
+    c->stats.launches++;
   }
   lgt_status st = read_back(c, c->ws.err, sizeof(int));
   if (st != LGT_OK) return st;
@@ -580,8 +579,9 @@ static int skip_temporal(const lgt_ctx *c) {
 // spent: the next sweep re-anchors)
 static lgt_status anchor_materialise(lgt_ctx *c) {
   if (c->phase != 3 || !c->d_dirty) return LGT_OK;
-  LGT_CUDA(launch_apply_D(c->g, c->G, c->u64, c->u64, nullptr, skip_temporal(c), c->stream));
-  c->stats.launches++;
+  // the FP32 copy in u32 is spent with D: it lends its memory to the orthonormal G
+  LGT_CUDA(launch_apply_D(c->g, c->G, c->u64, c->u64, nullptr, skip_temporal(c), c->u32, c->stream));
+  c->stats.launches += 2;
   c->d_dirty = 0;
   c->anchored = 0;
   return LGT_OK;
@@ -1020,8 +1020,9 @@ extern "C" lgt_status lgt_slab_sync(lgt_ctx *ctx) {
 // --------------------------------------------------------------- promotion
 static lgt_status promote(lgt_ctx *c) {
   if (c->phase != 0) return LGT_OK;
-  LGT_CUDA(launch_apply_G(c->g, c->G, c->u64, c->u64, nullptr, skip_temporal(c), c->stream));
-  c->stats.launches++;
+  // the bulk links are spent: their memory holds the orthonormal G
+  LGT_CUDA(launch_apply_G(c->g, c->G, c->u64, c->u64, nullptr, skip_temporal(c), c->u32, c->stream));
+  c->stats.launches += 2;
   c->phase = 1;
   if (c->prm.polish_algo == LGT_POLISH_OR) c->cfg.algo = ALGO_OR;  // the sweeps after promotion overrelax
   if (c->prm.omega_polish != 0.0) c->cfg.omega = c->prm.omega_polish;
@@ -1365,10 +1366,15 @@ static lgt_status to_output(lgt_ctx *c, double *out, int out_on_device, int work
     dst = tmp;
   }
   cudaError_t e;
-  if (c->phase == 3 && c->d_dirty) e = launch_apply_D(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->stream);
-  else if (c->phase >= 1) e = launch_egress(work_fmt(c), g, c->u64, dst, c->stream);
+  if (c->phase == 3 && c->d_dirty) {
+    // through the memory of the anchor's FP32 copy, which is made anew after
+    e = launch_apply_D(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->u32, c->stream);
+    if (e == cudaSuccess) e = launch_copy_f32_12(g, c->u64, c->u32, c->stream);
+    c->stats.launches += 2;
+  } else if (c->phase >= 1) e = launch_egress(work_fmt(c), g, c->u64, dst, c->stream);
   else if (working) e = launch_egress(read_fmt(c), g, c->u32, dst, c->stream, c->G, skip_temporal(c));
-  else e = launch_apply_G(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->stream);
+  else if (!c->g_dirty) e = launch_egress(FMT_F64, g, c->u64, dst, c->stream);  // G = 1
+  else e = launch_apply_G(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->k0, c->stream), c->stats.launches += c->k0 ? 1 : 0;  // k0: the polish's, idle
   c->stats.launches++;
   if (e == cudaSuccess && tmp) e = cudaMemcpyAsync(out, tmp, aos_bytes, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

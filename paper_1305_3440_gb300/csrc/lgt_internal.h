@@ -389,9 +389,11 @@ cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Work
                            double coulomb_target, int block, cudaStream_t st, int mag = 0, const void *G = nullptr,
                            int skip_temporal = 0);
 
-// AoS complex128 (device) -> SoA of format fmt, with SU(3) / finiteness check
-// (err bit 1 set on failure).
-cudaError_t launch_ingest(int fmt, const Geom &g, const double *aos, void *soa, int *err, cudaStream_t st);
+// AoS complex128 (device) -> SoA in FP64 (u64) and, unless bulk_fmt is FMT_F64, in
+// the bulk's FP32 storage (u32), with SU(3) / finiteness check (err bit 0 set on
+// failure).
+cudaError_t launch_ingest(int bulk_fmt, const Geom &g, const double *aos, void *u64, void *u32, int *err,
+                          cudaStream_t st);
 
 // SoA of format fmt -> AoS complex128 (device); FMT_FIX_*: the working links G U G^+
 cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st,
@@ -402,9 +404,13 @@ cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st);
 
 // U(x,mu) <- G(x) U(x,mu) G(x+mu)^dagger in FP64 with G reunitarised in FP64.
 // Writes to u64_out (SoA FP64, may equal u64_in) or, if aos_out != NULL,
-// to AoS.  skip_temporal: leave mu = 0 untouched.
+// to AoS.  skip_temporal: leave mu = 0 untouched.  scratch (nullable): 144 B per
+// site for the orthonormalised G (without it every link repeats that for both its
+// ends: 3.5 instead of 1.6 ms at 32^4).
 cudaError_t launch_apply_G(const Geom &g, const void *G, const void *u64_in, void *u64_out, double *aos_out,
-                           int skip_temporal, cudaStream_t st);
+                           int skip_temporal, void *scratch, cudaStream_t st);
+// FP32-12 copy of FP64 links
+cudaError_t launch_copy_f32_12(const Geom &g, const void *u64, void *u32, cudaStream_t st);
 
 // Temporal slabs: active[t] = (lo <= t < hi) for the nt slices.
 cudaError_t launch_slice_mask(uint8_t *active, int nt, int lo, int hi, cudaStream_t st);
@@ -422,7 +428,7 @@ cudaError_t launch_loop_decide(LoopState *L, const double *fused_totals, int gau
                                cudaGraphConditionalHandle h, cudaStream_t st);
 // Anchored polish: G = 1 + D (pairs) applied in FP64 (as launch_apply_G).
 cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, void *u64_out, double *aos_out,
-                           int skip_temporal, cudaStream_t st);
+                           int skip_temporal, void *scratch, cudaStream_t st);
 // Anchored polish set-up from the FP64 field u64: K0 (pairs), the FP32-12 copy
 // in u32, D = 0.
 cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge,

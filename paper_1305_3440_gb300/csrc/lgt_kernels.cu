@@ -1,6 +1,6 @@
 // lgt_kernels.cu -- single-lattice launches: half-sweep dispatch, exact
-// measurement, fused-estimate finish, ingest/egress, the accumulated
-// transformation G and the FP64 <-> FP32-pair conversion.  The sweep kernels
+// measurement, fused-estimate finish, the polish set-up and the FP64 <-> FP32-pair
+// conversion (the field in and out: lgt_io.cu).  The sweep kernels
 // themselves live in lgt_sweep_f32.cu and lgt_sweep_hi.cu (block-size
 // variants, compiled in parallel), their bodies in lgt_sweep.cuh.
 #include <cuda_runtime.h>
@@ -360,111 +360,6 @@ cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Work
   return cudaGetLastError();
 }
 
-// ------------------------------------------------------- layout / ingest
-// thread -> (parity, direction, within-parity index); lexicographic site
-__device__ __forceinline__ bool link_of_thread(const Geom &g, long long gid, int &p, int &mu, int &i, Coords &c,
-                                               long long &lex) {
-  if (gid >= (long long)g.vh * 8) return false;
-  i = (int)(gid % g.vh);
-  const int pm = (int)(gid / g.vh);
-  p = pm >> 2;
-  mu = pm & 3;
-  const int t = i / g.vs_half;
-  c = coords_in_slice(g, p, t, i - t * g.vs_half);
-  lex = (long long)c.x1 + (long long)g.n1 * (c.x2 + (long long)g.n2 * (c.x3 + (long long)g.n3 * c.t));
-  return true;
-}
-
-template <int FMT>
-__global__ void k_ingest(Geom g, const double *aos, void *soa, int *err) {
-  int p, mu, i;
-  Coords c;
-  long long lex;
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (!link_of_thread(g, gid, p, mu, i, c, lex)) return;
-  const double *src = aos + ((size_t)lex * 4 + mu) * 18;
-  double u[18];
-  bool finite = true;
-#pragma unroll
-  for (int k = 0; k < 18; k++) {
-    u[k] = src[k];
-    finite = finite && isfinite(u[k]);
-  }
-  // SU(3) check: |U^dagger U - 1|_max and |det U - 1|
-  double worst = 0.0;
-#pragma unroll
-  for (int a = 0; a < 3; a++)
-#pragma unroll
-    for (int b = 0; b < 3; b++) {
-      double re = 0.0, im = 0.0;
-#pragma unroll
-      for (int k = 0; k < 3; k++) {  // sum_k conj(U_ka) U_kb
-        re += u[LGT_RE(k, a)] * u[LGT_RE(k, b)] + u[LGT_IM(k, a)] * u[LGT_IM(k, b)];
-        im += u[LGT_RE(k, a)] * u[LGT_IM(k, b)] - u[LGT_IM(k, a)] * u[LGT_RE(k, b)];
-      }
-      re -= (a == b) ? 1.0 : 0.0;
-      worst = fmax(worst, fmax(fabs(re), fabs(im)));
-    }
-  double dre = 0.0, dim = 0.0;
-#pragma unroll
-  for (int cc = 0; cc < 3; cc++) {
-    const int a1 = (cc + 1) % 3, b1 = (cc + 2) % 3;
-    const double mre = u[LGT_RE(1, a1)] * u[LGT_RE(2, b1)] - u[LGT_IM(1, a1)] * u[LGT_IM(2, b1)] -
-                       (u[LGT_RE(1, b1)] * u[LGT_RE(2, a1)] - u[LGT_IM(1, b1)] * u[LGT_IM(2, a1)]);
-    const double mim = u[LGT_RE(1, a1)] * u[LGT_IM(2, b1)] + u[LGT_IM(1, a1)] * u[LGT_RE(2, b1)] -
-                       (u[LGT_RE(1, b1)] * u[LGT_IM(2, a1)] + u[LGT_IM(1, b1)] * u[LGT_RE(2, a1)]);
-    dre += u[LGT_RE(0, cc)] * mre - u[LGT_IM(0, cc)] * mim;
-    dim += u[LGT_RE(0, cc)] * mim + u[LGT_IM(0, cc)] * mre;
-  }
-  worst = fmax(worst, fmax(fabs(dre - 1.0), fabs(dim)));
-  if (!finite || !(worst < 1e-10)) atomicOr(err, 1);
-  typedef typename LinkIO<FMT>::real R;
-  R r[18];
-#pragma unroll
-  for (int k = 0; k < 18; k++) r[k] = (R)u[k];
-  LinkIO<FMT>::store(soa, g.vh, p, mu, i, r);
-}
-
-template <int FMT>
-__global__ void k_egress(Geom g, const void *soa, double *aos, const void *G, int skip_temporal) {
-  int p, mu, i;
-  Coords c;
-  long long lex;
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (!link_of_thread(g, gid, p, mu, i, c, lex)) return;
-  double u[18];
-  load_field_d<FMT>(g, soa, G, skip_temporal, p, mu, i, u);
-  double *dst = aos + ((size_t)lex * 4 + mu) * 18;
-#pragma unroll
-  for (int k = 0; k < 18; k++) dst[k] = u[k];
-}
-
-cudaError_t launch_ingest(int fmt, const Geom &g, const double *aos, void *soa, int *err, cudaStream_t st) {
-  const long long n = (long long)g.vh * 8;
-  const int blk = 256;
-  const unsigned grid = (unsigned)((n + blk - 1) / blk);
-  if (fmt == FMT_F64) k_ingest<FMT_F64><<<grid, blk, 0, st>>>(g, aos, soa, err);
-  else if (fmt == FMT_F32_18) k_ingest<FMT_F32_18><<<grid, blk, 0, st>>>(g, aos, soa, err);
-  else if (fmt == FMT_F32_12) k_ingest<FMT_F32_12><<<grid, blk, 0, st>>>(g, aos, soa, err);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st, const void *G,
-                          int skip_temporal) {
-  const long long n = (long long)g.vh * 8;
-  const int blk = 256;
-  const unsigned grid = (unsigned)((n + blk - 1) / blk);
-  if (fmt == FMT_F64) k_egress<FMT_F64><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
-  else if (fmt == FMT_F32_18) k_egress<FMT_F32_18><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
-  else if (fmt == FMT_F32_12) k_egress<FMT_F32_12><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
-  else if (fmt == FMT_PAIR) k_egress<FMT_PAIR><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
-  else if (fmt == FMT_FIX_18) k_egress<FMT_FIX_18><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
-  else if (fmt == FMT_FIX_12) k_egress<FMT_FIX_12><<<grid, blk, 0, st>>>(g, soa, aos, G, skip_temporal);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
-}
-
 // ------------------------------------------------ accumulated transformation
 __global__ void k_g_identity(Geom g, void *G) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -480,76 +375,6 @@ cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st) {
   const long long n = (long long)g.vh * 2;
   const int blk = 256;
   k_g_identity<<<(unsigned)((n + blk - 1) / blk), blk, 0, st>>>(g, G);
-  return cudaGetLastError();
-}
-
-__device__ __forceinline__ void load_G_fp64(const void *G, int vh, int p, int i, double m[18]) {
-  float f[18];
-  GIO::load(G, vh, p, i, f);
-#pragma unroll
-  for (int k = 0; k < 18; k++) m[k] = (double)f[k];
-  reunitarise(m);
-}
-
-// G = 1 + D of the anchored polish in FP64 (pairs widened, row 2 rebuilt in
-// FP64, rows orthonormalised: unitary to FP64 rounding)
-__device__ __forceinline__ void load_G_from_D(const void *D, int vh, int p, int i, double m[18]) {
-  f2 d[18];
-  DIO::load_pair(D, vh, p, i, d);
-#pragma unroll
-  for (int k = 0; k < 12; k++) m[k] = (double)d[k].hi + (double)d[k].lo;
-  m[LGT_RE(0, 0)] += 1.0;
-  m[LGT_RE(1, 1)] += 1.0;
-  reunitarise(m);
-}
-
-// U_mu(x) <- G(x) U_mu(x) G(x+mu)^+ in FP64; SRC 0: G of the bulk phase
-// (FP32), SRC 1: G = 1 + D of the anchored polish (pairs)
-template <int SRC>
-__global__ void k_apply_G(Geom g, const void *G, const void *u_in, void *u_out, double *aos_out, int skip_temporal) {
-  int p, mu, i;
-  Coords c;
-  long long lex;
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (!link_of_thread(g, gid, p, mu, i, c, lex)) return;
-  double u[18], r[18], gx[18], gy[18], tmp[18];
-  LinkIO<FMT_F64>::load(u_in, g.vh, p, mu, i, u);
-  if (skip_temporal && mu == 0) {
-#pragma unroll
-    for (int k = 0; k < 18; k++) r[k] = u[k];
-  } else {
-    if (SRC == 0) {
-      load_G_fp64(G, g.vh, p, i, gx);
-      load_G_fp64(G, g.vh, p ^ 1, cb_shift(g, c, mu, +1), gy);
-    } else {
-      load_G_from_D(G, g.vh, p, i, gx);
-      load_G_from_D(G, g.vh, p ^ 1, cb_shift(g, c, mu, +1), gy);
-    }
-    mat_mul(gx, u, tmp);
-    mat_mul_dag(tmp, gy, r);
-  }
-  if (aos_out) {
-    double *dst = aos_out + ((size_t)lex * 4 + mu) * 18;
-#pragma unroll
-    for (int k = 0; k < 18; k++) dst[k] = r[k];
-  } else {
-    LinkIO<FMT_F64>::store(u_out, g.vh, p, mu, i, r);
-  }
-}
-
-cudaError_t launch_apply_G(const Geom &g, const void *G, const void *u64_in, void *u64_out, double *aos_out,
-                           int skip_temporal, cudaStream_t st) {
-  const long long n = (long long)g.vh * 8;
-  const int blk = 128;
-  k_apply_G<0><<<(unsigned)((n + blk - 1) / blk), blk, 0, st>>>(g, G, u64_in, u64_out, aos_out, skip_temporal);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, void *u64_out, double *aos_out,
-                           int skip_temporal, cudaStream_t st) {
-  const long long n = (long long)g.vh * 8;
-  const int blk = 128;
-  k_apply_G<1><<<(unsigned)((n + blk - 1) / blk), blk, 0, st>>>(g, D, u64_in, u64_out, aos_out, skip_temporal);
   return cudaGetLastError();
 }
 

@@ -213,8 +213,7 @@ cudaError_t admit(lgt_server *s, Job *j, int *bad_input) {
   void *stage = nullptr;
   if ((e = dev_alloc(s, &stage, aos_bytes_of(g))) != cudaSuccess) return e;
   e = cudaMemcpyAsync(stage, j->input.data(), aos_bytes_of(g), cudaMemcpyHostToDevice, s->stream);
-  if (e == cudaSuccess) e = launch_ingest(FMT_F64, g, (const double *)stage, j->u64, j->ws.err, s->stream);
-  if (e == cudaSuccess && j->u32) e = launch_ingest(j->bulk_fmt, g, (const double *)stage, j->u32, j->ws.err, s->stream);
+  if (e == cudaSuccess) e = launch_ingest(j->bulk_fmt, g, (const double *)stage, j->u64, j->u32, j->ws.err, s->stream);
   if (e == cudaSuccess && j->G) e = launch_g_identity(g, j->G, s->stream);
   int err_h = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&err_h, j->ws.err, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
@@ -230,7 +229,7 @@ cudaError_t admit(lgt_server *s, Job *j, int *bad_input) {
 cudaError_t anchor_materialise(lgt_server *s, Job *j) {
   if (j->phase != 3 || !j->d_dirty) return cudaSuccess;
   j->d_dirty = j->anchored = false;
-  return launch_apply_D(j->g, j->G, j->u64, j->u64, nullptr, j->skip_temporal(), s->stream);
+  return launch_apply_D(j->g, j->G, j->u64, j->u64, nullptr, j->skip_temporal(), j->u32, s->stream);
 }
 
 cudaError_t anchor_setup(lgt_server *s, Job *j) {
@@ -507,7 +506,7 @@ cudaError_t collect(lgt_server *s, Job *j) {
   if ((e = dev_alloc(s, &stage, aos_bytes_of(j->g))) != cudaSuccess) return e;
   if (j->phase >= 1) e = launch_egress(j->work_fmt(), j->g, j->u64, (double *)stage, s->stream);
   else e = launch_apply_G(j->g, j->G, j->u64, nullptr, (double *)stage,
-                          (j->prm.gauge == LGT_COULOMB && !j->prm.transform_temporal) ? 1 : 0, s->stream);
+                          j->skip_temporal(), j->k0, s->stream);
   j->output.resize(aos_bytes_of(j->g) / sizeof(double));
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(j->output.data(), stage, aos_bytes_of(j->g), cudaMemcpyDeviceToHost, s->stream);
@@ -523,7 +522,7 @@ cudaError_t collect(lgt_server *s, Job *j) {
 }
 
 cudaError_t promote_job(lgt_server *s, Job *j) {
-  cudaError_t e = launch_apply_G(j->g, j->G, j->u64, j->u64, nullptr, j->skip_temporal(), s->stream);
+  cudaError_t e = launch_apply_G(j->g, j->G, j->u64, j->u64, nullptr, j->skip_temporal(), j->u32, s->stream);
   j->phase = 1;
   if (j->prm.polish_algo == LGT_POLISH_OR) j->cfg.algo = ALGO_OR;  // the sweeps after promotion overrelax
   if (j->prm.omega_polish != 0.0) j->cfg.omega = j->prm.omega_polish;
