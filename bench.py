@@ -187,7 +187,7 @@ def algorithmic_bytes_per_site(kind: str) -> int:
     in (FP32-12 48 B, FP32-18 72 B; Coulomb gauge 6), G(x) in and out (2 rows: 48
     B) and the other parity's G (48 B per site: each is read by 8 neighbours,
     compulsory once).  FP32-pair and FP64 polish: 8 links of 144 B in and out.
-    Anchored polish: K0(x) (144 B) and the 8 links' FP32-12 copies (384 B) in, its
+    Anchored polish: K0(x) (112 B) and the 8 links' FP32-12 copies (384 B) in, its
     own D (96 B: rows 0, 1 as pairs) in and out, and the other parity's D high parts
     (48 B per site)."""
     if kind == "fp32_12":
@@ -197,9 +197,9 @@ def algorithmic_bytes_per_site(kind: str) -> int:
     if kind == "fp32_18":
         return 8 * 72 + 3 * 48
     if kind == "anchor":
-        return 144 + 8 * 48 + 48 + 2 * 96
+        return 112 + 8 * 48 + 48 + 2 * 96
     if kind == "anchor_coulomb":  # spatial directions only
-        return 144 + 6 * 48 + 48 + 2 * 96
+        return 112 + 6 * 48 + 48 + 2 * 96
     return 16 * 144
 
 

@@ -109,10 +109,10 @@ typedef enum {
  *   sweeps relax the gauge transformation G = 1 + D alone: the local update
  *   at x sees K(x) = G(x) [K0(x) + C(x)], the K(x) of the same sweep on the
  *   transformed links G U' G^+ (Sec. 3), with the constant
- *   K0 = sum_mu U'_mu(x) + U'_mu(x-mu)^+ stored once as FP32 pairs and the
- *   small C = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+ formed in
+ *   K0 = sum_mu U'_mu(x) + U'_mu(x-mu)^+ stored once (its Hermitian part in
+ *   FP32, its anti-Hermitian part as FP32 pairs) and the small C = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+ formed in
  *   FP32; rotation angles, SU(2) elements and delta = g - 1 in FP32 from the
- *   small quantities; D accumulated as FP32 pairs.  Only D is written (768
+ *   small quantities; D accumulated as FP32 pairs.  Only D is written (736
  *   bytes of compulsory traffic per site update against 2304 for PAIR).
  *   Measurements and output form G U' G^+ in FP64 with G orthonormalised in
  *   FP64 (an exact gauge transform); a measurement makes it the new anchor.

@@ -11,22 +11,29 @@
 // these are the paper's sweeps with the transformation kept apart from the
 // links, which allows each term to be stored at the precision it needs:
 //   * M = K0 + C with the constant K0(x) = sum_mu U'_mu(x) + U'_mu(x-mu)^+,
-//     formed once in FP64 and stored as FP32 pairs, and the small
+//     formed once in FP64 and kept as its Hermitian part (FP32) and its
+//     anti-Hermitian part A0 (FP32 pairs), and the small
 //     C(x) = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+, which FP32
 //     resolves to |D| 2^-24 from FP32 copies of U' and the high parts of D;
 //   * K = M + D(x) M with the small product in FP32;
-//   * the rotation angles in FP32 from the pair-precision K, each SU(2)
-//     element in FP32 near-identity form (unit to ~|r|^2 2^-24) and
+//   * the rotation angles in FP32.  What must be resolved near the maximum is the
+//     anti-Hermitian part of K (theta and the vector part of every subgroup's
+//     quaternion are differences of its entries), so it is carried apart as the
+//     small number it is, from A0 through the subgroup steps: FP32 relative to
+//     itself, where holding all of K in pairs spent a pair addition (11
+//     operations) on each of its entries at every stage; the Hermitian part
+//     gives the quaternion's scalar part, which FP32 rounds anyway;
+//   * each SU(2) element in FP32 near-identity form (unit to ~|r|^2 2^-24) and
 //     delta = g - 1 in FP32 from the small quantities (error ~|delta| 2^-24);
 //   * D <- D + delta + delta D accumulated as an FP32 pair, so G stays unitary
 //     to ~1e-10 over a polish (what its rounding per update sums to), far below
 //     the ~1e-7 violations that theta < 1e-14 resolves; the field is formed as
 //     G U' G^+ in FP64 with G orthonormalised in FP64, an exact gauge transform
 //     of the input whatever G's rounding.
-// Per site update the sweep reads K0 (144 B), 8 FP32 links (384 B), the high
+// Per site update the sweep reads K0 (112 B), 8 FP32 links (384 B), the high
 // parts of 8 neighbours' D (384 B, each neighbour's read by 8 sites, so 48 B
 // of compulsory traffic) and its own D (96 B), and writes its own D (96 B):
-// 768 B of compulsory traffic; no link is written.
+// 736 B of compulsory traffic; no link is written.
 #pragma once
 
 #include "lgt_device.cuh"
@@ -40,21 +47,21 @@ namespace lgt {
 //       = conj((-D_02, -D_12, D_00 + D_11) + D_0 x D_1),
 // formed from the small entries only (error relative to |D|).
 __device__ __forceinline__ void small_row2(float d[18]) {
-  float cre[3], cim[3];
 #pragma unroll
   for (int k = 0; k < 3; k++) {
-    const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
-    const float ar1 = d[LGT_RE(0, k1)], ai1 = d[LGT_IM(0, k1)], ar2 = d[LGT_RE(0, k2)], ai2 = d[LGT_IM(0, k2)];
-    const float br1 = d[LGT_RE(1, k1)], bi1 = d[LGT_IM(1, k1)], br2 = d[LGT_RE(1, k2)], bi2 = d[LGT_IM(1, k2)];
-    cre[k] = (ar1 * br2 - ai1 * bi2) - (ar2 * br1 - ai2 * bi1);
-    cim[k] = (ar1 * bi2 + ai1 * br2) - (ar2 * bi1 + ai2 * br1);
-  }
-  const float lre[3] = {-d[LGT_RE(0, 2)], -d[LGT_RE(1, 2)], d[LGT_RE(0, 0)] + d[LGT_RE(1, 1)]};
-  const float lim[3] = {-d[LGT_IM(0, 2)], -d[LGT_IM(1, 2)], d[LGT_IM(0, 0)] + d[LGT_IM(1, 1)]};
-#pragma unroll
-  for (int k = 0; k < 3; k++) {
-    d[LGT_RE(2, k)] = lre[k] + cre[k];
-    d[LGT_IM(2, k)] = -(lim[k] + cim[k]);
+    const int a = (k + 1) % 3, b = (k + 2) % 3;
+    float re = k == 0 ? -d[LGT_RE(0, 2)] : (k == 1 ? -d[LGT_RE(1, 2)] : d[LGT_RE(0, 0)] + d[LGT_RE(1, 1)]);
+    float im = k == 0 ? d[LGT_IM(0, 2)] : (k == 1 ? d[LGT_IM(1, 2)] : -d[LGT_IM(0, 0)] - d[LGT_IM(1, 1)]);
+    re = fmaf(d[LGT_RE(0, a)], d[LGT_RE(1, b)], re);
+    im = fmaf(-d[LGT_RE(0, a)], d[LGT_IM(1, b)], im);
+    re = fmaf(-d[LGT_IM(0, a)], d[LGT_IM(1, b)], re);
+    im = fmaf(-d[LGT_IM(0, a)], d[LGT_RE(1, b)], im);
+    re = fmaf(-d[LGT_RE(0, b)], d[LGT_RE(1, a)], re);
+    im = fmaf(d[LGT_RE(0, b)], d[LGT_IM(1, a)], im);
+    re = fmaf(d[LGT_IM(0, b)], d[LGT_IM(1, a)], re);
+    im = fmaf(d[LGT_IM(0, b)], d[LGT_RE(1, a)], im);
+    d[LGT_RE(2, k)] = re;
+    d[LGT_IM(2, k)] = im;
   }
 }
 
@@ -85,18 +92,6 @@ __device__ __forceinline__ void small_row2_pair(f2 d[18]) {
 // parity p at (p * 3 + k) * vh + i), so a neighbour's term reads 48 B.
 struct DIO {
   static __device__ __forceinline__ size_t lo_offset(int vh) { return (size_t)6 * vh; }
-  static __device__ __forceinline__ void load_hi(const void *base, int vh, int p, int i, float d[18]) {
-    const float4 *b4 = reinterpret_cast<const float4 *>(base) + (size_t)(p * 3) * vh + i;
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      const float4 v = __ldg(b4 + (size_t)k * vh);
-      d[4 * k] = v.x;
-      d[4 * k + 1] = v.y;
-      d[4 * k + 2] = v.z;
-      d[4 * k + 3] = v.w;
-    }
-    small_row2(d);
-  }
   static __device__ __forceinline__ void load_pair(const void *base, int vh, int p, int i, f2 d[18]) {
     const float4 *h4 = reinterpret_cast<const float4 *>(base) + (size_t)(p * 3) * vh + i;
     const float4 *l4 = h4 + lo_offset(vh);
@@ -110,19 +105,6 @@ struct DIO {
     }
     small_row2_pair(d);
   }
-  // rows 0, 1 as pairs only (row 2 left unset)
-  static __device__ __forceinline__ void load_pair_rows(const void *base, int vh, int p, int i, f2 d[12]) {
-    const float4 *h4 = reinterpret_cast<const float4 *>(base) + (size_t)(p * 3) * vh + i;
-    const float4 *l4 = h4 + lo_offset(vh);
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-      const float4 h = __ldg(h4 + (size_t)k * vh), l = __ldg(l4 + (size_t)k * vh);
-      d[4 * k] = {h.x, l.x};
-      d[4 * k + 1] = {h.y, l.y};
-      d[4 * k + 2] = {h.z, l.z};
-      d[4 * k + 3] = {h.w, l.w};
-    }
-  }
   static __device__ __forceinline__ void store_pair(void *base, int vh, int p, int i, const f2 d[18]) {
     float4 *h4 = reinterpret_cast<float4 *>(base) + (size_t)(p * 3) * vh + i;
     float4 *l4 = h4 + lo_offset(vh);
@@ -134,23 +116,61 @@ struct DIO {
   }
 };
 
-// K0(x): one 3x3 complex matrix per site as FP32 pairs, 9 float4 chunks
-// (chunk c of parity p at (p * 9 + c) * vh + i).
+// K0(x) as its Hermitian part H (FP32) and its anti-Hermitian part A (FP32 pairs),
+// 28 floats in 7 float4 chunks (chunk c of parity p at (p * 7 + c) * vh + i):
+//   0: H_00 H_11 H_22 and Im A_00     1: Im A_11 Im A_22 H_01    2: H_02 H_12
+//   3: A_01 A_02                      4: A_12, low Im A_00 Im A_11
+//   5: low Im A_22, low A_01, low Re A_02   6: low Im A_02, low A_12, tau
+// A is the traceless part: Im tr K0, which is not small, drops out of theta and of
+// every rotation; tau = Im tr K0 / 3 is kept for the products with K0.
+struct AnchorK0 {
+  float h[3];     // H_aa
+  float ho[6];    // H_01, H_02, H_12 (re, im)
+  float ad[3];    // Im A_aa
+  float ao[6];    // A_01, A_02, A_12 (re, im)
+  float adl[3], aol[6];  // low parts
+  float tau;             // Im tr K0 / 3
+};
 struct K0IO {
-  static __device__ __forceinline__ void load(const void *base, int vh, int p, int i, f2 m[18]) {
-    const float4 *b = reinterpret_cast<const float4 *>(base) + (size_t)(p * 9) * vh + i;
+  static __device__ __forceinline__ void load(const void *base, int vh, int p, int i, AnchorK0 &k) {
+    const float4 *b = reinterpret_cast<const float4 *>(base) + (size_t)(p * 7) * vh + i;
+    float4 v[7];
 #pragma unroll
-    for (int c = 0; c < 9; c++) {
-      const float4 v = __ldg(b + (size_t)c * vh);
-      m[2 * c] = {v.x, v.y};
-      m[2 * c + 1] = {v.z, v.w};
-    }
+    for (int c = 0; c < 7; c++) v[c] = __ldcs(b + (size_t)c * vh);
+    k.h[0] = v[0].x, k.h[1] = v[0].y, k.h[2] = v[0].z, k.ad[0] = v[0].w;
+    k.ad[1] = v[1].x, k.ad[2] = v[1].y, k.ho[0] = v[1].z, k.ho[1] = v[1].w;
+    k.ho[2] = v[2].x, k.ho[3] = v[2].y, k.ho[4] = v[2].z, k.ho[5] = v[2].w;
+    k.ao[0] = v[3].x, k.ao[1] = v[3].y, k.ao[2] = v[3].z, k.ao[3] = v[3].w;
+    k.ao[4] = v[4].x, k.ao[5] = v[4].y, k.adl[0] = v[4].z, k.adl[1] = v[4].w;
+    k.adl[2] = v[5].x, k.aol[0] = v[5].y, k.aol[1] = v[5].z, k.aol[2] = v[5].w;
+    k.aol[3] = v[6].x, k.aol[4] = v[6].y, k.aol[5] = v[6].z, k.tau = v[6].w;
   }
-  static __device__ __forceinline__ void store(void *base, int vh, int p, int i, const f2 m[18]) {
-    float4 *b = reinterpret_cast<float4 *>(base) + (size_t)(p * 9) * vh + i;
+  // from K0 in FP64
+  static __device__ __forceinline__ void store(void *base, int vh, int p, int i, const double K[18]) {
+    float4 *b = reinterpret_cast<float4 *>(base) + (size_t)(p * 7) * vh + i;
+    float f[28];
+    auto pair = [&](int hi, int lo, double v) {
+      f[hi] = __double2float_rn(v);
+      f[lo] = __double2float_rn(v - (double)f[hi]);
+    };
+    const int ad[3] = {3, 4, 5}, adl[3] = {18, 19, 20};
+    const double tau = (K[LGT_IM(0, 0)] + K[LGT_IM(1, 1)] + K[LGT_IM(2, 2)]) * (1.0 / 3.0);
 #pragma unroll
-    for (int c = 0; c < 9; c++)
-      b[(size_t)c * vh] = make_float4(m[2 * c].hi, m[2 * c].lo, m[2 * c + 1].hi, m[2 * c + 1].lo);
+    for (int a = 0; a < 3; a++) {
+      f[a] = __double2float_rn(K[LGT_RE(a, a)]);
+      pair(ad[a], adl[a], K[LGT_IM(a, a)] - tau);
+    }
+#pragma unroll
+    for (int n = 0; n < 3; n++) {  // (0,1), (0,2), (1,2)
+      const int a = n == 2 ? 1 : 0, c = n == 0 ? 1 : 2;
+      f[6 + 2 * n] = __double2float_rn(0.5 * (K[LGT_RE(a, c)] + K[LGT_RE(c, a)]));
+      f[7 + 2 * n] = __double2float_rn(0.5 * (K[LGT_IM(a, c)] - K[LGT_IM(c, a)]));
+      pair(12 + 2 * n, 21 + 2 * n, 0.5 * (K[LGT_RE(a, c)] - K[LGT_RE(c, a)]));
+      pair(13 + 2 * n, 22 + 2 * n, 0.5 * (K[LGT_IM(a, c)] + K[LGT_IM(c, a)]));
+    }
+    f[27] = __double2float_rn(tau);
+#pragma unroll
+    for (int c = 0; c < 7; c++) b[(size_t)c * vh] = make_float4(f[4 * c], f[4 * c + 1], f[4 * c + 2], f[4 * c + 3]);
   }
 };
 
@@ -188,27 +208,96 @@ __device__ __forceinline__ void acc_dag_mul_dag(const float a[18], const float b
     }
 }
 
-// Sec. 3 local update for the anchored polish: the block projections from the
-// pair-precision K (no cancellation loss near convergence), the rotation
-// angles and each subgroup element in FP32 near-identity form (1 + e0, r):
-// unit to ~|r|^2 2^-24, i.e. ~1e-15 for the |r| <~ 1e-4 of polishing (only G's
-// unitarity depends on it, and G is orthonormalised in FP64 when the field is
-// formed).  W is steered between subgroups in FP32 as in the pair polish.
-template <int ALGO>
-__device__ __forceinline__ void anchor_local_update(f2 W[18], RotF rf[3], float omega, uint64_t sr_thr, uint4 draws) {
+// K(x) = M + D M of the anchored polish, M = K0 + C: all of it as floats (W), and
+// its anti-Hermitian part apart (see above).
+struct AnchorK {
+  float W[18];
+  float ad[3], ao[6];  // Im A_aa (less tau); A_01, A_02, A_12
+};
+__device__ __forceinline__ void anchor_K(const AnchorK0 &k0, const float C[18], const float dh[18], AnchorK &K) {
+  float M[18], T[18];
 #pragma unroll
-  for (int s = 0; s < 3; s++) {
-    const int i = (s == 2) ? 1 : 0;
-    const int j = (s == 0) ? 1 : 2;
-    const float q0 = pair_to_float(pair_add(W[LGT_RE(i, i)], W[LGT_RE(j, j)]));
-    const float q1 = pair_to_float(pair_add(W[LGT_IM(i, j)], W[LGT_IM(j, i)]));
-    const float q2 = pair_to_float(pair_add(W[LGT_RE(i, j)], pair_neg(W[LGT_RE(j, i)])));
-    const float q3 = pair_to_float(pair_add(W[LGT_IM(i, i)], pair_neg(W[LGT_IM(j, j)])));
-    const uint32_t d = s == 0 ? draws.x : (s == 1 ? draws.y : draws.z);
-    rf[s] = subgroup_rotation<ALGO>(q0, q1, q2, q3, omega, (uint64_t)d < sr_thr);
-    if (s == 0) steer_rows<0, 1>(W, rf[s]);
-    if (s == 1) steer_rows<0, 2>(W, rf[s]);
+  for (int a = 0; a < 3; a++) {
+    M[LGT_RE(a, a)] = k0.h[a] + C[LGT_RE(a, a)];
+    M[LGT_IM(a, a)] = (k0.ad[a] + k0.tau) + C[LGT_IM(a, a)];
   }
+#pragma unroll
+  for (int n = 0; n < 3; n++) {
+    const int a = n == 2 ? 1 : 0, c = n == 0 ? 1 : 2;
+    M[LGT_RE(a, c)] = (k0.ho[2 * n] + k0.ao[2 * n]) + C[LGT_RE(a, c)];
+    M[LGT_IM(a, c)] = (k0.ho[2 * n + 1] + k0.ao[2 * n + 1]) + C[LGT_IM(a, c)];
+    M[LGT_RE(c, a)] = (k0.ho[2 * n] - k0.ao[2 * n]) + C[LGT_RE(c, a)];
+    M[LGT_IM(c, a)] = (k0.ao[2 * n + 1] - k0.ho[2 * n + 1]) + C[LGT_IM(c, a)];
+  }
+  mat_mul(dh, M, T);
+#pragma unroll
+  for (int e = 0; e < 18; e++) {
+    K.W[e] = M[e] + T[e];
+    T[e] += C[e];  // K = K0 + T
+  }
+#pragma unroll
+  for (int a = 0; a < 3; a++) K.ad[a] = k0.ad[a] + (k0.adl[a] + T[LGT_IM(a, a)]);
+#pragma unroll
+  for (int n = 0; n < 3; n++) {
+    const int a = n == 2 ? 1 : 0, c = n == 0 ? 1 : 2;
+    K.ao[2 * n] = k0.ao[2 * n] + fmaf(0.5f, T[LGT_RE(a, c)] - T[LGT_RE(c, a)], k0.aol[2 * n]);
+    K.ao[2 * n + 1] = k0.ao[2 * n + 1] + fmaf(0.5f, T[LGT_IM(a, c)] + T[LGT_IM(c, a)], k0.aol[2 * n + 1]);
+  }
+}
+
+// Re tr K and tr[Delta Delta^dagger], Delta the traceless part of (K - K^+)/(2i)
+__device__ __forceinline__ void anchor_violation(const AnchorK &K, float &retr, float &delta2) {
+  retr = K.W[LGT_RE(0, 0)] + K.W[LGT_RE(1, 1)] + K.W[LGT_RE(2, 2)];
+  const float tr3 = (K.ad[0] + K.ad[1] + K.ad[2]) * (1.0f / 3.0f);
+  float s = 0.0f, t = 0.0f;
+#pragma unroll
+  for (int a = 0; a < 3; a++) s = fmaf(K.ad[a] - tr3, K.ad[a] - tr3, s);
+#pragma unroll
+  for (int e = 0; e < 6; e++) t = fmaf(K.ao[e], K.ao[e], t);
+  delta2 = fmaf(2.0f, t, s);
+}
+
+// Sec. 3 local update for the anchored polish: the quaternions' scalar parts from
+// W, their vector parts from the anti-Hermitian part; each subgroup element in
+// FP32 near-identity form (1 + e0, r), unit to ~|r|^2 2^-24, i.e. ~1e-15 for the
+// |r| <~ 1e-4 of polishing (only G's unitarity depends on it, and G is
+// orthonormalised in FP64 when the field is formed).  W <- W + rho W between the
+// subgroups, as far as the later ones see it.
+template <int ALGO>
+__device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], float omega, uint64_t sr_thr, uint4 draws) {
+  float *W = K.W;
+  // (0,1)
+  RotF r = rf[0] = subgroup_rotation<ALGO>(W[LGT_RE(0, 0)] + W[LGT_RE(1, 1)], 2.0f * K.ao[1], 2.0f * K.ao[0],
+                                           K.ad[0] - K.ad[1], omega, (uint64_t)draws.x < sr_thr);
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    const float xi = W[LGT_RE(0, c)], yi = W[LGT_IM(0, c)];
+    const float xj = W[LGT_RE(1, c)], yj = W[LGT_IM(1, c)];
+    const float t0r = r.e0 * xi - r.r3 * yi + r.r2 * xj - r.r1 * yj, t0i = r.e0 * yi + r.r3 * xi + r.r2 * yj + r.r1 * xj;
+    W[LGT_RE(0, c)] += t0r;
+    W[LGT_IM(0, c)] += t0i;
+    if (c == 0) K.ad[0] += t0i;
+    if (c == 2) K.ao[2] = fmaf(0.5f, t0r, K.ao[2]), K.ao[3] = fmaf(0.5f, t0i, K.ao[3]);
+    if (c > 0) {
+      const float t1r = -r.r2 * xi - r.r1 * yi + r.e0 * xj + r.r3 * yj, t1i = -r.r2 * yi + r.r1 * xi + r.e0 * yj - r.r3 * xj;
+      if (c == 1) W[LGT_RE(1, 1)] += t1r, K.ad[1] += t1i;
+      else K.ao[4] = fmaf(0.5f, t1r, K.ao[4]), K.ao[5] = fmaf(0.5f, t1i, K.ao[5]);
+    }
+  }
+  // (0,2)
+  r = rf[1] = subgroup_rotation<ALGO>(W[LGT_RE(0, 0)] + W[LGT_RE(2, 2)], 2.0f * K.ao[3], 2.0f * K.ao[2],
+                                      K.ad[0] - K.ad[2], omega, (uint64_t)draws.y < sr_thr);
+#pragma unroll
+  for (int c = 1; c < 3; c++) {
+    const float xi = W[LGT_RE(0, c)], yi = W[LGT_IM(0, c)];
+    const float xj = W[LGT_RE(2, c)], yj = W[LGT_IM(2, c)];
+    const float tr = -r.r2 * xi - r.r1 * yi + r.e0 * xj + r.r3 * yj, ti = -r.r2 * yi + r.r1 * xi + r.e0 * yj - r.r3 * xj;
+    if (c == 1) K.ao[4] = fmaf(-0.5f, tr, K.ao[4]), K.ao[5] = fmaf(0.5f, ti, K.ao[5]);  // A_12 -= conj(t_21) / 2
+    else W[LGT_RE(2, 2)] += tr, K.ad[2] += ti;
+  }
+  // (1,2)
+  rf[2] = subgroup_rotation<ALGO>(W[LGT_RE(1, 1)] + W[LGT_RE(2, 2)], 2.0f * K.ao[5], 2.0f * K.ao[4],
+                                  K.ad[1] - K.ad[2], omega, (uint64_t)draws.z < sr_thr);
 }
 
 // delta = g - 1 for g = R2 R1 R0 from FP32 near-identity elements, written with
@@ -260,9 +349,9 @@ __device__ __forceinline__ void float_delta(const RotF rf[3], float d[18]) {
   d[LGT_RE(2, 2)] = (dr[2] + dr[1]) + t0r, d[LGT_IM(2, 2)] = (di[2] + di[1]) + t0i;
 }
 
-// G <- g G on rows 0 and 1: D <- D + delta + delta D, D a pair (rows 0, 1),
-// delta and the small product delta D in FP32 (dh: D's high parts with row 2)
-__device__ __forceinline__ void d_update_lite(f2 D[12], const float dh[18], const float d[18]) {
+// G <- g G on rows 0 and 1: D <- D + (delta + delta D), D a pair (rows 0, 1), the
+// increment in FP32 (dh: D's high parts with row 2)
+__device__ __forceinline__ void d_update(f2 D[12], const float dh[18], const float d[18]) {
 #pragma unroll
   for (int i = 0; i < 2; i++)
 #pragma unroll
@@ -270,11 +359,13 @@ __device__ __forceinline__ void d_update_lite(f2 D[12], const float dh[18], cons
       float re = 0.0f, im = 0.0f;
 #pragma unroll
       for (int k = 0; k < 3; k++) {
-        re += d[LGT_RE(i, k)] * dh[LGT_RE(k, j)] - d[LGT_IM(i, k)] * dh[LGT_IM(k, j)];
-        im += d[LGT_RE(i, k)] * dh[LGT_IM(k, j)] + d[LGT_IM(i, k)] * dh[LGT_RE(k, j)];
+        re = fmaf(d[LGT_RE(i, k)], dh[LGT_RE(k, j)], re);
+        re = fmaf(-d[LGT_IM(i, k)], dh[LGT_IM(k, j)], re);
+        im = fmaf(d[LGT_RE(i, k)], dh[LGT_IM(k, j)], im);
+        im = fmaf(d[LGT_IM(i, k)], dh[LGT_RE(k, j)], im);
       }
-      D[LGT_RE(i, j)] = pair_add(pair_add(D[LGT_RE(i, j)], f2{d[LGT_RE(i, j)], 0.0f}), f2{re, 0.0f});
-      D[LGT_IM(i, j)] = pair_add(pair_add(D[LGT_IM(i, j)], f2{d[LGT_IM(i, j)], 0.0f}), f2{im, 0.0f});
+      D[LGT_RE(i, j)] = pair_add(D[LGT_RE(i, j)], f2{d[LGT_RE(i, j)] + re, 0.0f});
+      D[LGT_IM(i, j)] = pair_add(D[LGT_IM(i, j)], f2{d[LGT_IM(i, j)] + im, 0.0f});
     }
 }
 

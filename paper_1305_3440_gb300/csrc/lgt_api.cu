@@ -222,7 +222,7 @@ struct lgt_ctx {
   void *G;        // accumulated transformation of the bulk phase; D = G - 1 of the anchored polish
   int fixed;      // the bulk sweeps keep the links in u32 as loaded and update G alone (lgt_fixed_links)
   int g_dirty;    // bulk sweeps have run since the load: G != 1 (fixed: the working links are G u32 G^+)
-  void *k0;       // anchored polish: K0 (pairs)
+  void *k0;       // anchored polish: K0 (AnchorK0)
   int anchored;   // anchored polish: K0, the FP32-12 copy in u32 and D refer to the field in u64
   int d_dirty;    // anchored polish: D != 0 (sweeps since the field in u64 was last formed)
   int64_t anchor_sweeps;  // anchored polish: sweeps since the last anchor set-up

@@ -106,11 +106,10 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_staged(const BatchSweep 
   sweep_body_f32_staged<GAUGE, ALGO>(a, p, t, local - t * J.nbx);
 }
 
-// Anchored polish sweeps of the batch at <= 80 registers (6 blocks of 128
-// threads = 24 warps per SM, as launch configuration 11 of the single-lattice
-// polish kernels): the update is issue-bound, so the extra warps pay.
+// Anchored polish sweeps of the batch at <= 128 registers (4 blocks of 128 threads
+// per SM).
 template <int GAUGE, int ALGO>
-__global__ void __launch_bounds__(128, 6) k_sweep_batch_anchor(const BatchSweep *jobs, int n, int p, int s) {
+__global__ void __launch_bounds__(128, 4) k_sweep_batch_anchor(const BatchSweep *jobs, int n, int p, int s) {
   const int b = batch_block(jobs, p);
   const int k = batch_row(&jobs[0].block_begin, (int)sizeof(BatchSweep), n, b);
   const BatchSweep &J = jobs[k];
@@ -119,7 +118,7 @@ __global__ void __launch_bounds__(128, 6) k_sweep_batch_anchor(const BatchSweep 
   a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
   const int local = b - J.block_begin;
   const int t = local / J.nbx;
-  sweep_body_anchor<GAUGE, ALGO>(a, p, t, local - t * J.nbx, J.nbx);
+  sweep_body_anchor<GAUGE, ALGO, 1>(a, p, t, local - t * J.nbx);
 }
 
 typedef void (*batch_fn)(const BatchSweep *, int, int, int);

@@ -26,7 +26,7 @@ enum { FMT_F64 = 0, FMT_F32_18 = 1, FMT_F32_12 = 2 };
 // converts in place.
 enum { FMT_PAIR = 3 };
 // Anchored polish (lgt_anchor.cuh): not a link format but the sweep over a
-// fixed anchor field (FP32-12 copy + K0 pairs) with D = G - 1 as pairs.
+// fixed anchor field (FP32-12 copy + K0) with D = G - 1 as pairs.
 enum { FMT_ANCHOR = 4 };
 // Fixed-link bulk sweeps (lgt_fixed.cuh): likewise sweeps, over FP32 links that
 // stay as loaded (18- or 12-real storage) with G as the only state.

@@ -360,6 +360,92 @@ __device__ __forceinline__ void sweep_body_fixed(const SweepArgs &a, int p, int 
   fused_store<float, 1>(a, p, t, bx, acc);
 }
 
+// terms loaded ahead (80 registers, configuration 11: none)
+__host__ __device__ constexpr int anchor_depth(int cfg) { return cfg == 11 ? 0 : (cfg == 3 ? 1 : 2); }
+
+// Anchored polishing sweep (lgt_anchor.cuh): a.links = FP32-12 copy of the anchor
+// field U', a.G = D = G - 1 (pairs), a.aux = K0.  One thread per site; only D(x) is
+// written.  Loads, indices and the unrolled terms as sweep_body_fixed's.  Against
+// the looped body with K in pairs at 80 registers: 32^4 half-sweep 84 -> 67 us (5.8
+// TB/s in compulsory bytes), 8^4 8.0 -> 6.3 us.
+template <int GAUGE, int ALGO, int DEPTH>
+__device__ __forceinline__ void sweep_body_anchor(const SweepArgs &a, int p, int t, int bx) {
+  if (a.active && !a.active[t]) return;
+  const int j = bx * (int)blockDim.x + (int)threadIdx.x;
+  float acc[2] = {0.0f, 0.0f};
+  if (j < a.g.vs_half) {
+    constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
+    constexpr int N = 2 * (4 - MU0);
+    const SiteNb nb(a.g, a.inv_half1, a.inv_n2, p, t, j);
+    const int i = t * a.g.vs_half + j;
+    const int q = p ^ 1;
+    const size_t S = (size_t)a.g.vh * 16;
+    const char *const L = (const char *)a.links;
+    const char *const Lp = L + (size_t)(p * 12) * S, *const Lq = L + (size_t)(q * 12) * S;
+    const char *const Dq = (const char *)a.G + (size_t)(q * 3) * S;
+    char *const Dp = (char *)a.G + (size_t)(p * 3) * S;
+    char *const Dl = Dp + 6 * S;  // the low parts
+    const unsigned o = (unsigned)i * 16u;
+    auto load = [&](int n, FixedTerm<FMT_F32_12> &T) {
+      const int mu = MU0 + n / 2;
+      const bool fwd = !(n & 1);
+      const unsigned on = o + (unsigned)(nb.offset(a.g, mu, fwd ? 1 : -1) * 16);
+      const char *const Lb = (fwd ? Lp : Lq) + (size_t)(mu * 3) * S;
+#pragma unroll
+      for (int k = 0; k < 3; k++) put4(T.u, k, ld_link(Lb + (size_t)k * S, fwd ? o : on));
+#pragma unroll
+      for (int k = 0; k < 3; k++) put4(T.g, k, ld_G(Dq + (size_t)k * S, on));
+    };
+    // C(x) = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+  (small; FP32)
+    float C[18], dh[18];
+    mat_zero(C);
+    {
+      FixedTerm<FMT_F32_12> T[DEPTH + 1];
+#pragma unroll
+      for (int n = 0; n < DEPTH; n++) load(n, T[n]);
+#pragma unroll
+      for (int n = 0; n < N; n++) {
+        if (n + DEPTH < N) load(n + DEPTH, T[(n + DEPTH) % (DEPTH + 1)]);
+        if (n == N - 1) {
+#pragma unroll
+          for (int k = 0; k < 3; k++) put4(dh, k, ld_G(Dp + (size_t)k * S, o));
+        }
+        FixedTerm<FMT_F32_12> &X = T[n % (DEPTH + 1)];
+        fma_row2(X.u);
+        small_row2(X.g);
+        if (!(n & 1)) acc_mul_dag(X.u, X.g, C);
+        else acc_dag_mul_dag(X.u, X.g, C);
+      }
+    }
+    small_row2(dh);  // D(x), high parts
+    float d[18];
+    {
+      AnchorK0 k0;
+      K0IO::load(a.aux, a.g.vh, p, i, k0);
+      AnchorK K;
+      anchor_K(k0, C, dh, K);
+      anchor_violation(K, acc[0], acc[1]);
+      uint4 draws = make_uint4(0, 0, 0, 0);
+      if (ALGO == ALGO_SR) draws = sr_draws(a, nb.coords(t));
+      RotF rf[3];
+      anchor_local_update<ALGO>(K, rf, (float)a.omega, a.sr_thr, draws);
+      float_delta(rf, d);
+    }
+    f2 D[12];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      const float4 l = ld_G(Dl + (size_t)k * S, o);
+      D[4 * k] = {dh[4 * k], l.x};
+      D[4 * k + 1] = {dh[4 * k + 1], l.y};
+      D[4 * k + 2] = {dh[4 * k + 2], l.z};
+      D[4 * k + 3] = {dh[4 * k + 3], l.w};
+    }
+    d_update(D, dh, d);
+    DIO::store_pair(a.G, a.g.vh, p, i, D);
+  }
+  fused_store<float, 1>(a, p, t, bx, acc);
+}
+
 // ------------------------------------------------------------ working links
 // The bulk's working link U_mu(x) -> G(x) U_mu(x) G(x+mu)^+ in FP32 (12-real
 // storage: rows 0, 1 formed and row 2 rebuilt, as a stored working link; 18-real:

@@ -429,11 +429,12 @@ cudaError_t launch_loop_decide(LoopState *L, const double *fused_totals, int gau
 // Anchored polish: G = 1 + D (pairs) applied in FP64 (as launch_apply_G).
 cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, void *u64_out, double *aos_out,
                            int skip_temporal, void *scratch, cudaStream_t st);
-// Anchored polish set-up from the FP64 field u64: K0 (pairs), the FP32-12 copy
+// Anchored polish set-up from the FP64 field u64: K0 (AnchorK0), the FP32-12 copy
 // in u32, D = 0.
 cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge,
                                 cudaStream_t st);
-// bytes of K0 and of D (hi and lo arrays) for vh sites per parity
+// bytes of K0 (112 B per site; 144 where the bulk phase keeps the orthonormal FP64 G
+// there, see launch_apply_G) and of D (hi and lo arrays) for vh sites per parity
 inline size_t k0_bytes(int vh) { return (size_t)vh * 2 * 144; }
 inline size_t d_bytes(int vh) { return (size_t)vh * 2 * 96; }
 cudaError_t launch_convert_pair(const Geom &g, void *u, int to_pair, cudaStream_t st);

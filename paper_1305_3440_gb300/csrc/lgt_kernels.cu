@@ -380,7 +380,7 @@ cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st) {
 
 // ------------------------------------------------ anchored polish set-up
 // For every site of either parity: K0(x) = sum_{mu >= mu0} U_mu(x) + U_mu(x-mu)^+
-// in FP64, stored as FP32 pairs (hi = fl32(v), lo = fl32(v - hi)); the FP32-12
+// in FP64, stored as its Hermitian and anti-Hermitian parts (AnchorK0); the FP32-12
 // copy of the site's forward links; D(x) = 0.
 __global__ void k_anchor_setup(Geom g, const void *u64, void *u32, void *K0, void *D, int mu0) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -403,14 +403,10 @@ __global__ void k_anchor_setup(Geom g, const void *u64, void *u32, void *K0, voi
       acc_add_dag(K, u);
     }
   }
-  f2 k2[18], z[18];
+  f2 z[18];
 #pragma unroll
-  for (int k = 0; k < 18; k++) {
-    const float hi = __double2float_rn(K[k]);
-    k2[k] = {hi, __double2float_rn(K[k] - (double)hi)};
-    z[k] = {0.0f, 0.0f};
-  }
-  K0IO::store(K0, g.vh, p, i, k2);
+  for (int k = 0; k < 18; k++) z[k] = {0.0f, 0.0f};
+  K0IO::store(K0, g.vh, p, i, K);
   DIO::store_pair(D, g.vh, p, i, z);
 }
 

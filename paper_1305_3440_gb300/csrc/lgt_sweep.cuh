@@ -1202,71 +1202,10 @@ __device__ __forceinline__ void sweep_body_pair(const SweepArgs &a, int p, int t
 }
 
 
-// Anchored polishing sweep (lgt_anchor.cuh): a.links = FP32-12 copy of the
-// anchor field U', a.G = D = G - 1 (pairs), a.aux = K0 (pairs).  One thread per
-// site; only D(x) is written.  K(x) in pair precision; rotations, delta = g - 1
-// and delta D in FP32; D accumulated as a pair.
-template <int GAUGE, int ALGO>
-__device__ __forceinline__ void sweep_body_anchor(const SweepArgs &a, int p, int t, int bx, int nbx) {
-  typedef LinkIO<FMT_F32_12> IO;
-  if (a.active && !a.active[t]) return;
-  const int j = bx * blockDim.x + threadIdx.x;
-  float acc[2] = {0.0f, 0.0f};
-  if (j < a.g.vs_half) {
-    constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
-    const Coords c = coords_in_slice(a.g, p, t, j);
-    const int i = t * a.g.vs_half + j;
-    const int q = p ^ 1;
-    // C(x) = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+  (small; FP32)
-    float C[18];
-    mat_zero(C);
-#pragma unroll 1
-    for (int mu = MU0; mu < 4; mu++) {
-      float u[18], dn[18];
-      IO::load(a.links, a.g.vh, p, mu, i, u);
-      DIO::load_hi(a.G, a.g.vh, q, cb_shift(a.g, c, mu, +1), dn);
-      acc_mul_dag(u, dn, C);
-      const int nb = cb_shift(a.g, c, mu, -1);
-      IO::load(a.links, a.g.vh, q, mu, nb, u);
-      DIO::load_hi(a.G, a.g.vh, q, nb, dn);
-      acc_dag_mul_dag(u, dn, C);
-    }
-    // M = K0 + C, then K = M + D(x) M (the small product in FP32)
-    f2 K[18];
-    K0IO::load(a.aux, a.g.vh, p, i, K);
-#pragma unroll
-    for (int e = 0; e < 18; e++) K[e] = pair_add(K[e], f2{C[e], 0.0f});
-    float dh[18];  // D(x), high parts, row 2 rebuilt
-    DIO::load_hi(a.G, a.g.vh, p, i, dh);
-    {
-      float mh[18], dm[18];
-#pragma unroll
-      for (int e = 0; e < 18; e++) mh[e] = K[e].hi;
-      mat_mul(dh, mh, dm);
-#pragma unroll
-      for (int e = 0; e < 18; e++) K[e] = pair_add(K[e], f2{dm[e], 0.0f});
-    }
-    pair_violation(K, acc[0], acc[1]);
-    uint4 draws = make_uint4(0, 0, 0, 0);
-    if (ALGO == ALGO_SR) draws = sr_draws(a, c);
-    RotF rf[3];
-    anchor_local_update<ALGO>(K, rf, (float)a.omega, a.sr_thr, draws);
-    float d[18];
-    float_delta(rf, d);
-    f2 D[18];
-    DIO::load_pair_rows(a.G, a.g.vh, p, i, D);
-    d_update_lite(D, dh, d);
-    DIO::store_pair(a.G, a.g.vh, p, i, D);
-  }
-  fused_store<float, 1>(a, p, t, bx, acc);
-}
-
-
 template <int FMT, int GAUGE, int ALGO>
 __device__ __forceinline__ void sweep_dispatch(const SweepArgs &a, int p, int t, int bx, int nbx) {
   if (FMT == FMT_F64) sweep_body_f64<GAUGE, ALGO>(a, p, t, bx, nbx);
   else if (FMT == FMT_PAIR) sweep_body_pair<GAUGE, ALGO>(a, p, t, bx, nbx);
-  else if (FMT == FMT_ANCHOR) sweep_body_anchor<GAUGE, ALGO>(a, p, t, bx, nbx);
   else sweep_body_f32<(FMT == FMT_F32_12 ? FMT_F32_12 : FMT_F32_18), GAUGE, ALGO>(a, p, t, bx, nbx);
 }
 

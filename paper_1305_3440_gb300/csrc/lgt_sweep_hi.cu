@@ -1,6 +1,7 @@
 // lgt_sweep_hi.cu -- the higher-precision half-sweep kernels: FP64 (every
 // operation in FP64), FP32-pair and anchored (the polishing sweeps), one
 // instantiation per gauge, algorithm and launch configuration.
+#include "lgt_fixed.cuh"
 #include "lgt_sweep.cuh"
 
 namespace lgt {
@@ -33,7 +34,7 @@ __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) 
   const SweepArgs a = resolve_loop(in);
   int t, bx;
   sweep_block_tile(a, p, t, bx);
-  sweep_body_anchor<GAUGE, ALGO>(a, p, t, bx, gridDim.x);
+  sweep_body_anchor<GAUGE, ALGO, anchor_depth(CFG)>(a, p, t, bx);
 }
 
 template <int CFG>
