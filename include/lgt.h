@@ -219,15 +219,16 @@ typedef struct {
  * server always) use none of these: they keep the FP32 links as loaded and update the accumulated
  * transformation G alone, K(x) = G(x) sum_mu [U_mu(x) G(x+mu)^+ +
  * U_mu(x-mu)^+ G(x-mu)^+], which is the K(x) of the rewritten links G U G^+;
- * tuned over the thread and register budgets of 3, 8 and 9.  The working links
+ * tuned over the thread and register budgets of 3, 8 and 9 and, four threads
+ * per site, 4.  The working links
  * are then G U G^+ formed in FP32 when they are asked for or measured.  FP32
  * rounding leaves such a field at theta ~ 6e-13 (rewritten links: 3e-14) but the
  * input transformed by G there too (rewritten links: 1e-8, G and the links
  * drifting apart), so the bulk phase of lgt_fix and of served jobs ends at theta <
  * max(theta_switch, 2e-12).
- * The anchored polish (the default after promotion) runs in 0-3 and in 11
- * (<= 80 registers, 24 warps per SM).  A configuration that a phase's kernel
- * lacks (4-15 after promotion, except 11 for the anchored polish; 7, 10 and
+ * The anchored polish (the default after promotion) runs in 0-3, in 4 (four
+ * threads per site) and in 11 (<= 80 registers, 24 warps per SM).  A
+ * configuration that a phase's kernel lacks (4-15 after promotion, except 4 and 11 for the anchored polish; 7, 10 and
  * 12-15 on FP32-18 links; all but 0-3, 13 and 14 in the maximally Abelian
  * gauge) falls back to configuration 0 for that phase.  Every
  * configuration groups the fused estimate by the same 8 sites; results differ

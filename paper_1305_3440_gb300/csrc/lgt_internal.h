@@ -237,7 +237,8 @@ struct SweepCfg {
 //    15:  64 threads, <= 112 registers, 9 blocks per SM: the links only in
 //         shared memory (24 KB), G loaded into registers beside the copies
 // The fixed-link bulk sweeps (FMT_FIX_*, lgt_fixed.cuh) are compiled for 3, 8 and
-// 9 (64 or 128 threads at <= 128 registers, 128 at <= 96).
+// 9 (64 or 128 threads at <= 128 registers, 128 at <= 96) and, four threads per
+// site, 4; the anchored polish for 4 too.
 // The one-thread and four-thread layouts form K(x) in the same order, the lean
 // ones link by link; every configuration groups the fused estimate by the same
 // 8 sites; results differ only in FP32 rounding (the order of K's sums and
@@ -264,9 +265,9 @@ __host__ __device__ constexpr int lgt_cfg_stage_chunks(int c) { return c == 15 ?
 __host__ __device__ constexpr int lgt_cfg_sites(int c) { return lgt_cfg_quad(c) ? lgt_cfg_threads(c) / 4 : lgt_cfg_threads(c); }
 // whether a storage format has kernels for a configuration
 __host__ __device__ constexpr bool lgt_cfg_supported(int fmt, int c) {
-  return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 8 || c == 9
+  return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 4 || c == 8 || c == 9
                                                   : c >= 0 && c < LGT_NCFG &&
-         (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && c == 11)) &&
+         (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && (c == 4 || c == 11))) &&
          (!(lgt_cfg_pipe(c) || lgt_cfg_stream(c) || lgt_cfg_staged(c)) || fmt == FMT_F32_12);
 }
 // the maximally Abelian gauge has kernels in the one-thread-per-site

@@ -11,7 +11,8 @@ __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) 
   const SweepArgs a = resolve_loop(in);
   int t, bx;
   sweep_block_tile(a, p, t, bx);
-  sweep_body_fixed<LFMT, GAUGE, ALGO, fixed_depth(LFMT, lgt_cfg_minblocks(CFG) * lgt_cfg_threads(CFG))>(a, p, t, bx);
+  if constexpr (lgt_cfg_quad(CFG)) sweep_body_fixed_quad<LFMT, GAUGE>(a, p, t, bx);
+  else sweep_body_fixed<LFMT, GAUGE, ALGO, fixed_depth(LFMT, lgt_cfg_minblocks(CFG) * lgt_cfg_threads(CFG))>(a, p, t, bx);
 }
 
 template <int CFG>
@@ -36,6 +37,7 @@ sweep_fn pick_sweep_fixed(int fmt, int gauge, int algo, int cfg) {
   const int lfmt = fmt == FMT_FIX_18 ? FMT_F32_18 : FMT_F32_12;
   switch (cfg) {
     case 3: return pick_cfg<3>(lfmt, gauge, algo);
+    case 4: return pick_cfg<4>(lfmt, gauge, algo);
     case 8: return pick_cfg<8>(lfmt, gauge, algo);
     case 9: return pick_cfg<9>(lfmt, gauge, algo);
   }

@@ -34,12 +34,13 @@ __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) 
   const SweepArgs a = resolve_loop(in);
   int t, bx;
   sweep_block_tile(a, p, t, bx);
-  sweep_body_anchor<GAUGE, ALGO, anchor_depth(CFG)>(a, p, t, bx);
+  if constexpr (lgt_cfg_quad(CFG)) sweep_body_anchor_quad<GAUGE, ALGO>(a, p, t, bx);
+  else sweep_body_anchor<GAUGE, ALGO, anchor_depth(CFG)>(a, p, t, bx);
 }
 
 template <int CFG>
 static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
-  if constexpr (CFG == 11) {  // 24 warps per SM at <= 80 registers: the anchored polish only
+  if constexpr (CFG == 4 || CFG == 11) {  // four threads per site; 24 warps per SM at <= 80 registers: the anchored polish only
     if (fmt != FMT_ANCHOR || algo == ALGO_SA || gauge == GAUGE_MAG) return nullptr;
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_anchor<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_anchor<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_COULOMB, ALGO_OR, CFG>;
@@ -78,6 +79,7 @@ sweep_fn pick_sweep_hi(int fmt, int gauge, int algo, int cfg) {
     case 1: return pick_cfg<1>(fmt, gauge, algo);
     case 2: return pick_cfg<2>(fmt, gauge, algo);
     case 3: return pick_cfg<3>(fmt, gauge, algo);
+    case 4: return pick_cfg<4>(fmt, gauge, algo);
     case 11: return pick_cfg<11>(fmt, gauge, algo);
   }
   return nullptr;

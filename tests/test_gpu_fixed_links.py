@@ -90,3 +90,81 @@ def test_working_field_is_measured_as_it_is_read(lgt, bulk, temporal):
     finally:
         lgt.lgt_destroy(ctx)
     assert np.array_equal(after, straight)
+
+
+_FORCED = """
+import sys
+import numpy as np
+sys.path.insert(0, {root!r}); sys.path.insert(0, {tests!r})
+import oracle as O
+from paper_1305_3440_gb300 import lgt, synth
+from lattice_np import check_fp32_bound, fp32_half_sweep_bound
+cfg = {cfg}
+near = synth.field((4, 4, 4, 8), 0.3, 1)
+O.fix(near, omega=1.7, tol=1e-12, max_sweeps=2000, check_every=1)
+for gauge in (O.LANDAU, O.COULOMB):
+    for dims in {dims}:
+        U = synth.field(dims, 0.5, 93)
+        for bulk in (lgt.LGT_FP32_18, lgt.LGT_FP32_12):
+            for parity in (0, 1):
+                ref = U.copy()
+                O.half_sweep(ref, parity, gauge=gauge, omega=1.7)
+                bound = fp32_half_sweep_bound(O.site_conditioning(U, parity, gauge=gauge, omega=1.7), parity, 16.0)
+                ctx = lgt.lgt_create(lgt.lgt_params_default(dims=dims, bulk=bulk, gauge=gauge, omega=1.7), U)
+                lgt.lgt_half_sweep(ctx, parity)
+                out = lgt.lgt_get_working_links(ctx, dims)
+                st = lgt.lgt_get_stats(ctx)
+                F, th, _, _ = lgt.lgt_estimate(ctx, dims[0])
+                lgt.lgt_destroy(ctx)
+                assert st.launch_config[0] == cfg, list(st.launch_config)
+                ratio, _, _ = check_fp32_bound(np.abs(out - ref), bound)
+                assert ratio <= 1.0, (gauge, dims, bulk, parity, ratio)
+                if parity == 0 and gauge == O.LANDAU:  # the parity-0 slots hold every link once
+                    assert abs(F - O.measure(U)["F"]) < 16 * 2.0**-24
+    if cfg not in (3, 4):
+        continue
+    for algo in (O.OR, O.SR):  # the anchored polish
+        kw = dict(gauge=gauge, algo=algo, omega=1.7, p=0.8, seed=5)
+        ref = near.copy()
+        O.sweeps(ref, 2, **kw)
+        ctx = lgt.lgt_create(lgt.lgt_params_default(dims=near.shape[:4], bulk=lgt.LGT_FP32_12, omega_polish=0.0, **kw), near)
+        lgt.lgt_promote(ctx)
+        lgt.lgt_sweep(ctx, 2)
+        out = lgt.lgt_get_links(ctx, near.shape[:4])
+        st = lgt.lgt_get_stats(ctx)
+        lgt.lgt_destroy(ctx)
+        assert st.launch_config[1] == cfg, list(st.launch_config)
+        err = np.abs(out - ref).max()
+        # theta of the field in this gauge sets |g - 1|, the angles are FP32
+        m = O.measure(near, gauge)
+        th = m["theta_t"].max() if gauge == O.COULOMB else m["theta"]
+        assert err < 1e-12 + 2e-6 * np.sqrt(th), (gauge, algo, err, th)
+print("ok")
+"""
+
+
+@pytest.mark.parametrize("cfg", [3, 4, 8, 9])
+def test_every_tuned_configuration(lgt, cfg, tmp_path):
+    """Each configuration the autotuner may pick for the fixed-link bulk and (3, 4)
+    the anchored polish -- one thread per site at three budgets, four threads per site
+    (4) -- forced through a tuning cache file, at the edges of its blocks and quads:
+    half-sweeps within the per-site FP32 bound of the oracle, the fused F, and two
+    polish sweeps within the accuracy of FP32 rotation angles."""
+    import os
+    import subprocess
+    import sys
+    import torch
+    here = os.path.dirname(os.path.abspath(__file__))
+    dims = [(2, 2, 2, 2), (2, 4, 6, 2), (2, 6, 10, 14), (4, 2, 2, 34)]
+    name = torch.cuda.get_device_name().replace(" ", "_")
+    cache = tmp_path / "tuned"
+    with open(cache, "w") as f:
+        for fmt in (4, 5, 6):  # anchored polish; fixed links, 18- and 12-real
+            for gauge in (0, 1):
+                for algo in (0, 1):
+                    for d in dims + [(4, 4, 4, 8)]:
+                        f.write(f"{fmt} {gauge} {algo} {d[0]} {d[1]} {d[2]} {d[3]} {name} {cfg if fmt > 4 or cfg < 5 else 0}\n")
+    code = _FORCED.format(root=os.path.dirname(here), tests=here, cfg=cfg, dims=dims)
+    r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, LGT_AUTOTUNE_CACHE=str(cache)),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout + r.stderr
