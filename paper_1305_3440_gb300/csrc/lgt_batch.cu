@@ -58,10 +58,10 @@ __global__ void __launch_bounds__(256) k_measure_batch(const BatchMeas *jobs, in
   measure_body<FMT>(J.a, t, p, rem - p * J.nbx, J.nbx);
 }
 
-// FP32 overrelaxation sweeps of the batch: the fixed-link update at launch configuration
-// 8's budget (128 threads, <= 128 registers, 4 blocks per SM).
-template <int LFMT, int GAUGE, int ALGO>
-__global__ void __launch_bounds__(128, 4) k_sweep_batch_fixed(const BatchSweep *jobs, int n, int p, int s) {
+// FP32 overrelaxation bulk and anchored polish sweeps of the batch (FMT_MIX): each
+// row's own body at 128 threads, <= 128 registers, 4 blocks per SM.
+__global__ void __launch_bounds__(128, 4) k_sweep_batch_mix(const BatchSweep *jobs, int n, int p, int s) {
+  pdl_enter();
   const int b = batch_block(jobs, p);
   const int k = batch_row(&jobs[0].block_begin, (int)sizeof(BatchSweep), n, b);
   const BatchSweep &J = jobs[k];
@@ -70,7 +70,17 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_fixed(const BatchSweep *
   a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
   const int local = b - J.block_begin;
   const int t = local / J.nbx;
-  sweep_body_fixed<LFMT, GAUGE, ALGO, fixed_depth(LFMT, 512)>(a, p, t, local - t * J.nbx);
+  const int bx = local - t * J.nbx;
+  switch (J.kind) {
+    case lgt_mix_kind(FMT_FIX_12, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_12, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_18, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_18, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, ALGO_OR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, ALGO_OR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_SR): sweep_body_anchor<GAUGE_LANDAU, ALGO_SR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_SR): sweep_body_anchor<GAUGE_COULOMB, ALGO_SR, 1>(a, p, t, bx); break;
+  }
 }
 
 // FP32-18 stochastic-relaxation sweeps of the batch: the lean one-thread layout (K streamed,
@@ -106,27 +116,7 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_staged(const BatchSweep 
   sweep_body_f32_staged<GAUGE, ALGO>(a, p, t, local - t * J.nbx);
 }
 
-// Anchored polish sweeps of the batch at <= 128 registers (4 blocks of 128 threads
-// per SM).
-template <int GAUGE, int ALGO>
-__global__ void __launch_bounds__(128, 4) k_sweep_batch_anchor(const BatchSweep *jobs, int n, int p, int s) {
-  const int b = batch_block(jobs, p);
-  const int k = batch_row(&jobs[0].block_begin, (int)sizeof(BatchSweep), n, b);
-  const BatchSweep &J = jobs[k];
-  SweepArgs a = J.a;
-  a.sweep += (unsigned long long)s;
-  a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
-  const int local = b - J.block_begin;
-  const int t = local / J.nbx;
-  sweep_body_anchor<GAUGE, ALGO, 1>(a, p, t, local - t * J.nbx);
-}
-
 typedef void (*batch_fn)(const BatchSweep *, int, int, int);
-
-static batch_fn pick_batch_anchor(int gauge, int algo) {
-  if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_batch_anchor<GAUGE_LANDAU, ALGO_SR> : k_sweep_batch_anchor<GAUGE_LANDAU, ALGO_OR>;
-  return algo == ALGO_SR ? k_sweep_batch_anchor<GAUGE_COULOMB, ALGO_SR> : k_sweep_batch_anchor<GAUGE_COULOMB, ALGO_OR>;
-}
 
 // the staged kernel's shared memory (27 chunks of 16 B per thread), opted in once per kernel
 static cudaError_t staged_smem(batch_fn fn, int block, int *smem) {
@@ -138,11 +128,6 @@ static cudaError_t staged_smem(batch_fn fn, int block, int *smem) {
   return e;
 }
 
-template <int LFMT>
-static batch_fn pick_batch_fixed(int gauge) {
-  return gauge == GAUGE_LANDAU ? k_sweep_batch_fixed<LFMT, GAUGE_LANDAU, ALGO_OR> : k_sweep_batch_fixed<LFMT, GAUGE_COULOMB, ALGO_OR>;
-}
-
 template <int FMT>
 static batch_fn pick_batch_fmt(int gauge, int algo) {
   if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_batch<FMT, GAUGE_LANDAU, ALGO_SR> : k_sweep_batch<FMT, GAUGE_LANDAU, ALGO_OR>;
@@ -150,15 +135,14 @@ static batch_fn pick_batch_fmt(int gauge, int algo) {
 }
 
 cudaError_t launch_half_sweep_batch(int fmt, int gauge, int algo, const BatchSweep *jobs, int n, int total_blocks,
-                                    int parity, int s, int block, cudaStream_t st) {
+                                    int parity, int s, int block, cudaStream_t st, bool after_sweep) {
   if (n <= 0 || total_blocks <= 0) return cudaSuccess;
   if (block != 128 || (gauge != GAUGE_LANDAU && gauge != GAUGE_COULOMB) || (algo != ALGO_OR && algo != ALGO_SR))
     return cudaErrorInvalidValue;
   batch_fn fn = nullptr;
   int smem = 0;
   if (fmt == FMT_F64) fn = pick_batch_fmt<FMT_F64>(gauge, algo);
-  else if (fmt == FMT_FIX_18 && algo == ALGO_OR) fn = pick_batch_fixed<FMT_F32_18>(gauge);
-  else if (fmt == FMT_FIX_12 && algo == ALGO_OR) fn = pick_batch_fixed<FMT_F32_12>(gauge);
+  else if (fmt == FMT_MIX) fn = k_sweep_batch_mix;
   else if (fmt == FMT_F32_18 && algo == ALGO_SR)
     fn = gauge == GAUGE_LANDAU ? k_sweep_batch_lean<FMT_F32_18, GAUGE_LANDAU, ALGO_SR> : k_sweep_batch_lean<FMT_F32_18, GAUGE_COULOMB, ALGO_SR>;
   else if (fmt == FMT_F32_12 && algo == ALGO_SR) {
@@ -167,10 +151,21 @@ cudaError_t launch_half_sweep_batch(int fmt, int gauge, int algo, const BatchSwe
     if (e != cudaSuccess) return e;
   }
   else if (fmt == FMT_PAIR) fn = pick_batch_fmt<FMT_PAIR>(gauge, algo);
-  else if (fmt == FMT_ANCHOR) fn = pick_batch_anchor(gauge, algo);
   if (!fn) return cudaErrorInvalidValue;
-  fn<<<total_blocks, block, smem, st>>>(jobs, n, parity & 1, s);
-  return cudaGetLastError();
+  if (fmt != FMT_MIX || !after_sweep) {
+    fn<<<total_blocks, block, smem, st>>>(jobs, n, parity & 1, s);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(total_blocks);
+  lc.blockDim = dim3(block);
+  lc.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, fn, jobs, n, parity & 1, s);
 }
 
 cudaError_t launch_measure_batch(int fmt, const BatchMeas *jobs, int n, int total_blocks, int block, cudaStream_t st) {

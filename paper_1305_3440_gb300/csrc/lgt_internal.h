@@ -172,6 +172,7 @@ struct BatchSweep {
   SweepArgs a;
   int block_begin;  // first block of this lattice in the batched grid
   int nbx;          // blocks per timeslice
+  int kind;         // FMT_MIX launches: the row's kernel, lgt_mix_kind
 };
 struct BatchMeas {
   MeasArgs a;
@@ -440,12 +441,22 @@ inline size_t k0_bytes(int vh) { return (size_t)vh * 2 * 144; }
 inline size_t d_bytes(int vh) { return (size_t)vh * 2 * 96; }
 cudaError_t launch_convert_pair(const Geom &g, void *u, int to_pair, cudaStream_t st);
 
+// FMT_MIX: one batched launch over lattices of the fixed-link bulk (either storage)
+// and of the anchored polish, in either gauge.  Their kernels have the same block
+// and register budget and a block runs one of them, so a served half-sweep is one
+// launch instead of up to four one after the other, each too small to fill the chip.
+constexpr int FMT_MIX = 16;
+constexpr bool lgt_mixes(int fmt) { return fmt == FMT_FIX_18 || fmt == FMT_FIX_12 || fmt == FMT_ANCHOR; }
+constexpr int lgt_mix_kind(int fmt, int gauge, int algo) { return (fmt * 2 + gauge) * 2 + algo; }
+
 // Batched half-sweep over n lattices of one kernel variant (fmt, gauge,
 // algo): blocks [jobs[k].block_begin, jobs[k+1].block_begin) belong to
 // lattice k; total_blocks in all.  s: sweep offset within the batch (SR
 // counter and reunitarisation schedule: jobs[k].a.sweep + s, count_base + s).
+// after_sweep: the launch before it in the stream is a batched half-sweep too
+// (FMT_MIX: programmatic stream serialisation, as the single-lattice sweeps).
 cudaError_t launch_half_sweep_batch(int fmt, int gauge, int algo, const BatchSweep *jobs, int n, int total_blocks,
-                                    int parity, int s, int block, cudaStream_t st);
+                                    int parity, int s, int block, cudaStream_t st, bool after_sweep = false);
 // Batched exact measurement over n lattices of one storage format.
 cudaError_t launch_measure_batch(int fmt, const BatchMeas *jobs, int n, int total_blocks, int block, cudaStream_t st);
 // Fill the batch row of a lattice (pointers into its workspace).

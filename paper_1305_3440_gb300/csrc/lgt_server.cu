@@ -4,9 +4,9 @@
 //   1. admit queued jobs (FIFO) while their device footprint fits the HBM
 //      budget: allocate, upload, ingest (SU(3) check), measure;
 //   2. advance every live job by up to check_every sweeps: for each sweep and
-//      parity, one batched half-sweep launch per kernel variant (storage
-//      format x gauge x algorithm) covers the sites of all live jobs of that
-//      variant;
+//      parity, one batched half-sweep launch covers the sites of all live FP32
+//      overrelaxation and anchored polish jobs (FMT_MIX), and one per kernel variant
+//      (storage format x gauge x algorithm) those of the others;
 //   3. one batched reduction of the sweeps' fused estimates gives each job's
 //      F and theta; jobs that start, or whose estimate says converged, get a
 //      batched exact measurement instead (with the plaquette when it
@@ -95,6 +95,10 @@ struct Job {
   int sweep_fmt() const {
     return phase == 3 ? (int)FMT_ANCHOR : (phase == 0 && fixed ? lgt_fixed_fmt(bulk_fmt) : work_fmt());
   }
+  // batched launch of its sweeps: (format, gauge, algorithm)
+  int batch_fmt() const { return lgt_mixes(sweep_fmt()) ? FMT_MIX : sweep_fmt(); }
+  int batch_gauge() const { return lgt_mixes(sweep_fmt()) ? 0 : cfg.gauge; }
+  int batch_algo() const { return lgt_mixes(sweep_fmt()) ? 0 : cfg.algo; }
   void *sweep_links() const { return (phase == 0 || phase == 3) ? u32 : u64; }
   int skip_temporal() const { return (prm.gauge == LGT_COULOMB && !prm.transform_temporal) ? 1 : 0; }
   double theta_of(const double *tot) const {
@@ -331,6 +335,7 @@ cudaError_t issue(lgt_server *s, const TickPlan &P) {
                            s->stream)) != cudaSuccess)
     return e;
   size_t si = 0;
+  bool after_sweep = false;
   for (int sw = 0; sw < P.kmax; sw++) {
     const size_t first = si;
     while (si < P.segs.size() && P.segs[si].s == sw) si++;
@@ -338,8 +343,9 @@ cudaError_t issue(lgt_server *s, const TickPlan &P) {
       for (size_t q = first; q < si; q++) {
         const Segment &g = P.segs[q];
         e = launch_half_sweep_batch(g.fmt, g.gauge, g.algo, s->d_sweep + g.offset, g.n, g.blocks, parity, sw,
-                                    kServerBlock, s->stream);
+                                    kServerBlock, s->stream, after_sweep);
         if (e != cudaSuccess) return e;
+        after_sweep = g.fmt == FMT_MIX;  // its successor may be placed while it drains
       }
   }
   if (P.nfrows && (e = launch_fused_finish_batch(s->d_fused, (int)P.nfrows, P.fblocks, s->stream)) != cudaSuccess)
@@ -381,19 +387,19 @@ cudaError_t tick(lgt_server *s) {
   std::vector<BatchSweep> rows;
   std::vector<Job *> order(live);
   std::stable_sort(order.begin(), order.end(), [](const Job *a, const Job *b) {
-    const int ka = (a->sweep_fmt() * 2 + a->cfg.gauge) * 2 + a->cfg.algo;
-    const int kb = (b->sweep_fmt() * 2 + b->cfg.gauge) * 2 + b->cfg.algo;
+    const int ka = (a->batch_fmt() * 2 + a->batch_gauge()) * 2 + a->batch_algo();
+    const int kb = (b->batch_fmt() * 2 + b->batch_gauge()) * 2 + b->batch_algo();
     return ka < kb;
   });
   for (int sw = 0; sw < kmax; sw++) {
     size_t i = 0;
     while (i < order.size()) {
       const Job *h = order[i];
-      Segment seg = {h->sweep_fmt(), h->cfg.gauge, h->cfg.algo, sw, rows.size(), 0, 0};
+      Segment seg = {h->batch_fmt(), h->batch_gauge(), h->batch_algo(), sw, rows.size(), 0, 0};
       size_t k = i;
       for (; k < order.size(); k++) {
         Job *j = order[k];
-        if (j->sweep_fmt() != seg.fmt || j->cfg.gauge != seg.gauge || j->cfg.algo != seg.algo) break;
+        if (j->batch_fmt() != seg.fmt || j->batch_gauge() != seg.gauge || j->batch_algo() != seg.algo) break;
         if (sw >= j->nthis) continue;
         BatchSweep r{};
         fill_sweep_args(&r.a, j->g, j->sweep_links(), (j->phase == 0 || j->phase == 3) ? j->G : nullptr, j->ws,
@@ -403,6 +409,7 @@ cudaError_t tick(lgt_server *s) {
         r.a.count_base = j->sweeps_bulk;
         r.block_begin = seg.blocks;
         r.nbx = j->nbx;
+        r.kind = lgt_mix_kind(j->sweep_fmt(), j->cfg.gauge, j->cfg.algo);
         rows.push_back(r);
         seg.n++;
         seg.blocks += j->nbx * j->g.nt;
