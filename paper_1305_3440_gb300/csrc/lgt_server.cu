@@ -802,10 +802,13 @@ extern "C" lgt_status lgt_poll(lgt_server *s, uint64_t job_id, lgt_result *res, 
   }
   Job *j = it->second;
   if (j->state != JOB_DONE) return LGT_EAGAIN;
+  s->jobs.erase(it);
+  // the job is this call's alone now: its links are copied without the lock, which
+  // the worker takes after every tick
+  lk.unlock();
   if (res) *res = j->res;
   if (links_out && !j->output.empty()) memcpy(links_out, j->output.data(), j->output.size() * sizeof(double));
   const lgt_status st = (lgt_status)j->res.status;
-  s->jobs.erase(it);
   delete j;
   return st;
 }
