@@ -58,9 +58,17 @@ __device__ __forceinline__ int tile_units(const Geom &g) {
   return (int)(left < kPairs ? left : kPairs) * kPairUnits;
 }
 
+// (a caller's buffer need only be aligned to its doubles: 8-byte accesses then)
+__device__ __forceinline__ bool wide(const double *aos) { return (reinterpret_cast<uintptr_t>(aos) & 15) == 0; }
+
 __device__ __forceinline__ void tile_load(const Geom &g, const double *aos, double2 *tile) {
-  const double2 *src = reinterpret_cast<const double2 *>(aos) + (size_t)blockIdx.x * kPairs * kPairUnits;
+  const double *from = aos + (size_t)blockIdx.x * kPairs * kPairUnits * 2;
   const int n = tile_units(g);
+  if (!wide(aos)) {
+    for (int u = (int)threadIdx.x; u < n; u += kThreads) tile[u + u / kPairUnits] = make_double2(from[2 * u], from[2 * u + 1]);
+    return;
+  }
+  const double2 *src = reinterpret_cast<const double2 *>(from);
 #pragma unroll
   for (int k = 0; k < kPairs * kPairUnits / kThreads; k++) {
     const int u = k * kThreads + (int)threadIdx.x;
@@ -69,8 +77,17 @@ __device__ __forceinline__ void tile_load(const Geom &g, const double *aos, doub
 }
 
 __device__ __forceinline__ void tile_store(const Geom &g, double *aos, const double2 *tile) {
-  double2 *dst = reinterpret_cast<double2 *>(aos) + (size_t)blockIdx.x * kPairs * kPairUnits;
+  double *to = aos + (size_t)blockIdx.x * kPairs * kPairUnits * 2;
   const int n = tile_units(g);
+  if (!wide(aos)) {
+    for (int u = (int)threadIdx.x; u < n; u += kThreads) {
+      const double2 v = tile[u + u / kPairUnits];
+      to[2 * u] = v.x;
+      to[2 * u + 1] = v.y;
+    }
+    return;
+  }
+  double2 *dst = reinterpret_cast<double2 *>(to);
 #pragma unroll
   for (int k = 0; k < kPairs * kPairUnits / kThreads; k++) {
     const int u = k * kThreads + (int)threadIdx.x;

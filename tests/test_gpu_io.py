@@ -70,6 +70,52 @@ def test_output_is_the_same_before_and_after_promotion(lgt, polish, gauge):
     assert np.array_equal(out[0], out[1])
 
 
+@pytest.mark.parametrize("bulk", ["fp64", "fp32_18", "fp32_12"])
+def test_device_buffers_need_only_the_alignment_of_doubles(lgt, bulk):
+    """Links read from and written to device memory that is 8 but not 16 bytes aligned:
+    load, output with and without a transformation, the working links, and the
+    measurement straight from the caller's buffer, against the aligned buffer's."""
+    import torch
+    dims = (4, 6, 10, 14)
+    U = synth.field(dims, 0.5, 44)
+    n = 2 * U.size
+    p = lgt.lgt_params_default(dims=dims, bulk=getattr(lgt, "LGT_" + bulk.upper()), omega=1.6)
+    got = {}
+    for off in (0, 1):
+        def buffer():
+            t = torch.full((n + 2,), 7.0, dtype=torch.float64, device="cuda")
+            return t, t[off:off + n].view(dims + (4, 3, 3, 2))
+        whole, links = buffer()
+        assert links.data_ptr() % 16 == 8 * off
+        links.copy_(torch.view_as_real(torch.from_numpy(U)))
+        sums = torch.empty(8 + 2 * dims[0], dtype=torch.float64, device="cuda")
+        outs = []
+        ctx = lgt.lgt_create(p, links)
+        try:
+            for sweeps in (0, 2):
+                if sweeps:
+                    lgt.lgt_sweep(ctx, sweeps)
+                for read in (lgt.lgt_get_links, lgt.lgt_get_working_links):
+                    w, out = buffer()
+                    read(ctx, out=out)
+                    assert float(w[n + off:].min()) == 7.0 and (off == 0 or float(w[0]) == 7.0)
+                    outs.append(out.cpu().numpy())
+            lgt.lgt_promote(ctx)
+            lgt.lgt_sweep(ctx, 1)
+            w, out = buffer()
+            lgt.lgt_get_links(ctx, out=out)
+            outs.append(out.cpu().numpy())
+        finally:
+            lgt.lgt_destroy(ctx)
+        torch.cuda.synchronize()
+        lgt.lgt_measure_noalloc(dims, links, sums)
+        torch.cuda.synchronize()
+        got[off] = outs + [sums.cpu().numpy()]
+    assert np.array_equal(got[0][0], U.view(np.float64).reshape(dims + (4, 3, 3, 2)))
+    for a, b in zip(got[0], got[1]):
+        assert np.array_equal(a, b)
+
+
 def _deviation(u):
     """max(|U^+ U - 1|, |Re det U - 1|, |Im det U|) of one matrix in extended precision."""
     u = u.astype(np.clongdouble)
