@@ -66,20 +66,24 @@ __device__ __forceinline__ void load_field_d(const Geom &g, const void *links, c
   }
 }
 
-// X += s * (U - U^dagger)
+// X += s (U - U^dagger) / 2 on the diagonal, s (U - U^dagger) above it (what
+// traceless_norm reads; 15 operations of the FP64 pipe, which bounds the measurement)
 __device__ __forceinline__ void acc_antiherm(double X[18], const double u[18], double s) {
+#pragma unroll
+  for (int a = 0; a < 3; a++) X[LGT_IM(a, a)] += s * u[LGT_IM(a, a)];
 #pragma unroll
   for (int a = 0; a < 3; a++)
 #pragma unroll
-    for (int b = 0; b < 3; b++) {
-      X[LGT_RE(a, b)] += s * (u[LGT_RE(a, b)] - u[LGT_RE(b, a)]);
-      X[LGT_IM(a, b)] += s * (u[LGT_IM(a, b)] + u[LGT_IM(b, a)]);
+    for (int b = a + 1; b < 3; b++) {
+      X[LGT_RE(a, b)] = (X[LGT_RE(a, b)] + s * u[LGT_RE(a, b)]) - s * u[LGT_RE(b, a)];
+      X[LGT_IM(a, b)] = (X[LGT_IM(a, b)] + s * u[LGT_IM(a, b)]) + s * u[LGT_IM(b, a)];
     }
 }
 
-// tr[D D^dagger] for D = traceless part of X/(2i), X anti-Hermitian
+// tr[D D^dagger] for D = traceless part of X/(2i), X anti-Hermitian (as
+// acc_antiherm holds it)
 __device__ __forceinline__ double traceless_norm(const double X[18]) {
-  const double d0 = 0.5 * X[LGT_IM(0, 0)], d1 = 0.5 * X[LGT_IM(1, 1)], d2 = 0.5 * X[LGT_IM(2, 2)];
+  const double d0 = X[LGT_IM(0, 0)], d1 = X[LGT_IM(1, 1)], d2 = X[LGT_IM(2, 2)];
   const double tr3 = (d0 + d1 + d2) * (1.0 / 3.0);
   double s = (d0 - tr3) * (d0 - tr3) + (d1 - tr3) * (d1 - tr3) + (d2 - tr3) * (d2 - tr3);
 #pragma unroll
@@ -128,19 +132,22 @@ __device__ __forceinline__ void measure_body(const MeasArgs &a, int t, int p, in
       }
       v[2] = traceless_norm(XL);
     }
-    for (int mu = 0; mu < 4 && !a.mag; mu++) {
-      double u[18];
-      load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, p, mu, i, u);
-      const double rt = u[LGT_RE(0, 0)] + u[LGT_RE(1, 1)] + u[LGT_RE(2, 2)];
-      v[0] += rt;
-      acc_antiherm(XL, u, 1.0);
-      if (mu > 0) {
-        v[1] += rt;
-        acc_antiherm(XS, u, 1.0);
+    for (int mu = 3; mu >= 0 && !a.mag; mu--) {  // the spatial directions, then the temporal one beside their sum
+      if (mu == 0) {
+#pragma unroll
+        for (int k = 0; k < 18; k++) XL[k] = XS[k];
+        v[1] = v[0];
       }
-      load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, q, mu, cb_shift(a.g, c, mu, -1), u);
-      acc_antiherm(XL, u, -1.0);
-      if (mu > 0) acc_antiherm(XS, u, -1.0);
+      auto add = [&](double *Y) {
+        double u[18];
+        load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, p, mu, i, u);
+        v[0] += u[LGT_RE(0, 0)] + u[LGT_RE(1, 1)] + u[LGT_RE(2, 2)];
+        acc_antiherm(Y, u, 1.0);
+        load_field_d<FMT>(a.g, a.links, a.G, a.skip_temporal, q, mu, cb_shift(a.g, c, mu, -1), u);
+        acc_antiherm(Y, u, -1.0);
+      };
+      if (mu > 0) add(XS);
+      else add(XL);
     }
     if (!a.mag) {
       v[2] = traceless_norm(XL);
