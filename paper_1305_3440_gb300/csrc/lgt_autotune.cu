@@ -51,7 +51,7 @@ void load_file_locked() {
   int fmt, gauge, algo, nt, n3, n2, n1, block;
   char name[256];
   while (fscanf(f, "%d %d %d %d %d %d %d %255s %d", &fmt, &gauge, &algo, &nt, &n3, &n2, &n1, name, &block) == 9)
-    if (block >= 0 && block < LGT_NCFG) g_tuned[TuneKey(fmt, gauge, algo, nt, n3, n2, n1, name)] = block;
+    if (block >= 0 && block < LGT_NCFG_TUNED) g_tuned[TuneKey(fmt, gauge, algo, nt, n3, n2, n1, name)] = block;
   fclose(f);
 }
 
@@ -93,7 +93,7 @@ int lgt_tune_sweep(const Geom &g, int fmt, const SweepCfg &cfg, void *links, voi
   // (as the driver issues them: 8 launches, or one streaming launch)
   float best_ms = 1e30f;
   int best = 0;
-  for (int k = 0; k < LGT_NCFG && e == cudaSuccess; k++) {
+  for (int k = 0; k < LGT_NCFG_TUNED && e == cudaSuccess; k++) {
     if (!lgt_cfg_supported_gauge(fmt, cfg.gauge, k)) continue;
     e = launch_half_sweeps(fmt, g, links, G, ws, cfg, 0, 2, 0, 0, 0, 0, k, st, aux);
     for (int trial = 0; trial < 3 && e == cudaSuccess; trial++) {

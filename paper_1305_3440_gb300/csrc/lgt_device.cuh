@@ -339,7 +339,7 @@ __device__ __forceinline__ R rsqrt_t(R x);
 template <>
 __device__ __forceinline__ float rsqrt_t<float>(float x) { return rsqrtf(x); }
 template <>
-__device__ __forceinline__ double rsqrt_t<double>(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }  // one function, not a root and a division
 
 // Reunitarise: Gram-Schmidt on rows 0 and 1, then row 2 = conj(row0 x row1).
 template <typename R>

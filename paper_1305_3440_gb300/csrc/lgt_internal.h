@@ -246,9 +246,15 @@ struct SweepCfg {
 // where the compiler fuses multiply-adds).  The maximally Abelian gauge has
 // kernels in configurations 0-3, 13 and 14.
 constexpr int LGT_NCFG = 16;
-__host__ __device__ constexpr int lgt_cfg_threads(int c) { return (c == 2 || c == 5) ? 256 : ((c == 3 || c == 14 || c == 15) ? 64 : 128); }
+// Beyond the configurations a caller may name, the autotuner has
+//    16: 32 threads, <= 255 registers, FP64 sweeps.  Those are bound by the FP64
+//        pipe of each SM, so a small lattice wants its sites spread evenly over
+//        the SMs: 12^4 has 84 blocks of 128 sites a half-sweep for 152 SMs (48 us;
+//        with 324 blocks of 32 sites the fullest SM has 96 sites).
+constexpr int LGT_NCFG_TUNED = 17;
+__host__ __device__ constexpr int lgt_cfg_threads(int c) { return c == 16 ? 32 : (c == 2 || c == 5) ? 256 : ((c == 3 || c == 14 || c == 15) ? 64 : 128); }
 __host__ __device__ constexpr int lgt_cfg_minblocks(int c) {
-  return c == 1 ? 3
+  return c == 16 ? 8 : c == 1 ? 3
                 : (c == 3 ? 8
                           : (c == 4 ? 4
                                     : (c == 5 ? 2
@@ -267,6 +273,7 @@ __host__ __device__ constexpr int lgt_cfg_sites(int c) { return lgt_cfg_quad(c) 
 // whether a storage format has kernels for a configuration
 __host__ __device__ constexpr bool lgt_cfg_supported(int fmt, int c) {
   return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 4 || c == 8 || c == 9
+         : c == 16 ? fmt == FMT_F64
                                                   : c >= 0 && c < LGT_NCFG &&
          (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && (c == 4 || c == 11))) &&
          (!(lgt_cfg_pipe(c) || lgt_cfg_stream(c) || lgt_cfg_staged(c)) || fmt == FMT_F32_12);
@@ -277,7 +284,7 @@ __host__ __device__ constexpr bool lgt_cfg_mag(int c) { return (c >= 0 && c <= 3
 // whether a (format, gauge) pair has kernels for a configuration
 __host__ __device__ constexpr bool lgt_cfg_supported_gauge(int fmt, int gauge, int c) {
   return lgt_cfg_supported(fmt, c) &&
-         (gauge != GAUGE_MAG || (lgt_cfg_mag(c) && (fmt == FMT_F64 || fmt == FMT_F32_18 || fmt == FMT_F32_12)));
+         (gauge != GAUGE_MAG || ((lgt_cfg_mag(c) || c == 16) && (fmt == FMT_F64 || fmt == FMT_F32_18 || fmt == FMT_F32_12)));
 }
 // dynamic shared memory of the pipelined and streaming configurations: 2 buffers x 27 chunks x 16 B per thread
 constexpr int LGT_PIPE_SMEM_PER_THREAD = 2 * 27 * 16;

@@ -45,8 +45,8 @@ static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_anchor<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_anchor<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_COULOMB, ALGO_OR, CFG>;
   }
-  if (gauge == GAUGE_MAG) {  // maximally Abelian gauge: FP64 only here, configurations 0-3
-    if constexpr (lgt_cfg_mag(CFG)) {
+  if (gauge == GAUGE_MAG) {  // maximally Abelian gauge: FP64 only here, configurations 0-3 and 16
+    if constexpr (lgt_cfg_mag(CFG) || CFG == 16) {
       if (fmt == FMT_F64 && algo == ALGO_OR) return k_sweep_f64<GAUGE_MAG, ALGO_OR, CFG>;
       if (fmt == FMT_F64 && algo == ALGO_SR) return k_sweep_f64<GAUGE_MAG, ALGO_SR, CFG>;
     }
@@ -61,6 +61,7 @@ static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_f64<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_f64<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_f64<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_f64<GAUGE_COULOMB, ALGO_OR, CFG>;
   }
+  if constexpr (CFG == 16) return nullptr;
   if (algo == ALGO_SA) return nullptr;
   if (fmt == FMT_PAIR) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_pair<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_pair<GAUGE_LANDAU, ALGO_OR, CFG>;
@@ -81,6 +82,7 @@ sweep_fn pick_sweep_hi(int fmt, int gauge, int algo, int cfg) {
     case 3: return pick_cfg<3>(fmt, gauge, algo);
     case 4: return pick_cfg<4>(fmt, gauge, algo);
     case 11: return pick_cfg<11>(fmt, gauge, algo);
+    case 16: return pick_cfg<16>(fmt, gauge, algo);
   }
   return nullptr;
 }
