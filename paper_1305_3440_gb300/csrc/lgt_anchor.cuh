@@ -132,11 +132,20 @@ struct AnchorK0 {
   float tau;             // Im tr K0 / 3
 };
 struct K0IO {
+  // EARLY: before the wait for the launch before (relaxed at GPU scope, as ld_early)
+  template <bool EARLY>
   static __device__ __forceinline__ void load(const void *base, int vh, int p, int i, AnchorK0 &k) {
     const float4 *b = reinterpret_cast<const float4 *>(base) + (size_t)(p * 7) * vh + i;
     float4 v[7];
 #pragma unroll
-    for (int c = 0; c < 7; c++) v[c] = __ldcs(b + (size_t)c * vh);
+    for (int c = 0; c < 7; c++) {
+      if constexpr (EARLY)
+        asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+                     : "=f"(v[c].x), "=f"(v[c].y), "=f"(v[c].z), "=f"(v[c].w)
+                     : "l"(b + (size_t)c * vh)
+                     : "memory");
+      else v[c] = __ldcs(b + (size_t)c * vh);
+    }
     k.h[0] = v[0].x, k.h[1] = v[0].y, k.h[2] = v[0].z, k.ad[0] = v[0].w;
     k.ad[1] = v[1].x, k.ad[2] = v[1].y, k.ho[0] = v[1].z, k.ho[1] = v[1].w;
     k.ho[2] = v[2].x, k.ho[3] = v[2].y, k.ho[4] = v[2].z, k.ho[5] = v[2].w;

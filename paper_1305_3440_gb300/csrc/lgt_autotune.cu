@@ -4,7 +4,8 @@
 // block and a register budget, see lgt_internal.h), which trade occupancy
 // against register spills; the best one depends on the kernel variant and the
 // lattice shape.  The tuner times every configuration on a scratch field of
-// unit links (the kernels' work does not depend on the link values), keeps the
+// unit links (with unit G where the links are fixed, with zero K0 and D for the
+// anchored polish: the kernels' work does not depend on the values), keeps the
 // fastest per (format, gauge, algorithm, dims, GPU) for the life of the
 // process, and, if the environment variable LGT_AUTOTUNE_CACHE names a file,
 // reads earlier results from it and appends new ones.

@@ -33,6 +33,7 @@ __device__ __forceinline__ int batch_block(const BatchSweep *jobs, int p) {
   return (jobs[0].a.snake && (p & 1)) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x;
 }
 
+// FP64 and FP32-pair sweeps of the batch
 template <int FMT, int GAUGE, int ALGO>
 __global__ void __launch_bounds__(256) k_sweep_batch(const BatchSweep *jobs, int n, int p, int s) {
   const int b = batch_block(jobs, p);
@@ -43,7 +44,8 @@ __global__ void __launch_bounds__(256) k_sweep_batch(const BatchSweep *jobs, int
   a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
   const int local = b - J.block_begin;
   const int t = local / J.nbx;
-  sweep_dispatch<FMT, GAUGE, ALGO>(a, p, t, local - t * J.nbx, J.nbx);
+  if constexpr (FMT == FMT_F64) sweep_body_f64<GAUGE, ALGO>(a, p, t, local - t * J.nbx, J.nbx);
+  else sweep_body_pair<GAUGE, ALGO>(a, p, t, local - t * J.nbx, J.nbx);
 }
 
 template <int FMT>
@@ -59,7 +61,8 @@ __global__ void __launch_bounds__(256) k_measure_batch(const BatchMeas *jobs, in
 }
 
 // FP32 overrelaxation bulk and anchored polish sweeps of the batch (FMT_MIX): each
-// row's own body at 128 threads, <= 128 registers, 4 blocks per SM.
+// row's own body at 128 threads, <= 128 registers, 4 blocks per SM.  The job table
+// is read first, so the wait for the launch before is the kernel's first act.
 __global__ void __launch_bounds__(128, 4) k_sweep_batch_mix(const BatchSweep *jobs, int n, int p, int s) {
   pdl_enter();
   const int b = batch_block(jobs, p);
@@ -72,14 +75,14 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_mix(const BatchSweep *jo
   const int t = local / J.nbx;
   const int bx = local - t * J.nbx;
   switch (J.kind) {
-    case lgt_mix_kind(FMT_FIX_12, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_FIX_12, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_FIX_18, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_FIX_18, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, ALGO_OR, 1>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, ALGO_OR, 1>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_SR): sweep_body_anchor<GAUGE_LANDAU, ALGO_SR, 1>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_SR): sweep_body_anchor<GAUGE_COULOMB, ALGO_SR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_12, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_12, 512), false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_12, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_12, 512), false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_18, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_18, 512), false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_18, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_18, 512), false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, ALGO_OR, 1, false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, ALGO_OR, 1, false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_SR): sweep_body_anchor<GAUGE_LANDAU, ALGO_SR, 1, false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_SR): sweep_body_anchor<GAUGE_COULOMB, ALGO_SR, 1, false>(a, p, t, bx); break;
   }
 }
 

@@ -52,6 +52,24 @@ __device__ __forceinline__ float2 ld_link2(const char *base, unsigned off) {
   asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(base + off));
   return v;
 }
+// The same before griddepcontrol.wait (what a launch may read before it: see
+// sweep_start): relaxed at GPU scope, so served by L2 whatever this SM's L1 holds.
+__device__ __forceinline__ float4 ld_early(const char *base, unsigned off) {
+  float4 v;
+  asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(base + off)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_early2(const char *base, unsigned off) {
+  float2 v;
+  asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v2.f32 {%0,%1}, [%2];"
+               : "=f"(v.x), "=f"(v.y)
+               : "l"(base + off)
+               : "memory");
+  return v;
+}
 __device__ __forceinline__ float4 ld_G(const char *base, unsigned off) {
   float4 v;
   asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
@@ -195,18 +213,39 @@ __device__ __forceinline__ void local_update_rows(float W[18], float g[12], floa
   g[LGT_IM(1, 2)] = bi[2] * ar[1] - br[2] * ai[1];
 }
 
-// Terms loaded ahead: 2 at the 128-register budget (512 threads per SM), 1 at
-// fewer registers or with the longer 18-real links.
+// Neighbours' G loaded ahead, in terms: 2 at the 128-register budget (512 threads
+// per SM), 1 at fewer registers or with the longer 18-real links, 4 or 3 at 255
+// registers, which also hold the links of all terms (fixed_links_ahead).
 __host__ __device__ constexpr int fixed_depth(int lfmt, int threads_per_sm) {
-  return lfmt == FMT_F32_12 && threads_per_sm <= 512 ? 2 : 1;
+  return threads_per_sm <= 256 ? (lfmt == FMT_F32_12 ? 4 : 3) : (lfmt == FMT_F32_12 && threads_per_sm <= 512 ? 2 : 1);
 }
+// links loaded before the wait for the launch before, in terms
+__host__ __device__ constexpr int fixed_links_ahead(int depth, int n) { return depth >= 3 ? n : depth + 1; }
 
-// The links and the neighbour's G of one term of M(x): rows 0, 1 of U (three
-// rows with 18-real storage) and rows 0, 1 of G.
-template <int LFMT>
-struct FixedTerm {
-  float u[18], g[18];
-};
+// Start of a sweep over links that no sweep writes.  What the launches before it
+// in its run leave alone -- the links, K0, the activity mask -- may be read before
+// griddepcontrol.wait: a launch is let in only after every block of the launch
+// before has passed its own wait, and a run's first launch, which is a plain one,
+// after all that wrote those.  G, the loop state and the slots are touched after
+// the wait only.  On a lattice that leaves the SMs room the next launch's blocks
+// so have their indices and links ready when the launch before ends, and only the
+// G loads and the update lie between one launch's end and the next one's; on a
+// large one they fill the last wave's gap.  Half-sweep with all loads after the
+// wait -> as here: 8^4 bulk 3.46 -> 2.99 us, polish 3.87 -> 3.33; 16^4 5.13 -> 4.83
+// and 6.73 -> 6.32; 32^4 bulk 46.0 -> 44.7.
+__device__ __forceinline__ bool sweep_slice_active(const SweepArgs &a, int t) {
+  if (!a.active) return true;
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u8 %0, [%1];" : "=r"(v) : "l"(a.active + t) : "memory");
+  return v != 0;
+}
+// the wait, and the arguments with the loop state's values (PDL: false where the
+// kernel has waited)
+template <bool PDL>
+__device__ __forceinline__ SweepArgs sweep_start(const SweepArgs &in) {
+  if constexpr (PDL) pdl_enter();
+  return resolve_loop(in);
+}
 
 // Rows 0, 1 of G orthonormalised to first order in their error.  G is a factor
 // of every K(x) around it and row 2 of every product is rebuilt from rows 0, 1,
@@ -250,25 +289,25 @@ __device__ __forceinline__ void orthonormalise_rows(float r[12]) {
 // the product and its row 2 from those (it is in SU(3)); each entry is formed
 // before it is added, one rounding at M's size per term.
 template <int LFMT>
-__device__ __forceinline__ void fixed_term(FixedTerm<LFMT> &C, bool fwd, float M[18]) {
+__device__ __forceinline__ void fixed_term(float u[18], float g[18], bool fwd, float M[18]) {
   float r[18];
   if (fwd) {
-    fma_row2(C.g);
+    fma_row2(g);
     if constexpr (LFMT == FMT_F32_12) {
-      rows_mul_dag(C.u, C.g, r);
+      rows_mul_dag(u, g, r);
       fma_row2(r);
     } else {
-      mat_mul_dag(C.u, C.g, r);
+      mat_mul_dag(u, g, r);
     }
     acc_add(M, r);
   } else {
     if constexpr (LFMT == FMT_F32_12) {
-      fma_row2(C.u);
-      rows_mul(C.g, C.u, r);
+      fma_row2(u);
+      rows_mul(g, u, r);
       fma_row2(r);
     } else {
-      fma_row2(C.g);
-      mat_mul(C.g, C.u, r);
+      fma_row2(g);
+      mat_mul(g, u, r);
     }
     acc_add_dag(M, r);
   }
@@ -288,58 +327,71 @@ __device__ __forceinline__ void fixed_term(FixedTerm<LFMT> &C, bool fwd, float M
 // fastest configuration: 12-real links 32^4 Landau 59.7 -> 43 us, 64^4 Landau
 // 1034 -> 700 us and 48^3x96 Coulomb 620 -> 360 us (both at 6.3 to 6.6 TB/s of
 // DRAM traffic); 18-real links 14x10x12x18 6.2 -> 5.2 us.
-template <int LFMT, int GAUGE, int ALGO, int DEPTH>
-__device__ __forceinline__ void sweep_body_fixed(const SweepArgs &a, int p, int t, int bx) {
+template <int LFMT, int GAUGE, int ALGO, int DEPTH, bool PDL = true>
+__device__ __forceinline__ void sweep_body_fixed(const SweepArgs &in, int p, int t, int bx) {
   constexpr bool kRows = LFMT == FMT_F32_12;  // row 2 of a link is rebuilt, not stored
-  if (a.active && !a.active[t]) return;       // whole block belongs to one slice
+  constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
+  constexpr int N = 2 * (4 - MU0);
+  constexpr int NU = fixed_links_ahead(DEPTH, N), DG = DEPTH < N ? DEPTH : N;
+  constexpr int NC = kRows ? 3 : 4;  // 16-byte chunks per link
+  if (!sweep_slice_active(in, t)) {  // whole block belongs to one slice
+    if constexpr (PDL) pdl_enter();  // (a launch ends only after the one before it)
+    return;
+  }
   const int j = bx * (int)blockDim.x + (int)threadIdx.x;
+  const bool valid = j < in.g.vs_half;
+  const SiteNb nb(in.g, in.inv_half1, in.inv_n2, p, t, valid ? j : 0);
+  const int q = p ^ 1;
+  const size_t S = (size_t)in.g.vh * 16;  // bytes of one chunk's stream
+  const char *const L = (const char *)in.links;
+  const char *const Lp = L + (size_t)(p * 4 * NC) * S, *const Lq = L + (size_t)(q * 4 * NC) * S;
+  const char *const L2 = L + 32 * S;  // 18-real storage: the float2 chunk's streams
+  const char *const Gq = (const char *)in.G + (size_t)(q * 3) * S;
+  char *const Gp = (char *)in.G + (size_t)(p * 3) * S;
+  const unsigned o = (unsigned)(t * in.g.vs_half + j) * 16u;
+  // term n: direction MU0 + n / 2, forward link if n is even
+  auto site = [&](int n) { return o + (unsigned)(nb.offset(in.g, MU0 + n / 2, (n & 1) ? -1 : 1) * 16); };
+  float U[NU][18], G[DG + 1][18];
+  auto load_u = [&](int n, bool early) {
+    const int mu = MU0 + n / 2;
+    const bool fwd = !(n & 1);
+    const char *const Lb = (fwd ? Lp : Lq) + (size_t)(mu * NC) * S;
+    const unsigned ou = fwd ? o : site(n);
+#pragma unroll
+    for (int k = 0; k < NC; k++) put4(U[n % NU], k, early ? ld_early(Lb + (size_t)k * S, ou) : ld_link(Lb + (size_t)k * S, ou));
+    if (!kRows) {
+      const char *const Lw = L2 + (size_t)((fwd ? p : q) * 4 + mu) * (S / 2);
+      const float2 w = early ? ld_early2(Lw, ou / 2) : ld_link2(Lw, ou / 2);
+      U[n % NU][16] = w.x, U[n % NU][17] = w.y;
+    }
+  };
+  auto load_g = [&](int n) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) put4(G[n % (DG + 1)], k, ld_G(Gq + (size_t)k * S, site(n)));
+  };
+  if (valid) {
+#pragma unroll
+    for (int n = 0; n < NU; n++) load_u(n, true);
+  }
+  const SweepArgs a = sweep_start<PDL>(in);
   float acc[2] = {0.0f, 0.0f};
-  if (j < a.g.vs_half) {
-    constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
-    constexpr int N = 2 * (4 - MU0);
-    const SiteNb nb(a.g, a.inv_half1, a.inv_n2, p, t, j);
-    const int i = t * a.g.vs_half + j;
-    const int q = p ^ 1;
-    const size_t S = (size_t)a.g.vh * 16;  // bytes of one chunk's stream
-    constexpr int NC = kRows ? 3 : 4;      // 16-byte chunks per link
-    const char *const L = (const char *)a.links;
-    const char *const Lp = L + (size_t)(p * 4 * NC) * S, *const Lq = L + (size_t)(q * 4 * NC) * S;
-    const char *const L2 = L + 32 * S;  // 18-real storage: the float2 chunk's streams
-    const char *const Gq = (const char *)a.G + (size_t)(q * 3) * S;
-    char *const Gp = (char *)a.G + (size_t)(p * 3) * S;
-    const unsigned o = (unsigned)i * 16u;
-    // term n: direction MU0 + n / 2, forward link if n is even
-    auto load = [&](int n, FixedTerm<LFMT> &T) {
-      const int mu = MU0 + n / 2;
-      const bool fwd = !(n & 1);
-      const unsigned on = o + (unsigned)(nb.offset(a.g, mu, fwd ? 1 : -1) * 16);
-      const char *const Lb = (fwd ? Lp : Lq) + (size_t)(mu * NC) * S;
-      const unsigned ou = fwd ? o : on;
-#pragma unroll
-      for (int k = 0; k < NC; k++) put4(T.u, k, ld_link(Lb + (size_t)k * S, ou));
-      if (!kRows) {
-        const float2 w = ld_link2(L2 + (size_t)((fwd ? p : q) * 4 + mu) * (S / 2), ou / 2);
-        T.u[16] = w.x, T.u[17] = w.y;
-      }
-#pragma unroll
-      for (int k = 0; k < 3; k++) put4(T.g, k, ld_G(Gq + (size_t)k * S, on));
-    };
+  if (valid) {
     float W[18], gx[18];
     {
       float M[18];
       mat_zero(M);
-      FixedTerm<LFMT> T[DEPTH + 1];
 #pragma unroll
-      for (int n = 0; n < DEPTH; n++) load(n, T[n]);
+      for (int n = 0; n < DG; n++) load_g(n);
 #pragma unroll
       for (int n = 0; n < N; n++) {
-        if (n + DEPTH < N) {
-          load(n + DEPTH, T[(n + DEPTH) % (DEPTH + 1)]);
-        } else if (n + DEPTH == N) {
+        if (n + DG < N) {
+          if (n > 0 && n + NU - 1 < N) load_u(n + NU - 1, false);
+          load_g(n + DG);
+        } else if (n + DG == N) {
 #pragma unroll
           for (int k = 0; k < 3; k++) put4(gx, k, ld_G(Gp + (size_t)k * S, o));
         }
-        fixed_term<LFMT>(T[n % (DEPTH + 1)], !(n & 1), M);
+        fixed_term<LFMT>(U[n % NU], G[n % (DG + 1)], !(n & 1), M);
       }
       fma_row2(gx);
       mat_mul(gx, M, W);  // K(x) = G(x) M(x)
@@ -365,48 +417,58 @@ __device__ __forceinline__ void sweep_body_fixed(const SweepArgs &a, int p, int 
 // sum M(x) to all four, which then run the same update, and three of them store a
 // chunk of G each.  For lattices that leave most of the chip's schedulers with a
 // warp or none: the chain of a site is about half as long.  The autotuner takes it
-// up to 10^4 sites or so (half-sweep at 8^4: bulk 4.0 -> 3.6 us, polish 6.3 -> 3.9;
-// at 12^4 one thread per site is ahead in the bulk, 4.3 us).
+// up to 10^4 sites or so (half-sweep at 8^4: bulk 4.0 -> 3.5 us, polish 6.3 -> 3.9,
+// both 3.0 and 3.3 with the links read early; at 12^4 one thread per site is ahead
+// in the bulk).
 template <int LFMT, int GAUGE>
-__device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &a, int p, int t, int bx) {
-  if (a.active && !a.active[t]) return;  // whole block belongs to one slice
+__device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &in, int p, int t, int bx) {
+  if (!sweep_slice_active(in, t)) {  // whole block belongs to one slice
+    pdl_enter();
+    return;
+  }
   constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
   constexpr int NC = LFMT == FMT_F32_12 ? 3 : 4;
   const int m = (int)threadIdx.x & 3;
   const int j = bx * (int)(blockDim.x >> 2) + (int)(threadIdx.x >> 2);
-  const bool valid = j < a.g.vs_half;  // the shuffles below need every lane
-  const SiteNb nb(a.g, a.inv_half1, a.inv_n2, p, t, valid ? j : 0);
-  const int i = t * a.g.vs_half + (valid ? j : 0);
+  const bool valid = j < in.g.vs_half;  // the shuffles below need every lane
+  const SiteNb nb(in.g, in.inv_half1, in.inv_n2, p, t, valid ? j : 0);
+  const int i = t * in.g.vs_half + (valid ? j : 0);
   const int q = p ^ 1;
-  const size_t S = (size_t)a.g.vh * 16;
-  const char *const L = (const char *)a.links;
-  const char *const Gq = (const char *)a.G + (size_t)(q * 3) * S;
-  char *const Gp = (char *)a.G + (size_t)(p * 3) * S;
+  const size_t S = (size_t)in.g.vh * 16;
+  const char *const L = (const char *)in.links;
+  const char *const Gq = (const char *)in.G + (size_t)(q * 3) * S;
+  char *const Gp = (char *)in.G + (size_t)(p * 3) * S;
   const unsigned o = (unsigned)i * 16u;
   float M[18], W[18], gx[18];
   mat_zero(M);
-  FixedTerm<LFMT> T[2];
+  float U[2][18], G[2][18];
+  unsigned on[2];
+#pragma unroll
+  for (int d = 0; d < 2; d++) {  // forward, backward
+    on[d] = o + (unsigned)(nb.offset(in.g, m, d ? -1 : 1) * 16);
+    const unsigned ou = d ? on[d] : o;
+    const int pu = d ? q : p;
+    if (m >= MU0) {
+#pragma unroll
+      for (int k = 0; k < NC; k++) put4(U[d], k, ld_early(L + (size_t)((pu * 4 + m) * NC + k) * S, ou));
+      if (LFMT == FMT_F32_18) {
+        const float2 w = ld_early2(L + 32 * S + (size_t)(pu * 4 + m) * (S / 2), ou / 2);
+        U[d][16] = w.x, U[d][17] = w.y;
+      }
+    }
+  }
+  const SweepArgs a = sweep_start<true>(in);
   if (m >= MU0) {
 #pragma unroll
-    for (int d = 0; d < 2; d++) {  // forward, backward
-      const unsigned on = o + (unsigned)(nb.offset(a.g, m, d ? -1 : 1) * 16);
-      const unsigned ou = d ? on : o;
-      const int pu = d ? q : p;
+    for (int d = 0; d < 2; d++)
 #pragma unroll
-      for (int k = 0; k < NC; k++) put4(T[d].u, k, ld_link(L + (size_t)((pu * 4 + m) * NC + k) * S, ou));
-      if (LFMT == FMT_F32_18) {
-        const float2 w = ld_link2(L + 32 * S + (size_t)(pu * 4 + m) * (S / 2), ou / 2);
-        T[d].u[16] = w.x, T[d].u[17] = w.y;
-      }
-#pragma unroll
-      for (int k = 0; k < 3; k++) put4(T[d].g, k, ld_G(Gq + (size_t)k * S, on));
-    }
+      for (int k = 0; k < 3; k++) put4(G[d], k, ld_G(Gq + (size_t)k * S, on[d]));
   }
 #pragma unroll
   for (int k = 0; k < 3; k++) put4(gx, k, ld_G(Gp + (size_t)k * S, o));
   if (m >= MU0) {
-    fixed_term<LFMT>(T[0], true, M);
-    fixed_term<LFMT>(T[1], false, M);
+    fixed_term<LFMT>(U[0], G[0], true, M);
+    fixed_term<LFMT>(U[1], G[1], false, M);
   }
 #pragma unroll
   for (int e = 0; e < 18; e++) M[e] += __shfl_xor_sync(0xffffffffu, M[e], 1);
@@ -432,68 +494,80 @@ __device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &a, int p,
   fused_store<float, 4>(a, p, t, bx, acc);
 }
 
-// terms loaded ahead (80 registers, configuration 11: none)
-__host__ __device__ constexpr int anchor_depth(int cfg) { return cfg == 11 ? 0 : (cfg == 3 ? 1 : 2); }
+// neighbours' D loaded ahead, in terms (80 registers, configuration 11: none)
+__host__ __device__ constexpr int anchor_depth(int cfg) { return cfg == 16 ? 4 : (cfg == 11 ? 0 : (cfg == 3 ? 1 : 2)); }
 
 // Anchored polishing sweep (lgt_anchor.cuh): a.links = FP32-12 copy of the anchor
 // field U', a.G = D = G - 1 (pairs), a.aux = K0.  One thread per site; only D(x) is
 // written.  Loads, indices and the unrolled terms as sweep_body_fixed's.  Against
 // the looped body with K in pairs at 80 registers: 32^4 half-sweep 84 -> 67 us (5.8
 // TB/s in compulsory bytes), 8^4 8.0 -> 6.3 us.
-template <int GAUGE, int ALGO, int DEPTH>
-__device__ __forceinline__ void sweep_body_anchor(const SweepArgs &a, int p, int t, int bx) {
-  if (a.active && !a.active[t]) return;
+template <int GAUGE, int ALGO, int DEPTH, bool PDL = true>
+__device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, int t, int bx) {
+  constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
+  constexpr int N = 2 * (4 - MU0);
+  constexpr int NU = fixed_links_ahead(DEPTH, N), DG = DEPTH < N ? DEPTH : N;
+  if (!sweep_slice_active(in, t)) {
+    if constexpr (PDL) pdl_enter();
+    return;
+  }
   const int j = bx * (int)blockDim.x + (int)threadIdx.x;
+  const bool valid = j < in.g.vs_half;
+  const SiteNb nb(in.g, in.inv_half1, in.inv_n2, p, t, valid ? j : 0);
+  const int i = t * in.g.vs_half + j;
+  const int q = p ^ 1;
+  const size_t S = (size_t)in.g.vh * 16;
+  const char *const L = (const char *)in.links;
+  const char *const Lp = L + (size_t)(p * 12) * S, *const Lq = L + (size_t)(q * 12) * S;
+  const char *const Dq = (const char *)in.G + (size_t)(q * 3) * S;
+  char *const Dp = (char *)in.G + (size_t)(p * 3) * S;
+  char *const Dl = Dp + 6 * S;  // the low parts
+  const unsigned o = (unsigned)i * 16u;
+  auto site = [&](int n) { return o + (unsigned)(nb.offset(in.g, MU0 + n / 2, (n & 1) ? -1 : 1) * 16); };
+  float U[NU][18], G[DG + 1][18];
+  AnchorK0 k0;
+  auto load_u = [&](int n, bool early) {
+    const bool fwd = !(n & 1);
+    const char *const Lb = (fwd ? Lp : Lq) + (size_t)((MU0 + n / 2) * 3) * S;
+    const unsigned ou = fwd ? o : site(n);
+#pragma unroll
+    for (int k = 0; k < 3; k++) put4(U[n % NU], k, early ? ld_early(Lb + (size_t)k * S, ou) : ld_link(Lb + (size_t)k * S, ou));
+  };
+  auto load_g = [&](int n) {
+#pragma unroll
+    for (int k = 0; k < 3; k++) put4(G[n % (DG + 1)], k, ld_G(Dq + (size_t)k * S, site(n)));
+  };
+  if (valid) {
+#pragma unroll
+    for (int n = 0; n < NU; n++) load_u(n, true);
+    if (NU == N) K0IO::load<true>(in.aux, in.g.vh, p, i, k0);
+  }
+  const SweepArgs a = sweep_start<PDL>(in);
   float acc[2] = {0.0f, 0.0f};
-  if (j < a.g.vs_half) {
-    constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
-    constexpr int N = 2 * (4 - MU0);
-    const SiteNb nb(a.g, a.inv_half1, a.inv_n2, p, t, j);
-    const int i = t * a.g.vs_half + j;
-    const int q = p ^ 1;
-    const size_t S = (size_t)a.g.vh * 16;
-    const char *const L = (const char *)a.links;
-    const char *const Lp = L + (size_t)(p * 12) * S, *const Lq = L + (size_t)(q * 12) * S;
-    const char *const Dq = (const char *)a.G + (size_t)(q * 3) * S;
-    char *const Dp = (char *)a.G + (size_t)(p * 3) * S;
-    char *const Dl = Dp + 6 * S;  // the low parts
-    const unsigned o = (unsigned)i * 16u;
-    auto load = [&](int n, FixedTerm<FMT_F32_12> &T) {
-      const int mu = MU0 + n / 2;
-      const bool fwd = !(n & 1);
-      const unsigned on = o + (unsigned)(nb.offset(a.g, mu, fwd ? 1 : -1) * 16);
-      const char *const Lb = (fwd ? Lp : Lq) + (size_t)(mu * 3) * S;
-#pragma unroll
-      for (int k = 0; k < 3; k++) put4(T.u, k, ld_link(Lb + (size_t)k * S, fwd ? o : on));
-#pragma unroll
-      for (int k = 0; k < 3; k++) put4(T.g, k, ld_G(Dq + (size_t)k * S, on));
-    };
+  if (valid) {
     // C(x) = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+  (small; FP32)
     float C[18], dh[18];
     mat_zero(C);
-    {
-      FixedTerm<FMT_F32_12> T[DEPTH + 1];
 #pragma unroll
-      for (int n = 0; n < DEPTH; n++) load(n, T[n]);
+    for (int n = 0; n < DG; n++) load_g(n);
 #pragma unroll
-      for (int n = 0; n < N; n++) {
-        if (n + DEPTH < N) load(n + DEPTH, T[(n + DEPTH) % (DEPTH + 1)]);
-        if (n == N - 1) {
+    for (int n = 0; n < N; n++) {
+      if (n > 0 && n + NU - 1 < N) load_u(n + NU - 1, false);
+      if (n + DG < N) load_g(n + DG);
+      if (n == N - 1) {
 #pragma unroll
-          for (int k = 0; k < 3; k++) put4(dh, k, ld_G(Dp + (size_t)k * S, o));
-        }
-        FixedTerm<FMT_F32_12> &X = T[n % (DEPTH + 1)];
-        fma_row2(X.u);
-        small_row2(X.g);
-        if (!(n & 1)) acc_mul_dag(X.u, X.g, C);
-        else acc_dag_mul_dag(X.u, X.g, C);
+        for (int k = 0; k < 3; k++) put4(dh, k, ld_G(Dp + (size_t)k * S, o));
       }
+      float *const u = U[n % NU], *const g = G[n % (DG + 1)];
+      fma_row2(u);
+      small_row2(g);
+      if (!(n & 1)) acc_mul_dag(u, g, C);
+      else acc_dag_mul_dag(u, g, C);
     }
     small_row2(dh);  // D(x), high parts
     float d[18];
     {
-      AnchorK0 k0;
-      K0IO::load(a.aux, a.g.vh, p, i, k0);
+      if (NU < N) K0IO::load<false>(a.aux, a.g.vh, p, i, k0);
       AnchorK K;
       anchor_K(k0, C, dh, K);
       anchor_violation(K, acc[0], acc[1]);
@@ -520,47 +594,56 @@ __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &a, int p, int
 
 // The polish by four threads per site, as sweep_body_fixed_quad.
 template <int GAUGE, int ALGO>
-__device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &a, int p, int t, int bx) {
-  if (a.active && !a.active[t]) return;  // whole block belongs to one slice
+__device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int p, int t, int bx) {
+  if (!sweep_slice_active(in, t)) {  // whole block belongs to one slice
+    pdl_enter();
+    return;
+  }
   constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
   const int m = (int)threadIdx.x & 3;
   const int j = bx * (int)(blockDim.x >> 2) + (int)(threadIdx.x >> 2);
-  const bool valid = j < a.g.vs_half;  // the shuffles below need every lane
-  const SiteNb nb(a.g, a.inv_half1, a.inv_n2, p, t, valid ? j : 0);
-  const int i = t * a.g.vs_half + (valid ? j : 0);
+  const bool valid = j < in.g.vs_half;  // the shuffles below need every lane
+  const SiteNb nb(in.g, in.inv_half1, in.inv_n2, p, t, valid ? j : 0);
+  const int i = t * in.g.vs_half + (valid ? j : 0);
   const int q = p ^ 1;
-  const size_t S = (size_t)a.g.vh * 16;
-  const char *const L = (const char *)a.links;
-  const char *const Dq = (const char *)a.G + (size_t)(q * 3) * S;
-  char *const Dp = (char *)a.G + (size_t)(p * 3) * S;
+  const size_t S = (size_t)in.g.vh * 16;
+  const char *const L = (const char *)in.links;
+  const char *const Dq = (const char *)in.G + (size_t)(q * 3) * S;
+  char *const Dp = (char *)in.G + (size_t)(p * 3) * S;
   const unsigned o = (unsigned)i * 16u;
   float C[18], dh[18];
   mat_zero(C);
-  FixedTerm<FMT_F32_12> T[2];
+  float U[2][18], G[2][18];
+  unsigned on[2];
+  AnchorK0 k0;
+#pragma unroll
+  for (int d = 0; d < 2; d++) {  // forward, backward
+    on[d] = o + (unsigned)(nb.offset(in.g, m, d ? -1 : 1) * 16);
+    if (m >= MU0) {
+#pragma unroll
+      for (int k = 0; k < 3; k++) put4(U[d], k, ld_early(L + (size_t)(((d ? q : p) * 4 + m) * 3 + k) * S, d ? on[d] : o));
+    }
+  }
+  K0IO::load<true>(in.aux, in.g.vh, p, i, k0);
+  const SweepArgs a = sweep_start<true>(in);
   if (m >= MU0) {
 #pragma unroll
-    for (int d = 0; d < 2; d++) {  // forward, backward
-      const unsigned on = o + (unsigned)(nb.offset(a.g, m, d ? -1 : 1) * 16);
+    for (int d = 0; d < 2; d++)
 #pragma unroll
-      for (int k = 0; k < 3; k++) put4(T[d].u, k, ld_link(L + (size_t)(((d ? q : p) * 4 + m) * 3 + k) * S, d ? on : o));
-#pragma unroll
-      for (int k = 0; k < 3; k++) put4(T[d].g, k, ld_G(Dq + (size_t)k * S, on));
-    }
+      for (int k = 0; k < 3; k++) put4(G[d], k, ld_G(Dq + (size_t)k * S, on[d]));
   }
 #pragma unroll
   for (int k = 0; k < 3; k++) put4(dh, k, ld_G(Dp + (size_t)k * S, o));
   float4 lo[3];
 #pragma unroll
   for (int k = 0; k < 3; k++) lo[k] = ld_G(Dp + (6 + k) * S, o);
-  AnchorK0 k0;
-  K0IO::load(a.aux, a.g.vh, p, i, k0);
   if (m >= MU0) {
 #pragma unroll
     for (int d = 0; d < 2; d++) {
-      fma_row2(T[d].u);
-      small_row2(T[d].g);
-      if (d == 0) acc_mul_dag(T[d].u, T[d].g, C);
-      else acc_dag_mul_dag(T[d].u, T[d].g, C);
+      fma_row2(U[d]);
+      small_row2(G[d]);
+      if (d == 0) acc_mul_dag(U[d], G[d], C);
+      else acc_dag_mul_dag(U[d], G[d], C);
     }
   }
 #pragma unroll

@@ -239,7 +239,7 @@ struct SweepCfg {
 //         shared memory (24 KB), G loaded into registers beside the copies
 // The fixed-link bulk sweeps (FMT_FIX_*, lgt_fixed.cuh) are compiled for 3, 8 and
 // 9 (64 or 128 threads at <= 128 registers, 128 at <= 96) and, four threads per
-// site, 4; the anchored polish for 4 too.
+// site, 4; the anchored polish for 4 too; both for 16.
 // The one-thread and four-thread layouts form K(x) in the same order, the lean
 // ones link by link; every configuration groups the fused estimate by the same
 // 8 sites; results differ only in FP32 rounding (the order of K's sums and
@@ -247,10 +247,12 @@ struct SweepCfg {
 // kernels in configurations 0-3, 13 and 14.
 constexpr int LGT_NCFG = 16;
 // Beyond the configurations a caller may name, the autotuner has
-//    16: 32 threads, <= 255 registers, FP64 sweeps.  Those are bound by the FP64
-//        pipe of each SM, so a small lattice wants its sites spread evenly over
-//        the SMs: 12^4 has 84 blocks of 128 sites a half-sweep for 152 SMs (48 us;
-//        with 324 blocks of 32 sites the fullest SM has 96 sites).
+//    16: 32 threads, <= 255 registers, for lattices of a warp per scheduler or
+//        less.  FP64 sweeps are bound by the FP64 pipe of each SM, so such a
+//        lattice wants its sites spread evenly over the SMs: 12^4 has 84 blocks of
+//        128 sites a half-sweep for 152 SMs (48 us a half-sweep) and 324 of 32
+//        (42.5 us).  The fixed-link sweeps hold all their links in registers before
+//        the launch before has ended: 12^4 bulk Coulomb 3.9 (configuration 8) -> 3.6 us.
 constexpr int LGT_NCFG_TUNED = 17;
 __host__ __device__ constexpr int lgt_cfg_threads(int c) { return c == 16 ? 32 : (c == 2 || c == 5) ? 256 : ((c == 3 || c == 14 || c == 15) ? 64 : 128); }
 __host__ __device__ constexpr int lgt_cfg_minblocks(int c) {
@@ -272,8 +274,8 @@ __host__ __device__ constexpr int lgt_cfg_stage_chunks(int c) { return c == 15 ?
 __host__ __device__ constexpr int lgt_cfg_sites(int c) { return lgt_cfg_quad(c) ? lgt_cfg_threads(c) / 4 : lgt_cfg_threads(c); }
 // whether a storage format has kernels for a configuration
 __host__ __device__ constexpr bool lgt_cfg_supported(int fmt, int c) {
-  return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 4 || c == 8 || c == 9
-         : c == 16 ? fmt == FMT_F64
+  return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 4 || c == 8 || c == 9 || c == 16
+         : c == 16 ? fmt == FMT_F64 || fmt == FMT_ANCHOR
                                                   : c >= 0 && c < LGT_NCFG &&
          (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && (c == 4 || c == 11))) &&
          (!(lgt_cfg_pipe(c) || lgt_cfg_stream(c) || lgt_cfg_staged(c)) || fmt == FMT_F32_12);

@@ -19,8 +19,6 @@
 
 namespace lgt {
 
-
-
 // The fused estimate: the sum of (Re tr K, tr Delta^2) over each group of
 // LGT_FUSED_GROUP = 8 consecutive sites of a slice goes to the group's slot
 // (xor butterfly: fixed order; no block barrier, no atomics), and
@@ -81,6 +79,8 @@ __device__ __forceinline__ uint4 sr_draws(const SweepArgs &a, const Coords &c) {
 // which returns once that kernel has completed and its writes are visible, so
 // nothing of the field, the loop state or the estimate slots is touched before;
 // then it lets its own successor be scheduled.  Both are no-ops in a plain launch.
+// (The sweeps over links that no sweep writes read those before it: lgt_fixed.cuh,
+// sweep_slice_active.)
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1201,12 +1201,5 @@ __device__ __forceinline__ void sweep_body_pair(const SweepArgs &a, int p, int t
   fused_store<float, 1>(a, p, t, bx, acc);
 }
 
-
-template <int FMT, int GAUGE, int ALGO>
-__device__ __forceinline__ void sweep_dispatch(const SweepArgs &a, int p, int t, int bx, int nbx) {
-  if (FMT == FMT_F64) sweep_body_f64<GAUGE, ALGO>(a, p, t, bx, nbx);
-  else if (FMT == FMT_PAIR) sweep_body_pair<GAUGE, ALGO>(a, p, t, bx, nbx);
-  else sweep_body_f32<(FMT == FMT_F32_12 ? FMT_F32_12 : FMT_F32_18), GAUGE, ALGO>(a, p, t, bx, nbx);
-}
 
 }  // namespace lgt

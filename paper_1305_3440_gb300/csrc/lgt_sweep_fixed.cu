@@ -7,12 +7,10 @@ namespace lgt {
 
 template <int LFMT, int GAUGE, int ALGO, int CFG>
 __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) k_sweep_fixed(SweepArgs in, int p) {
-  pdl_enter();
-  const SweepArgs a = resolve_loop(in);
   int t, bx;
-  sweep_block_tile(a, p, t, bx);
-  if constexpr (lgt_cfg_quad(CFG)) sweep_body_fixed_quad<LFMT, GAUGE>(a, p, t, bx);
-  else sweep_body_fixed<LFMT, GAUGE, ALGO, fixed_depth(LFMT, lgt_cfg_minblocks(CFG) * lgt_cfg_threads(CFG))>(a, p, t, bx);
+  sweep_block_tile(in, p, t, bx);
+  if constexpr (lgt_cfg_quad(CFG)) sweep_body_fixed_quad<LFMT, GAUGE>(in, p, t, bx);
+  else sweep_body_fixed<LFMT, GAUGE, ALGO, fixed_depth(LFMT, lgt_cfg_minblocks(CFG) * lgt_cfg_threads(CFG))>(in, p, t, bx);
 }
 
 template <int CFG>
@@ -40,6 +38,7 @@ sweep_fn pick_sweep_fixed(int fmt, int gauge, int algo, int cfg) {
     case 4: return pick_cfg<4>(lfmt, gauge, algo);
     case 8: return pick_cfg<8>(lfmt, gauge, algo);
     case 9: return pick_cfg<9>(lfmt, gauge, algo);
+    case 16: return pick_cfg<16>(lfmt, gauge, algo);
   }
   return nullptr;
 }

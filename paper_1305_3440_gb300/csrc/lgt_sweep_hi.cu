@@ -30,12 +30,10 @@ __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) 
 
 template <int GAUGE, int ALGO, int CFG>
 __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) k_sweep_anchor(SweepArgs in, int p) {
-  pdl_enter();
-  const SweepArgs a = resolve_loop(in);
   int t, bx;
-  sweep_block_tile(a, p, t, bx);
-  if constexpr (lgt_cfg_quad(CFG)) sweep_body_anchor_quad<GAUGE, ALGO>(a, p, t, bx);
-  else sweep_body_anchor<GAUGE, ALGO, anchor_depth(CFG)>(a, p, t, bx);
+  sweep_block_tile(in, p, t, bx);
+  if constexpr (lgt_cfg_quad(CFG)) sweep_body_anchor_quad<GAUGE, ALGO>(in, p, t, bx);
+  else sweep_body_anchor<GAUGE, ALGO, anchor_depth(CFG)>(in, p, t, bx);
 }
 
 template <int CFG>
@@ -61,9 +59,8 @@ static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_f64<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_f64<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_f64<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_f64<GAUGE_COULOMB, ALGO_OR, CFG>;
   }
-  if constexpr (CFG == 16) return nullptr;
-  if (algo == ALGO_SA) return nullptr;
-  if (fmt == FMT_PAIR) {
+  if (algo == ALGO_SA || (CFG == 16 && fmt != FMT_ANCHOR)) return nullptr;
+  if constexpr (CFG != 16) if (fmt == FMT_PAIR) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_pair<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_pair<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_pair<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_pair<GAUGE_COULOMB, ALGO_OR, CFG>;
   }

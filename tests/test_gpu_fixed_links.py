@@ -121,7 +121,22 @@ for gauge in (O.LANDAU, O.COULOMB):
                 assert ratio <= 1.0, (gauge, dims, bulk, parity, ratio)
                 if parity == 0 and gauge == O.LANDAU:  # the parity-0 slots hold every link once
                     assert abs(F - O.measure(U)["F"]) < 16 * 2.0**-24
-    if cfg not in (3, 4):
+    if cfg == 16:  # FP64 sweeps: the same operations with u smaller by 2^-29
+        for dims in {dims}:
+            U = synth.field(dims, 0.5, 93)
+            for parity in (0, 1):
+                ref = U.copy()
+                O.half_sweep(ref, parity, gauge=gauge, omega=1.7)
+                bound = fp32_half_sweep_bound(O.site_conditioning(U, parity, gauge=gauge, omega=1.7), parity, 16.0) * 2.0**-29
+                ctx = lgt.lgt_create(lgt.lgt_params_default(dims=dims, bulk=lgt.LGT_FP64, gauge=gauge, omega=1.7), U)
+                lgt.lgt_half_sweep(ctx, parity)
+                out = lgt.lgt_get_links(ctx, dims)
+                st = lgt.lgt_get_stats(ctx)
+                lgt.lgt_destroy(ctx)
+                assert st.launch_config[0] == cfg, list(st.launch_config)
+                ratio, _, _ = check_fp32_bound(np.abs(out - ref), bound, 5e-6 * 2.0**-29)
+                assert ratio <= 1.0, (gauge, dims, parity, ratio)
+    if cfg not in (3, 4, 16):
         continue
     for algo in (O.OR, O.SR):  # the anchored polish
         kw = dict(gauge=gauge, algo=algo, omega=1.7, p=0.8, seed=5)
@@ -143,13 +158,13 @@ print("ok")
 """
 
 
-@pytest.mark.parametrize("cfg", [3, 4, 8, 9])
+@pytest.mark.parametrize("cfg", [3, 4, 8, 9, 16])
 def test_every_tuned_configuration(lgt, cfg, tmp_path):
-    """Each configuration the autotuner may pick for the fixed-link bulk and (3, 4)
-    the anchored polish -- one thread per site at three budgets, four threads per site
+    """Each configuration the autotuner may pick for the fixed-link bulk and (3, 4, 16)
+    the anchored polish -- one thread per site at four budgets, four threads per site
     (4) -- forced through a tuning cache file, at the edges of its blocks and quads:
     half-sweeps within the per-site FP32 bound of the oracle, the fused F, and two
-    polish sweeps within the accuracy of FP32 rotation angles."""
+    polish sweeps within the accuracy of FP32 rotation angles; 16 also for FP64."""
     import os
     import subprocess
     import sys
@@ -159,11 +174,13 @@ def test_every_tuned_configuration(lgt, cfg, tmp_path):
     name = torch.cuda.get_device_name().replace(" ", "_")
     cache = tmp_path / "tuned"
     with open(cache, "w") as f:
-        for fmt in (4, 5, 6):  # anchored polish; fixed links, 18- and 12-real
+        for fmt in (0, 4, 5, 6):  # FP64; anchored polish; fixed links, 18- and 12-real
+            if fmt == 0 and cfg != 16:
+                continue
             for gauge in (0, 1):
                 for algo in (0, 1):
                     for d in dims + [(4, 4, 4, 8)]:
-                        f.write(f"{fmt} {gauge} {algo} {d[0]} {d[1]} {d[2]} {d[3]} {name} {cfg if fmt > 4 or cfg < 5 else 0}\n")
+                        f.write(f"{fmt} {gauge} {algo} {d[0]} {d[1]} {d[2]} {d[3]} {name} {cfg if fmt > 4 or cfg in (3, 4, 16) else 0}\n")
     code = _FORCED.format(root=os.path.dirname(here), tests=here, cfg=cfg, dims=dims)
     r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, LGT_AUTOTUNE_CACHE=str(cache)),
                        capture_output=True, text=True, timeout=300)
