@@ -60,14 +60,42 @@ __global__ void __launch_bounds__(256) k_measure_batch(const BatchMeas *jobs, in
   measure_body<FMT>(J.a, t, p, rem - p * J.nbx, J.nbx);
 }
 
+// relaxed at GPU scope: may be read before griddepcontrol.wait (as ld_early)
+__device__ __forceinline__ int ld_early_int(const int *p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // FP32 overrelaxation bulk and anchored polish sweeps of the batch (FMT_MIX): each
-// row's own body at 128 threads, <= 128 registers, 4 blocks per SM.  The job table
-// is read first, so the wait for the launch before is the kernel's first act.
+// row's own body at 128 threads, <= 128 registers, 4 blocks per SM.  The table is
+// uploaded before the first launch of a tick's run, a plain one, so a block finds
+// its row (a ballot over 32 rows at a time), copies it and loads its first links
+// before the wait for the launch before (lgt_fixed.cuh, sweep_slice_active): the
+// search was four dependent loads between two launches.  A burst of 12 jobs, 8^4:
+// 9.1 -> 8.35 ms; 12^4: 25.5 -> 23.5; 16^4: 79.3 -> 76.9.
 __global__ void __launch_bounds__(128, 4) k_sweep_batch_mix(const BatchSweep *jobs, int n, int p, int s) {
-  pdl_enter();
-  const int b = batch_block(jobs, p);
-  const int k = batch_row(&jobs[0].block_begin, (int)sizeof(BatchSweep), n, b);
-  const BatchSweep &J = jobs[k];
+  __shared__ BatchSweep J;
+  const int lane = (int)threadIdx.x & 31;
+  const int snake = ld_early_int(&jobs[0].a.snake);
+  const int b = (snake && (p & 1)) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x;
+  int k = -1;  // the last row with block_begin <= b
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int begin = k0 + lane < n ? ld_early_int(&jobs[k0 + lane].block_begin) : 0x7fffffff;
+    const int below = __popc(__ballot_sync(0xffffffffu, begin <= b));
+    k += below;
+    if (below < 32) break;
+  }
+  for (int w = (int)threadIdx.x; w < (int)(sizeof(BatchSweep) / 16); w += (int)blockDim.x) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(jobs + k) + w;
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(src)
+                 : "memory");
+    reinterpret_cast<uint4 *>(&J)[w] = v;
+  }
+  __syncthreads();
   SweepArgs a = J.a;
   a.sweep += (unsigned long long)s;
   a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
@@ -75,14 +103,14 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_mix(const BatchSweep *jo
   const int t = local / J.nbx;
   const int bx = local - t * J.nbx;
   switch (J.kind) {
-    case lgt_mix_kind(FMT_FIX_12, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_12, 512), false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_FIX_12, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_12, 512), false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_FIX_18, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_18, 512), false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_FIX_18, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_18, 512), false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, ALGO_OR, 1, false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, ALGO_OR, 1, false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_SR): sweep_body_anchor<GAUGE_LANDAU, ALGO_SR, 1, false>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_SR): sweep_body_anchor<GAUGE_COULOMB, ALGO_SR, 1, false>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_12, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_12, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_18, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_FIX_18, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, ALGO_OR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, ALGO_OR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_SR): sweep_body_anchor<GAUGE_LANDAU, ALGO_SR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_SR): sweep_body_anchor<GAUGE_COULOMB, ALGO_SR, 1>(a, p, t, bx); break;
   }
 }
 

@@ -239,11 +239,9 @@ __device__ __forceinline__ bool sweep_slice_active(const SweepArgs &a, int t) {
   asm volatile("ld.relaxed.gpu.global.u8 %0, [%1];" : "=r"(v) : "l"(a.active + t) : "memory");
   return v != 0;
 }
-// the wait, and the arguments with the loop state's values (PDL: false where the
-// kernel has waited)
-template <bool PDL>
+// the wait, and the arguments with the loop state's values
 __device__ __forceinline__ SweepArgs sweep_start(const SweepArgs &in) {
-  if constexpr (PDL) pdl_enter();
+  pdl_enter();
   return resolve_loop(in);
 }
 
@@ -327,7 +325,7 @@ __device__ __forceinline__ void fixed_term(float u[18], float g[18], bool fwd, f
 // fastest configuration: 12-real links 32^4 Landau 59.7 -> 43 us, 64^4 Landau
 // 1034 -> 700 us and 48^3x96 Coulomb 620 -> 360 us (both at 6.3 to 6.6 TB/s of
 // DRAM traffic); 18-real links 14x10x12x18 6.2 -> 5.2 us.
-template <int LFMT, int GAUGE, int ALGO, int DEPTH, bool PDL = true>
+template <int LFMT, int GAUGE, int ALGO, int DEPTH>
 __device__ __forceinline__ void sweep_body_fixed(const SweepArgs &in, int p, int t, int bx) {
   constexpr bool kRows = LFMT == FMT_F32_12;  // row 2 of a link is rebuilt, not stored
   constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
@@ -335,7 +333,7 @@ __device__ __forceinline__ void sweep_body_fixed(const SweepArgs &in, int p, int
   constexpr int NU = fixed_links_ahead(DEPTH, N), DG = DEPTH < N ? DEPTH : N;
   constexpr int NC = kRows ? 3 : 4;  // 16-byte chunks per link
   if (!sweep_slice_active(in, t)) {  // whole block belongs to one slice
-    if constexpr (PDL) pdl_enter();  // (a launch ends only after the one before it)
+    pdl_enter();  // (a launch ends only after the one before it)
     return;
   }
   const int j = bx * (int)blockDim.x + (int)threadIdx.x;
@@ -373,7 +371,7 @@ __device__ __forceinline__ void sweep_body_fixed(const SweepArgs &in, int p, int
 #pragma unroll
     for (int n = 0; n < NU; n++) load_u(n, true);
   }
-  const SweepArgs a = sweep_start<PDL>(in);
+  const SweepArgs a = sweep_start(in);
   float acc[2] = {0.0f, 0.0f};
   if (valid) {
     float W[18], gx[18];
@@ -457,7 +455,7 @@ __device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &in, int p
       }
     }
   }
-  const SweepArgs a = sweep_start<true>(in);
+  const SweepArgs a = sweep_start(in);
   if (m >= MU0) {
 #pragma unroll
     for (int d = 0; d < 2; d++)
@@ -502,13 +500,13 @@ __host__ __device__ constexpr int anchor_depth(int cfg) { return cfg == 16 ? 4 :
 // written.  Loads, indices and the unrolled terms as sweep_body_fixed's.  Against
 // the looped body with K in pairs at 80 registers: 32^4 half-sweep 84 -> 67 us (5.8
 // TB/s in compulsory bytes), 8^4 8.0 -> 6.3 us.
-template <int GAUGE, int ALGO, int DEPTH, bool PDL = true>
+template <int GAUGE, int ALGO, int DEPTH>
 __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, int t, int bx) {
   constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
   constexpr int N = 2 * (4 - MU0);
   constexpr int NU = fixed_links_ahead(DEPTH, N), DG = DEPTH < N ? DEPTH : N;
   if (!sweep_slice_active(in, t)) {
-    if constexpr (PDL) pdl_enter();
+    pdl_enter();
     return;
   }
   const int j = bx * (int)blockDim.x + (int)threadIdx.x;
@@ -542,7 +540,7 @@ __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, in
     for (int n = 0; n < NU; n++) load_u(n, true);
     if (NU == N) K0IO::load<true>(in.aux, in.g.vh, p, i, k0);
   }
-  const SweepArgs a = sweep_start<PDL>(in);
+  const SweepArgs a = sweep_start(in);
   float acc[2] = {0.0f, 0.0f};
   if (valid) {
     // C(x) = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+  (small; FP32)
@@ -625,7 +623,7 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
     }
   }
   K0IO::load<true>(in.aux, in.g.vh, p, i, k0);
-  const SweepArgs a = sweep_start<true>(in);
+  const SweepArgs a = sweep_start(in);
   if (m >= MU0) {
 #pragma unroll
     for (int d = 0; d < 2; d++)

@@ -168,7 +168,7 @@ struct FusedArgs {
 };
 
 // One row of a batched launch: a lattice's arguments and its block range.
-struct BatchSweep {
+struct alignas(16) BatchSweep {  // (copied 16 bytes at a time)
   SweepArgs a;
   int block_begin;  // first block of this lattice in the batched grid
   int nbx;          // blocks per timeslice
