@@ -1,4 +1,5 @@
-// lgt_anchor.cuh -- the anchored polishing sweeps.
+// lgt_anchor.cuh -- the anchored polishing sweeps (overrelaxation; the same scheme by
+// stochastic relaxation: lgt_anchor_sr.cuh).
 //
 // After promotion the field U' (FP64) is already close to the gauge-fixed
 // field.  The anchored polish keeps U' fixed and relaxes the gauge
@@ -272,12 +273,11 @@ __device__ __forceinline__ void anchor_violation(const AnchorK &K, float &retr, 
 // |r| <~ 1e-4 of polishing (only G's unitarity depends on it, and G is
 // orthonormalised in FP64 when the field is formed).  W <- W + rho W between the
 // subgroups, as far as the later ones see it.
-template <int ALGO>
-__device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], float omega, uint64_t sr_thr, uint4 draws) {
+__device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], float omega) {
   float *W = K.W;
   // (0,1)
-  RotF r = rf[0] = subgroup_rotation<ALGO>(W[LGT_RE(0, 0)] + W[LGT_RE(1, 1)], 2.0f * K.ao[1], 2.0f * K.ao[0],
-                                           K.ad[0] - K.ad[1], omega, (uint64_t)draws.x < sr_thr);
+  RotF r = rf[0] = subgroup_rotation<ALGO_OR>(W[LGT_RE(0, 0)] + W[LGT_RE(1, 1)], 2.0f * K.ao[1], 2.0f * K.ao[0],
+                                           K.ad[0] - K.ad[1], omega, false);
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     const float xi = W[LGT_RE(0, c)], yi = W[LGT_IM(0, c)];
@@ -294,8 +294,8 @@ __device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], floa
     }
   }
   // (0,2)
-  r = rf[1] = subgroup_rotation<ALGO>(W[LGT_RE(0, 0)] + W[LGT_RE(2, 2)], 2.0f * K.ao[3], 2.0f * K.ao[2],
-                                      K.ad[0] - K.ad[2], omega, (uint64_t)draws.y < sr_thr);
+  r = rf[1] = subgroup_rotation<ALGO_OR>(W[LGT_RE(0, 0)] + W[LGT_RE(2, 2)], 2.0f * K.ao[3], 2.0f * K.ao[2],
+                                      K.ad[0] - K.ad[2], omega, false);
 #pragma unroll
   for (int c = 1; c < 3; c++) {
     const float xi = W[LGT_RE(0, c)], yi = W[LGT_IM(0, c)];
@@ -305,8 +305,8 @@ __device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], floa
     else W[LGT_RE(2, 2)] += tr, K.ad[2] += ti;
   }
   // (1,2)
-  rf[2] = subgroup_rotation<ALGO>(W[LGT_RE(1, 1)] + W[LGT_RE(2, 2)], 2.0f * K.ao[5], 2.0f * K.ao[4],
-                                  K.ad[1] - K.ad[2], omega, (uint64_t)draws.z < sr_thr);
+  rf[2] = subgroup_rotation<ALGO_OR>(W[LGT_RE(1, 1)] + W[LGT_RE(2, 2)], 2.0f * K.ao[5], 2.0f * K.ao[4],
+                                  K.ad[1] - K.ad[2], omega, false);
 }
 
 // delta = g - 1 for g = R2 R1 R0 from FP32 near-identity elements, written with

@@ -470,9 +470,11 @@ static lgt_status create_context(const lgt_params *params, const double *links, 
     c->use_loops = !(lv && lv[0] == '0');
   }
   // block sizes: given, or timed on the still-empty buffers
+  SweepCfg polish_cfg = c->cfg;
+  if (params->polish_algo == LGT_POLISH_OR) polish_cfg.algo = ALGO_OR;  // as promotion does
   const int polish_fmt = params->bulk == LGT_FP64 ? (int)FMT_F64
                          : (params->polish == LGT_POLISH_PAIR ? (int)FMT_PAIR
-                            : (params->polish == LGT_POLISH_ANCHOR ? (int)FMT_ANCHOR : (int)FMT_F64));
+                            : (params->polish == LGT_POLISH_ANCHOR ? lgt_anchor_fmt(polish_cfg.algo) : (int)FMT_F64));
   c->cfg_bulk = c->cfg_polish = lgt_cfg_of_block(params->block_size);
   if (params->launch_config > 0) {
     const int k = params->launch_config - 1;
@@ -484,8 +486,8 @@ static lgt_status create_context(const lgt_params *params, const double *links, 
       c->cfg_bulk = lgt_tune_sweep(g, c->fixed ? lgt_fixed_fmt(c->bulk_fmt) : c->bulk_fmt, c->cfg, c->u32, c->G, c->ws,
                                    c->stream, &te);
     if (te == cudaSuccess) {
-      if (polish_fmt == FMT_ANCHOR)
-        c->cfg_polish = lgt_tune_sweep(g, polish_fmt, c->cfg, c->u32, c->G, c->ws, c->stream, &te, c->k0);
+      if (polish_fmt == FMT_ANCHOR || polish_fmt == FMT_ANCHOR_SR)
+        c->cfg_polish = lgt_tune_sweep(g, polish_fmt, polish_cfg, c->u32, c->G, c->ws, c->stream, &te, c->k0);
       else
         c->cfg_polish = lgt_tune_sweep(g, polish_fmt, c->cfg, c->u64, nullptr, c->ws, c->stream, &te);
     }
@@ -563,7 +565,7 @@ static int work_fmt(const lgt_ctx *c) {
 }
 // kernel format of the current phase's sweeps
 static int sweep_fmt(const lgt_ctx *c) {
-  return c->phase == 3 ? (int)FMT_ANCHOR : (c->phase == 0 && c->fixed ? lgt_fixed_fmt(c->bulk_fmt) : work_fmt(c));
+  return c->phase == 3 ? lgt_anchor_fmt(c->cfg.algo) : (c->phase == 0 && c->fixed ? lgt_fixed_fmt(c->bulk_fmt) : work_fmt(c));
 }
 // format in which measurements and output read the working field: as stored, or
 // formed from the links and G once fixed-link sweeps have run
@@ -589,7 +591,7 @@ static lgt_status anchor_materialise(lgt_ctx *c) {
 
 static lgt_status anchor_setup(lgt_ctx *c) {
   if (c->phase != 3 || c->anchored) return LGT_OK;
-  LGT_CUDA(launch_anchor_setup(c->g, c->u64, c->u32, c->k0, c->G, c->cfg.gauge, c->stream));
+  LGT_CUDA(launch_anchor_setup(c->g, c->u64, c->u32, c->k0, c->G, c->cfg.gauge, c->cfg.algo, c->stream));
   c->stats.launches++;
   c->anchored = 1;
   c->anchor_sweeps = 0;

@@ -79,7 +79,7 @@ int lgt_tune_sweep(const Geom &g, int fmt, const SweepCfg &cfg, void *links, voi
     if (it != g_tuned.end()) return it->second;
   }
   cudaError_t e;
-  if (fmt == FMT_ANCHOR) {  // unit FP32-12 anchor, K0 = 0, D = 0
+  if (fmt == FMT_ANCHOR || fmt == FMT_ANCHOR_SR) {  // unit FP32-12 anchor, K0 = 0, D = 0
     e = launch_fill_unit(FMT_F32_12, g, links, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(aux, 0, k0_bytes(g.vh), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(G, 0, d_bytes(g.vh), st);

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lgt_anchor_sr.cuh"
 #include "lgt_fixed.cuh"
 #include "lgt_measure.cuh"
 #include "lgt_sweep.cuh"
@@ -107,10 +108,8 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_mix(const BatchSweep *jo
     case lgt_mix_kind(FMT_FIX_12, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_12, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_12, 512)>(a, p, t, bx); break;
     case lgt_mix_kind(FMT_FIX_18, GAUGE_LANDAU, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_LANDAU, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
     case lgt_mix_kind(FMT_FIX_18, GAUGE_COULOMB, ALGO_OR): sweep_body_fixed<FMT_F32_18, GAUGE_COULOMB, ALGO_OR, fixed_depth(FMT_F32_18, 512)>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, ALGO_OR, 1>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, ALGO_OR, 1>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_SR): sweep_body_anchor<GAUGE_LANDAU, ALGO_SR, 1>(a, p, t, bx); break;
-    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_SR): sweep_body_anchor<GAUGE_COULOMB, ALGO_SR, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_LANDAU, ALGO_OR): sweep_body_anchor<GAUGE_LANDAU, 1>(a, p, t, bx); break;
+    case lgt_mix_kind(FMT_ANCHOR, GAUGE_COULOMB, ALGO_OR): sweep_body_anchor<GAUGE_COULOMB, 1>(a, p, t, bx); break;
   }
 }
 
@@ -147,6 +146,21 @@ __global__ void __launch_bounds__(128, 4) k_sweep_batch_staged(const BatchSweep 
   sweep_body_f32_staged<GAUGE, ALGO>(a, p, t, local - t * J.nbx);
 }
 
+// Anchored polish sweeps by stochastic relaxation at <= 80 registers (24 warps per
+// SM), as launch configuration 11 of the single-lattice kernels: issue-bound.
+template <int GAUGE>
+__global__ void __launch_bounds__(128, 6) k_sweep_batch_anchor_sr(const BatchSweep *jobs, int n, int p, int s) {
+  const int b = batch_block(jobs, p);
+  const int k = batch_row(&jobs[0].block_begin, (int)sizeof(BatchSweep), n, b);
+  const BatchSweep &J = jobs[k];
+  SweepArgs a = J.a;
+  a.sweep += (unsigned long long)s;
+  a.reunit = a.reunit_every > 0 && ((a.count_base + s + 1) % a.reunit_every) == 0;
+  const int local = b - J.block_begin;
+  const int t = local / J.nbx;
+  anchor_sr::sweep_body_anchor_sr<GAUGE>(a, p, t, local - t * J.nbx);
+}
+
 typedef void (*batch_fn)(const BatchSweep *, int, int, int);
 
 // the staged kernel's shared memory (27 chunks of 16 B per thread), opted in once per kernel
@@ -181,6 +195,8 @@ cudaError_t launch_half_sweep_batch(int fmt, int gauge, int algo, const BatchSwe
     const cudaError_t e = staged_smem(fn, block, &smem);
     if (e != cudaSuccess) return e;
   }
+  else if (fmt == FMT_ANCHOR_SR && algo == ALGO_SR)
+    fn = gauge == GAUGE_LANDAU ? k_sweep_batch_anchor_sr<GAUGE_LANDAU> : k_sweep_batch_anchor_sr<GAUGE_COULOMB>;
   else if (fmt == FMT_PAIR) fn = pick_batch_fmt<FMT_PAIR>(gauge, algo);
   if (!fn) return cudaErrorInvalidValue;
   if (fmt != FMT_MIX || !after_sweep) {

@@ -28,6 +28,8 @@ enum { FMT_PAIR = 3 };
 // Anchored polish (lgt_anchor.cuh): not a link format but the sweep over a
 // fixed anchor field (FP32-12 copy + K0) with D = G - 1 as pairs.
 enum { FMT_ANCHOR = 4 };
+// The anchored polish by stochastic relaxation (lgt_anchor_sr.cuh; K0 as pairs).
+enum { FMT_ANCHOR_SR = 7 };
 // Fixed-link bulk sweeps (lgt_fixed.cuh): likewise sweeps, over FP32 links that
 // stay as loaded (18- or 12-real storage) with G as the only state.
 enum { FMT_FIX_18 = 5, FMT_FIX_12 = 6 };

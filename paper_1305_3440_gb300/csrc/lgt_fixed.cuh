@@ -500,7 +500,7 @@ __host__ __device__ constexpr int anchor_depth(int cfg) { return cfg == 16 ? 4 :
 // written.  Loads, indices and the unrolled terms as sweep_body_fixed's.  Against
 // the looped body with K in pairs at 80 registers: 32^4 half-sweep 84 -> 67 us (5.8
 // TB/s in compulsory bytes), 8^4 8.0 -> 6.3 us.
-template <int GAUGE, int ALGO, int DEPTH>
+template <int GAUGE, int DEPTH>
 __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, int t, int bx) {
   constexpr int MU0 = GAUGE == GAUGE_COULOMB ? 1 : 0;
   constexpr int N = 2 * (4 - MU0);
@@ -569,10 +569,8 @@ __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, in
       AnchorK K;
       anchor_K(k0, C, dh, K);
       anchor_violation(K, acc[0], acc[1]);
-      uint4 draws = make_uint4(0, 0, 0, 0);
-      if (ALGO == ALGO_SR) draws = sr_draws(a, nb.coords(t));
       RotF rf[3];
-      anchor_local_update<ALGO>(K, rf, (float)a.omega, a.sr_thr, draws);
+      anchor_local_update(K, rf, (float)a.omega);
       float_delta(rf, d);
     }
     f2 D[12];
@@ -591,7 +589,7 @@ __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, in
 }
 
 // The polish by four threads per site, as sweep_body_fixed_quad.
-template <int GAUGE, int ALGO>
+template <int GAUGE>
 __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int p, int t, int bx) {
   if (!sweep_slice_active(in, t)) {  // whole block belongs to one slice
     pdl_enter();
@@ -657,10 +655,8 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
     anchor_violation(K, vr, vd);
     if (valid && m == 0) acc[0] = vr, acc[1] = vd;
   }
-  uint4 draws = make_uint4(0, 0, 0, 0);
-  if (ALGO == ALGO_SR) draws = sr_draws(a, nb.coords(t));
   RotF rf[3];
-  anchor_local_update<ALGO>(K, rf, (float)a.omega, a.sr_thr, draws);
+  anchor_local_update(K, rf, (float)a.omega);
   float d[18];
   float_delta(rf, d);
   f2 D[12];

@@ -277,7 +277,7 @@ __host__ __device__ constexpr bool lgt_cfg_supported(int fmt, int c) {
   return (fmt == FMT_FIX_18 || fmt == FMT_FIX_12) ? c == 3 || c == 4 || c == 8 || c == 9 || c == 16
          : c == 16 ? fmt == FMT_F64 || fmt == FMT_ANCHOR
                                                   : c >= 0 && c < LGT_NCFG &&
-         (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && (c == 4 || c == 11))) &&
+         (!(lgt_cfg_quad(c) || lgt_cfg_lean(c)) || fmt == FMT_F32_18 || fmt == FMT_F32_12 || (fmt == FMT_ANCHOR && (c == 4 || c == 11)) || (fmt == FMT_ANCHOR_SR && c == 11)) &&
          (!(lgt_cfg_pipe(c) || lgt_cfg_stream(c) || lgt_cfg_staged(c)) || fmt == FMT_F32_12);
 }
 // the maximally Abelian gauge has kernels in the one-thread-per-site
@@ -442,10 +442,12 @@ cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, voi
                            int skip_temporal, void *scratch, cudaStream_t st);
 // Anchored polish set-up from the FP64 field u64: K0 (AnchorK0), the FP32-12 copy
 // in u32, D = 0.
-cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge,
+cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge, int algo,
                                 cudaStream_t st);
 // bytes of K0 (112 B per site; 144 where the bulk phase keeps the orthonormal FP64 G
 // there, see launch_apply_G) and of D (hi and lo arrays) for vh sites per parity
+// the anchored polish's sweeps: by algorithm
+constexpr int lgt_anchor_fmt(int algo) { return algo == ALGO_SR ? (int)FMT_ANCHOR_SR : (int)FMT_ANCHOR; }
 inline size_t k0_bytes(int vh) { return (size_t)vh * 2 * 144; }
 inline size_t d_bytes(int vh) { return (size_t)vh * 2 * 96; }
 cudaError_t launch_convert_pair(const Geom &g, void *u, int to_pair, cudaStream_t st);

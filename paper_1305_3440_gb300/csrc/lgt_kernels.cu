@@ -8,6 +8,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 
+#include "lgt_anchor_sr.cuh"
 #include "lgt_device.cuh"
 #include "lgt_fixed.cuh"
 #include "lgt_internal.h"
@@ -382,6 +383,7 @@ cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st) {
 // For every site of either parity: K0(x) = sum_{mu >= mu0} U_mu(x) + U_mu(x-mu)^+
 // in FP64, stored as its Hermitian and anti-Hermitian parts (AnchorK0); the FP32-12
 // copy of the site's forward links; D(x) = 0.
+template <int FMT>
 __global__ void k_anchor_setup(Geom g, const void *u64, void *u32, void *K0, void *D, int mu0) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= (long long)g.vh * 2) return;
@@ -406,16 +408,28 @@ __global__ void k_anchor_setup(Geom g, const void *u64, void *u32, void *K0, voi
   f2 z[18];
 #pragma unroll
   for (int k = 0; k < 18; k++) z[k] = {0.0f, 0.0f};
-  K0IO::store(K0, g.vh, p, i, K);
+  if constexpr (FMT == FMT_ANCHOR) {
+    K0IO::store(K0, g.vh, p, i, K);
+  } else {
+    f2 k2[18];
+#pragma unroll
+    for (int k = 0; k < 18; k++) {
+      const float hi = __double2float_rn(K[k]);
+      k2[k] = {hi, __double2float_rn(K[k] - (double)hi)};
+    }
+    anchor_sr::K0IO::store(K0, g.vh, p, i, k2);
+  }
   DIO::store_pair(D, g.vh, p, i, z);
 }
 
 cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge,
-                                cudaStream_t st) {
+                                int algo, cudaStream_t st) {
   const long long n = (long long)g.vh * 2;
   const int blk = 128;
-  k_anchor_setup<<<(unsigned)((n + blk - 1) / blk), blk, 0, st>>>(g, u64, u32, K0, D,
-                                                                 gauge == GAUGE_COULOMB ? 1 : 0);
+  const unsigned grid = (unsigned)((n + blk - 1) / blk);
+  const int mu0 = gauge == GAUGE_COULOMB ? 1 : 0;
+  if (lgt_anchor_fmt(algo) == FMT_ANCHOR) k_anchor_setup<FMT_ANCHOR><<<grid, blk, 0, st>>>(g, u64, u32, K0, D, mu0);
+  else k_anchor_setup<FMT_ANCHOR_SR><<<grid, blk, 0, st>>>(g, u64, u32, K0, D, mu0);
   return cudaGetLastError();
 }
 

@@ -93,7 +93,7 @@ struct Job {
   // the only bulk field ever measured is the loaded one, with G = 1)
   bool fixed = false;
   int sweep_fmt() const {
-    return phase == 3 ? (int)FMT_ANCHOR : (phase == 0 && fixed ? lgt_fixed_fmt(bulk_fmt) : work_fmt());
+    return phase == 3 ? lgt_anchor_fmt(cfg.algo) : (phase == 0 && fixed ? lgt_fixed_fmt(bulk_fmt) : work_fmt());
   }
   // batched launch of its sweeps: (format, gauge, algorithm)
   int batch_fmt() const { return lgt_mixes(sweep_fmt()) ? FMT_MIX : sweep_fmt(); }
@@ -240,7 +240,7 @@ cudaError_t anchor_setup(lgt_server *s, Job *j) {
   if (j->phase != 3 || j->anchored) return cudaSuccess;
   j->anchored = true;
   j->anchor_sweeps = 0;
-  return launch_anchor_setup(j->g, j->u64, j->u32, j->k0, j->G, j->cfg.gauge, s->stream);
+  return launch_anchor_setup(j->g, j->u64, j->u32, j->k0, j->G, j->cfg.gauge, j->cfg.algo, s->stream);
 }
 
 double coulomb_target(const Job *j) {

@@ -1,6 +1,7 @@
 // lgt_sweep_hi.cu -- the higher-precision half-sweep kernels: FP64 (every
 // operation in FP64), FP32-pair and anchored (the polishing sweeps), one
 // instantiation per gauge, algorithm and launch configuration.
+#include "lgt_anchor_sr.cuh"
 #include "lgt_fixed.cuh"
 #include "lgt_sweep.cuh"
 
@@ -28,21 +29,34 @@ __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) 
   sweep_body_pair<GAUGE, ALGO>(a, p, t, bx, gridDim.x);
 }
 
-template <int GAUGE, int ALGO, int CFG>
+template <int GAUGE, int CFG>
 __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) k_sweep_anchor(SweepArgs in, int p) {
   int t, bx;
   sweep_block_tile(in, p, t, bx);
-  if constexpr (lgt_cfg_quad(CFG)) sweep_body_anchor_quad<GAUGE, ALGO>(in, p, t, bx);
-  else sweep_body_anchor<GAUGE, ALGO, anchor_depth(CFG)>(in, p, t, bx);
+  if constexpr (lgt_cfg_quad(CFG)) sweep_body_anchor_quad<GAUGE>(in, p, t, bx);
+  else sweep_body_anchor<GAUGE, anchor_depth(CFG)>(in, p, t, bx);
+}
+
+template <int GAUGE, int CFG>
+__global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) k_sweep_anchor_sr(SweepArgs in, int p) {
+  pdl_enter();
+  const SweepArgs a = resolve_loop(in);
+  int t, bx;
+  sweep_block_tile(a, p, t, bx);
+  anchor_sr::sweep_body_anchor_sr<GAUGE>(a, p, t, bx);
 }
 
 template <int CFG>
 static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
-  if constexpr (CFG == 4 || CFG == 11) {  // four threads per site; 24 warps per SM at <= 80 registers: the anchored polish only
-    if (fmt != FMT_ANCHOR || algo == ALGO_SA || gauge == GAUGE_MAG) return nullptr;
-    if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_anchor<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_LANDAU, ALGO_OR, CFG>;
-    return algo == ALGO_SR ? k_sweep_anchor<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_COULOMB, ALGO_OR, CFG>;
+  if (fmt == FMT_ANCHOR || fmt == FMT_ANCHOR_SR) {
+    if (gauge == GAUGE_MAG || algo != (fmt == FMT_ANCHOR ? ALGO_OR : ALGO_SR)) return nullptr;
+    if (fmt == FMT_ANCHOR) return gauge == GAUGE_LANDAU ? k_sweep_anchor<GAUGE_LANDAU, CFG> : k_sweep_anchor<GAUGE_COULOMB, CFG>;
+    if constexpr (lgt_cfg_supported(FMT_ANCHOR_SR, CFG))
+      return gauge == GAUGE_LANDAU ? k_sweep_anchor_sr<GAUGE_LANDAU, CFG> : k_sweep_anchor_sr<GAUGE_COULOMB, CFG>;
+    return nullptr;
   }
+  // four threads per site; 24 warps per SM at <= 80 registers: the anchored polish only
+  if constexpr (CFG == 4 || CFG == 11) return nullptr;
   if (gauge == GAUGE_MAG) {  // maximally Abelian gauge: FP64 only here, configurations 0-3 and 16
     if constexpr (lgt_cfg_mag(CFG) || CFG == 16) {
       if (fmt == FMT_F64 && algo == ALGO_OR) return k_sweep_f64<GAUGE_MAG, ALGO_OR, CFG>;
@@ -59,14 +73,10 @@ static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_f64<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_f64<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_f64<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_f64<GAUGE_COULOMB, ALGO_OR, CFG>;
   }
-  if (algo == ALGO_SA || (CFG == 16 && fmt != FMT_ANCHOR)) return nullptr;
+  if (algo == ALGO_SA) return nullptr;
   if constexpr (CFG != 16) if (fmt == FMT_PAIR) {
     if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_pair<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_pair<GAUGE_LANDAU, ALGO_OR, CFG>;
     return algo == ALGO_SR ? k_sweep_pair<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_pair<GAUGE_COULOMB, ALGO_OR, CFG>;
-  }
-  if (fmt == FMT_ANCHOR) {
-    if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_anchor<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_LANDAU, ALGO_OR, CFG>;
-    return algo == ALGO_SR ? k_sweep_anchor<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_anchor<GAUGE_COULOMB, ALGO_OR, CFG>;
   }
   return nullptr;
 }

@@ -138,7 +138,7 @@ for gauge in (O.LANDAU, O.COULOMB):
                 assert ratio <= 1.0, (gauge, dims, parity, ratio)
     if cfg not in (3, 4, 16):
         continue
-    for algo in (O.OR, O.SR):  # the anchored polish
+    for algo in (O.OR, O.SR) if cfg == 3 else (O.OR,):  # the anchored polish (SR: configurations 0-3 and 11)
         kw = dict(gauge=gauge, algo=algo, omega=1.7, p=0.8, seed=5)
         ref = near.copy()
         O.sweeps(ref, 2, **kw)
@@ -174,13 +174,13 @@ def test_every_tuned_configuration(lgt, cfg, tmp_path):
     name = torch.cuda.get_device_name().replace(" ", "_")
     cache = tmp_path / "tuned"
     with open(cache, "w") as f:
-        for fmt in (0, 4, 5, 6):  # FP64; anchored polish; fixed links, 18- and 12-real
-            if fmt == 0 and cfg != 16:
+        for fmt in (0, 4, 5, 6, 7):  # FP64; anchored polish (7: SR); fixed links, 18- and 12-real
+            if (fmt == 0 and cfg != 16) or (fmt == 7 and cfg != 3):
                 continue
             for gauge in (0, 1):
                 for algo in (0, 1):
                     for d in dims + [(4, 4, 4, 8)]:
-                        f.write(f"{fmt} {gauge} {algo} {d[0]} {d[1]} {d[2]} {d[3]} {name} {cfg if fmt > 4 or cfg in (3, 4, 16) else 0}\n")
+                        f.write(f"{fmt} {gauge} {algo} {d[0]} {d[1]} {d[2]} {d[3]} {name} {cfg if fmt != 4 or cfg in (3, 4, 16) else 0}\n")
     code = _FORCED.format(root=os.path.dirname(here), tests=here, cfg=cfg, dims=dims)
     r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, LGT_AUTOTUNE_CACHE=str(cache)),
                        capture_output=True, text=True, timeout=300)
