@@ -440,7 +440,7 @@ cudaError_t launch_loop_decide(LoopState *L, const double *fused_totals, int gau
 // Anchored polish: G = 1 + D (pairs) applied in FP64 (as launch_apply_G).
 cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, void *u64_out, double *aos_out,
                            int skip_temporal, void *scratch, cudaStream_t st);
-// Anchored polish set-up from the FP64 field u64: K0 (AnchorK0), the FP32-12 copy
+// Anchored polish set-up from the FP64 field u64: K0 (AnchorK0; pairs for SR), the FP32-12 copy
 // in u32, D = 0.
 cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge, int algo,
                                 cudaStream_t st);
