@@ -462,8 +462,12 @@ __device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &in, int p
 #pragma unroll
       for (int k = 0; k < 3; k++) put4(G[d], k, ld_G(Gq + (size_t)k * S, on[d]));
   }
+  // (the lanes past the slice have site 0's indices, whose G another warp writes)
+  mat_zero(gx);
+  if (valid) {
 #pragma unroll
-  for (int k = 0; k < 3; k++) put4(gx, k, ld_G(Gp + (size_t)k * S, o));
+    for (int k = 0; k < 3; k++) put4(gx, k, ld_G(Gp + (size_t)k * S, o));
+  }
   if (m >= MU0) {
     fixed_term<LFMT>(U[0], G[0], true, M);
     fixed_term<LFMT>(U[1], G[1], false, M);
@@ -485,8 +489,9 @@ __device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &in, int p
   rows_mul(g, gx, r);
   if (a.reunit) reunitarise(r);
   else orthonormalise_rows(r);
+  __syncwarp();  // every thread of the quad has read G(x) before one of them writes it (shuffles order no memory)
 #pragma unroll
-  for (int k = 0; k < 3; k++)  // (every thread of the quad has read G(x): the shuffles are behind)
+  for (int k = 0; k < 3; k++)
     if (valid && m == k)
       *reinterpret_cast<float4 *>(Gp + (size_t)k * S + o) = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
   fused_store<float, 4>(a, p, t, bx, acc);
@@ -628,11 +633,15 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
 #pragma unroll
       for (int k = 0; k < 3; k++) put4(G[d], k, ld_G(Dq + (size_t)k * S, on[d]));
   }
+  // (the lanes past the slice: as sweep_body_fixed_quad)
+  mat_zero(dh);
+  float4 lo[3] = {};
+  if (valid) {
 #pragma unroll
-  for (int k = 0; k < 3; k++) put4(dh, k, ld_G(Dp + (size_t)k * S, o));
-  float4 lo[3];
+    for (int k = 0; k < 3; k++) put4(dh, k, ld_G(Dp + (size_t)k * S, o));
 #pragma unroll
-  for (int k = 0; k < 3; k++) lo[k] = ld_G(Dp + (6 + k) * S, o);
+    for (int k = 0; k < 3; k++) lo[k] = ld_G(Dp + (6 + k) * S, o);
+  }
   if (m >= MU0) {
 #pragma unroll
     for (int d = 0; d < 2; d++) {
@@ -668,8 +677,9 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
     D[4 * k + 3] = {dh[4 * k + 3], lo[k].w};
   }
   d_update(D, dh, d);
+  __syncwarp();  // every thread of the quad has read D(x) before one of them writes it
 #pragma unroll
-  for (int k = 0; k < 3; k++) {  // (every thread of the quad has read D(x): the shuffles are behind)
+  for (int k = 0; k < 3; k++) {
     if (valid && m == k) {
       *reinterpret_cast<float4 *>(Dp + (size_t)k * S + o) = make_float4(D[4 * k].hi, D[4 * k + 1].hi, D[4 * k + 2].hi, D[4 * k + 3].hi);
       *reinterpret_cast<float4 *>(Dp + (6 + k) * S + o) = make_float4(D[4 * k].lo, D[4 * k + 1].lo, D[4 * k + 2].lo, D[4 * k + 3].lo);
