@@ -127,6 +127,12 @@ struct SiteNb {
     if (dir > 0) return x == n - 1 ? -x * step : step;
     return x == 0 ? (n - 1) * step : -step;
   }
+  // the same in bytes of a 16-byte chunk's stream, modulo 2^32: added to a 32-bit byte
+  // offset it gives the neighbour's (the product in int would leave its range from
+  // 2^27 sites of a parity on)
+  __host__ __device__ __forceinline__ unsigned bytes(const Geom &g, int mu, int dir) const {
+    return (unsigned)offset(g, mu, dir) * 16u;
+  }
 };
 
 // ------------------------------------------------------------- link formats

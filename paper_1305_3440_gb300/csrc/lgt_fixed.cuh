@@ -348,7 +348,7 @@ __device__ __forceinline__ void sweep_body_fixed(const SweepArgs &in, int p, int
   char *const Gp = (char *)in.G + (size_t)(p * 3) * S;
   const unsigned o = (unsigned)(t * in.g.vs_half + j) * 16u;
   // term n: direction MU0 + n / 2, forward link if n is even
-  auto site = [&](int n) { return o + (unsigned)(nb.offset(in.g, MU0 + n / 2, (n & 1) ? -1 : 1) * 16); };
+  auto site = [&](int n) { return o + nb.bytes(in.g, MU0 + n / 2, (n & 1) ? -1 : 1); };
   float U[NU][18], G[DG + 1][18];
   auto load_u = [&](int n, bool early) {
     const int mu = MU0 + n / 2;
@@ -443,7 +443,7 @@ __device__ __forceinline__ void sweep_body_fixed_quad(const SweepArgs &in, int p
   unsigned on[2];
 #pragma unroll
   for (int d = 0; d < 2; d++) {  // forward, backward
-    on[d] = o + (unsigned)(nb.offset(in.g, m, d ? -1 : 1) * 16);
+    on[d] = o + nb.bytes(in.g, m, d ? -1 : 1);
     const unsigned ou = d ? on[d] : o;
     const int pu = d ? q : p;
     if (m >= MU0) {
@@ -526,7 +526,7 @@ __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, in
   char *const Dp = (char *)in.G + (size_t)(p * 3) * S;
   char *const Dl = Dp + 6 * S;  // the low parts
   const unsigned o = (unsigned)i * 16u;
-  auto site = [&](int n) { return o + (unsigned)(nb.offset(in.g, MU0 + n / 2, (n & 1) ? -1 : 1) * 16); };
+  auto site = [&](int n) { return o + nb.bytes(in.g, MU0 + n / 2, (n & 1) ? -1 : 1); };
   float U[NU][18], G[DG + 1][18];
   AnchorK0 k0;
   auto load_u = [&](int n, bool early) {
@@ -619,7 +619,7 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
   AnchorK0 k0;
 #pragma unroll
   for (int d = 0; d < 2; d++) {  // forward, backward
-    on[d] = o + (unsigned)(nb.offset(in.g, m, d ? -1 : 1) * 16);
+    on[d] = o + nb.bytes(in.g, m, d ? -1 : 1);
     if (m >= MU0) {
 #pragma unroll
       for (int k = 0; k < 3; k++) put4(U[d], k, ld_early(L + (size_t)(((d ? q : p) * 4 + m) * 3 + k) * S, d ? on[d] : o));

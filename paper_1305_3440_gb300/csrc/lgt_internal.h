@@ -331,6 +331,7 @@ sweep_fn pick_sweep_f32(int fmt, int gauge, int algo, int cfg);  // FP32-18, FP3
 sweep_fn pick_sweep_hi(int fmt, int gauge, int algo, int cfg);   // FP64, FP32-pair
 sweep_fn pick_sweep_fixed(int fmt, int gauge, int algo, int cfg);  // fixed-link FP32 bulk
 constexpr int LGT_FIXED_SA_CFG = 8;  // the fixed-link annealing sweeps' configuration
+constexpr int LGT_OFFSET32_SITES = 1 << 28;  // 16-byte chunks that 32-bit byte offsets reach
 // The bulk sweeps of a lattice keep their links fixed (FMT_FIX_*) wherever no
 // launch configuration asks for a kernel that rewrites them: overrelaxation in
 // Landau and Coulomb gauge (the maximally Abelian update is quadratic in g and
@@ -344,7 +345,7 @@ constexpr int LGT_FIXED_SA_CFG = 8;  // the fixed-link annealing sweeps' configu
 // smaller error against FP64 (5e-7 against 1.3e-5 on 64^4).
 inline bool lgt_fixed_links(int bulk_fmt, int gauge, int algo, const Geom &g) {
   return (bulk_fmt == FMT_F32_18 || bulk_fmt == FMT_F32_12) && gauge != GAUGE_MAG && algo == ALGO_OR &&
-         g.vh < (1 << 28);
+         g.vh < LGT_OFFSET32_SITES;
 }
 // The fixed-link bulk ends at this theta at the latest, theta_switch or not: the
 // FP32 rounding of G (one rotation of ~4e-8 per update, carried by all 8 links of

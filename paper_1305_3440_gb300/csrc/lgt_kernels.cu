@@ -212,6 +212,9 @@ static cudaError_t half_sweep(int fmt, const Geom &g, void *links, void *G, cons
                               cudaStream_t st, const void *aux, const LoopState *loop, int reunit_every, bool pdl) {
   sweep_fn fn = pick_sweep(fmt, c, cfg);
   if (!fn || !lgt_cfg_supported_gauge(fmt, c.gauge, cfg)) return cudaErrorInvalidValue;
+  // the anchored polish has the fixed-link sweeps' byte offsets too (a field this large
+  // exceeds the device's memory)
+  if (fmt == FMT_ANCHOR && g.vh >= LGT_OFFSET32_SITES) return cudaErrorInvalidValue;
   SweepArgs a{};
   fill_sweep_args(&a, g, links, G, w, c, sweep, reunit, use_mask);
   a.aux = aux;
