@@ -214,6 +214,10 @@ typedef struct {
  *                        14: 64 threads, <= 128 registers (8 blocks per SM);
  *                        15: 64 threads, <= 112 registers (9 blocks per SM),
  *                            the links staged and G loaded into registers.
+ * Beyond these the autotuner alone has 16: 32 threads, <= 255 registers, one
+ * thread per site, for FP64 sweeps, the anchored polish by overrelaxation and the
+ * sweeps of the next paragraph, in Landau and Coulomb gauge.  lgt_stats reports it;
+ * launch_config does not name it (17: LGT_EINVAL).
  * With neither launch_config nor block_size given, FP32 overrelaxation (bulk
  * and annealing) sweeps in Landau and Coulomb gauge (whole lattices; jobs of a
  * server always) use none of these: they keep the FP32 links as loaded and update the accumulated
@@ -341,7 +345,8 @@ typedef struct {
   double measure_ms;         /* device time of exact measurements */
   int64_t measure_launches;
   int32_t launch_config[2];  /* launch configuration of the bulk / polish sweep kernels
-                                (the table above lgt_params_default) */
+                                (the table above lgt_params_default; 16: the autotuner's
+                                own, described there) */
   int64_t loop_launches;     /* lgt_fix device loops: CUDA graph launches, each running
                                 chunks of check_every sweeps and their checks on the
                                 device until a check stops it */

@@ -286,7 +286,7 @@ __host__ __device__ constexpr bool lgt_cfg_mag(int c) { return (c >= 0 && c <= 3
 // whether a (format, gauge) pair has kernels for a configuration
 __host__ __device__ constexpr bool lgt_cfg_supported_gauge(int fmt, int gauge, int c) {
   return lgt_cfg_supported(fmt, c) &&
-         (gauge != GAUGE_MAG || ((lgt_cfg_mag(c) || c == 16) && (fmt == FMT_F64 || fmt == FMT_F32_18 || fmt == FMT_F32_12)));
+         (gauge != GAUGE_MAG || (lgt_cfg_mag(c) && (fmt == FMT_F64 || fmt == FMT_F32_18 || fmt == FMT_F32_12)));
 }
 // dynamic shared memory of the pipelined and streaming configurations: 2 buffers x 27 chunks x 16 B per thread
 constexpr int LGT_PIPE_SMEM_PER_THREAD = 2 * 27 * 16;

@@ -57,8 +57,8 @@ static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
   }
   // four threads per site; 24 warps per SM at <= 80 registers: the anchored polish only
   if constexpr (CFG == 4 || CFG == 11) return nullptr;
-  if (gauge == GAUGE_MAG) {  // maximally Abelian gauge: FP64 only here, configurations 0-3 and 16
-    if constexpr (lgt_cfg_mag(CFG) || CFG == 16) {
+  if (gauge == GAUGE_MAG) {  // maximally Abelian gauge: FP64 only here, configurations 0-3
+    if constexpr (lgt_cfg_mag(CFG)) {
       if (fmt == FMT_F64 && algo == ALGO_OR) return k_sweep_f64<GAUGE_MAG, ALGO_OR, CFG>;
       if (fmt == FMT_F64 && algo == ALGO_SR) return k_sweep_f64<GAUGE_MAG, ALGO_SR, CFG>;
     }
