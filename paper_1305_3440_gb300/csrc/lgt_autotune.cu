@@ -52,7 +52,9 @@ void load_file_locked() {
   int fmt, gauge, algo, nt, n3, n2, n1, block;
   char name[256];
   while (fscanf(f, "%d %d %d %d %d %d %d %255s %d", &fmt, &gauge, &algo, &nt, &n3, &n2, &n1, name, &block) == 9)
-    if (block >= 0 && block < LGT_NCFG_TUNED) g_tuned[TuneKey(fmt, gauge, algo, nt, n3, n2, n1, name)] = block;
+    // (a line naming a configuration without a kernel for its format and gauge, from
+    // another build or edited, is passed over: that case is timed again)
+    if (lgt_cfg_supported_gauge(fmt, gauge, block)) g_tuned[TuneKey(fmt, gauge, algo, nt, n3, n2, n1, name)] = block;
   fclose(f);
 }
 
