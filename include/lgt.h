@@ -306,8 +306,9 @@ LGT_API lgt_status lgt_estimate(lgt_ctx *ctx, double *F, double *theta, double *
  * reunitarised in FP64, applied to the retained FP64 input), then FP64
  * sweeps, checking the exact theta every check_every sweeps.  Coulomb: a
  * slice stops being updated once its theta_t is below the phase's target.
- * res (nullable) receives the outcome.  Returns LGT_OK when converged,
- * LGT_ENOTCONV after max_sweeps (state kept, may be continued). */
+ * res (nullable) receives the outcome.  Returns LGT_OK when converged (the
+ * final exact theta in res is below theta_tol), LGT_ENOTCONV after max_sweeps
+ * otherwise (state kept, may be continued). */
 LGT_API lgt_status lgt_fix(lgt_ctx *ctx, lgt_result *res);
 
 /* Leave the bulk phase now: G (reunitarised in FP64) is applied to the FP64

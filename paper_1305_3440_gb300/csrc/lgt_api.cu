@@ -1291,9 +1291,10 @@ extern "C" lgt_status lgt_fix(lgt_ctx *ctx, lgt_result *res) {
   const double tol = c->prm.theta_tol;
   bool certified = false;  // m is an exact measurement with the plaquette
   if (promoted) {
-    // the promoted field carries the rounding of the FP32 G (theta ~ 1e-8, far
-    // above any tolerance): polish first, every slice taking part until the
-    // first estimate
+    // not measured: the promoted field has the theta that the bulk left it with or,
+    // after rewritten links, what G drifted from them (~1e-8); it is polished first,
+    // every slice taking part until the first estimate.  Without sweeps left the
+    // measurement below decides.
     LGT_CUDA(cudaMemsetAsync(c->ws.active, 1, (size_t)c->g.nt, c->stream));
     c->active_slices = c->g.nt;
     m.theta = HUGE_VAL;
@@ -1332,7 +1333,7 @@ extern "C" lgt_status lgt_fix(lgt_ctx *ctx, lgt_result *res) {
     st = measure(c, 1, -1.0, &fin);
     if (st != LGT_OK) return st;
   }
-  const bool conv = m.theta < tol;
+  const bool conv = fin.theta < tol;
   if (res) {
     res->F = fin.F;
     res->theta = fin.theta;
@@ -1344,7 +1345,7 @@ extern "C" lgt_status lgt_fix(lgt_ctx *ctx, lgt_result *res) {
     res->reserved = 0;
   }
   if (!conv) {
-    lgt_set_error("not converged: theta = %.3e after %d sweeps", m.theta, c->prm.max_sweeps);
+    lgt_set_error("not converged: theta = %.3e after %d sweeps", fin.theta, c->prm.max_sweeps);
     return LGT_ENOTCONV;
   }
   return LGT_OK;

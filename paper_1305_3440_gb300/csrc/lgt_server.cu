@@ -540,8 +540,8 @@ cudaError_t promote_job(lgt_server *s, Job *j) {
     j->phase = 3;
     j->anchored = j->d_dirty = false;
   }
-  // as lgt_fix: no measurement of the promoted field (its theta is far above any
-  // tolerance); every slice takes part until the first estimate
+  // as lgt_fix: no measurement of the promoted field; every slice takes part until
+  // the first estimate
   if (e == cudaSuccess) e = cudaMemsetAsync(j->ws.active, 1, (size_t)j->g.nt, s->stream);
   j->measure_only = false;
   return e;
@@ -659,7 +659,12 @@ void worker_main(lgt_server *s) {
           fstatus.push_back(LGT_ENOTCONV);
         }
       }
-      for (size_t q = 0; q < finished.size() && e == cudaSuccess; q++) e = collect(s, finished[q]);
+      for (size_t q = 0; q < finished.size() && e == cudaSuccess; q++) {
+        e = collect(s, finished[q]);
+        // as lgt_fix: out of sweeps, the final measurement decides
+        if (e == cudaSuccess && fstatus[q] == LGT_ENOTCONV && finished[q]->res.theta < finished[q]->prm.theta_tol)
+          fstatus[q] = LGT_OK;
+      }
     }
     lk.lock();
     if (e != cudaSuccess) {
