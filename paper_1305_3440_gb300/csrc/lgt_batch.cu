@@ -199,20 +199,7 @@ cudaError_t launch_half_sweep_batch(int fmt, int gauge, int algo, const BatchSwe
     fn = gauge == GAUGE_LANDAU ? k_sweep_batch_anchor_sr<GAUGE_LANDAU> : k_sweep_batch_anchor_sr<GAUGE_COULOMB>;
   else if (fmt == FMT_PAIR) fn = pick_batch_fmt<FMT_PAIR>(gauge, algo);
   if (!fn) return cudaErrorInvalidValue;
-  if (fmt != FMT_MIX || !after_sweep) {
-    fn<<<total_blocks, block, smem, st>>>(jobs, n, parity & 1, s);
-    return cudaGetLastError();
-  }
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(total_blocks);
-  lc.blockDim = dim3(block);
-  lc.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = attr;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, fn, jobs, n, parity & 1, s);
+  return launch_sweep(fmt == FMT_MIX && after_sweep, fn, dim3(total_blocks), block, smem, st, jobs, n, parity & 1, s);
 }
 
 cudaError_t launch_measure_batch(int fmt, const BatchMeas *jobs, int n, int total_blocks, int block, cudaStream_t st) {

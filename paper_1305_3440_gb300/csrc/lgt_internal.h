@@ -327,6 +327,28 @@ inline int lgt_cfg_of_block(int block) { return block == 256 ? 2 : (block == 64 
 // fused-estimate slots: one per 8 consecutive sites of a slice
 constexpr int LGT_FUSED_GROUP = 8;
 typedef void (*sweep_fn)(SweepArgs, int);
+// Launch of a sweep kernel, single-lattice or batched.  overlap: its predecessor in
+// the stream is a sweep kernel too, so it may carry programmatic stream
+// serialisation (the kernels wait with griddepcontrol.wait); LGT_SWEEP_PDL=0 in the
+// environment: plain launches only.
+bool lgt_use_pdl();
+template <typename... P, typename... A>
+inline cudaError_t launch_sweep(bool overlap, void (*fn)(P...), dim3 grid, int block, int smem, cudaStream_t st,
+                                const A &...args) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(block);
+  lc.dynamicSmemBytes = (size_t)smem;
+  lc.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = attr;
+  lc.numAttrs = overlap && lgt_use_pdl() ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&lc, fn, P(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, not left for a later call
+  return e;
+}
 sweep_fn pick_sweep_f32(int fmt, int gauge, int algo, int cfg);  // FP32-18, FP32-12
 sweep_fn pick_sweep_hi(int fmt, int gauge, int algo, int cfg);   // FP64, FP32-pair
 sweep_fn pick_sweep_fixed(int fmt, int gauge, int algo, int cfg);  // fixed-link FP32 bulk

@@ -138,35 +138,14 @@ static int device_sms() {
 
 // Within a run of half-sweeps every launch after the first, whose predecessor in
 // the stream is then a sweep kernel, carries programmatic stream serialisation
-// (configurations with blocks per site tile; not the persistent ones)
-// (the kernels begin with griddepcontrol.wait): the next half-sweep's blocks are
-// scheduled while the previous one drains.  LGT_SWEEP_PDL=0 in the
-// environment: plain launches only.
-static bool use_pdl() {
+// (configurations with blocks per site tile; not the persistent ones): the next
+// half-sweep's blocks are scheduled while the previous one drains.
+bool lgt_use_pdl() {
   static const bool on = [] {
     const char *v = getenv("LGT_SWEEP_PDL");
     return !(v && v[0] == '0');
   }();
   return on;
-}
-
-static cudaError_t launch_fn(sweep_fn fn, dim3 grid, int block, int smem, cudaStream_t st, const SweepArgs &a,
-                             int parity, bool pdl) {
-  if (!pdl || !use_pdl()) {
-    fn<<<grid, block, smem, st>>>(a, parity);
-    return cudaGetLastError();
-  }
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = grid;
-  lc.blockDim = dim3(block);
-  lc.dynamicSmemBytes = (size_t)smem;
-  lc.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = attr;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, fn, a, parity);
 }
 
 // one launch of a sweep kernel (n_half > 1: streaming configuration only)
@@ -187,7 +166,7 @@ static cudaError_t launch_sweep_kernel(sweep_fn fn, int cfg, const Geom &g, Swee
     }
     // (persistent blocks fill the SMs' shared memory, so the successor's blocks
     // could only be placed as they exit: measured a little slower, left plain)
-    return launch_fn(fn, dim3(blocks), block, smem, st, a, parity & 1, false);
+    return launch_sweep(false, fn, dim3(blocks), block, smem, st, a, parity & 1);
   }
   int smem = 0;
   if (lgt_cfg_staged(cfg)) {  // one tile per block, its sites' operands staged in shared memory
@@ -198,7 +177,7 @@ static cudaError_t launch_sweep_kernel(sweep_fn fn, int cfg, const Geom &g, Swee
                                (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
   }
-  return launch_fn(fn, dim3(ceil_div(g.vs_half, lgt_cfg_sites(cfg)), a.t_count), block, smem, st, a, parity & 1, pdl);
+  return launch_sweep(pdl, fn, dim3(ceil_div(g.vs_half, lgt_cfg_sites(cfg)), a.t_count), block, smem, st, a, parity & 1);
 }
 
 static sweep_fn pick_sweep(int fmt, const SweepCfg &c, int cfg) {
