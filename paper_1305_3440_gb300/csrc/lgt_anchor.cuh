@@ -16,14 +16,19 @@
 //     anti-Hermitian part A0 (FP32 pairs), and the small
 //     C(x) = sum_mu U'_mu(x) D(x+mu)^+ + U'_mu(x-mu)^+ D(x-mu)^+, which FP32
 //     resolves to |D| 2^-24 from FP32 copies of U' and the high parts of D;
-//   * K = M + D(x) M with the small product in FP32;
+//   * K = M + D(x) M with the small product in FP32, its roundings kept at the size of
+//     the sum C + D M, not of the terms that cancel in it (anchor_K);
 //   * the rotation angles in FP32.  What must be resolved near the maximum is the
 //     anti-Hermitian part of K (theta and the vector part of every subgroup's
 //     quaternion are differences of its entries), so it is carried apart as the
-//     small number it is, from A0 through the subgroup steps: FP32 relative to
-//     itself, where holding all of K in pairs spent a pair addition (11
-//     operations) on each of its entries at every stage; the Hermitian part
-//     gives the quaternion's scalar part, which FP32 rounds anyway;
+//     small number it is, from A0 through the subgroup steps, its 9 reals with their
+//     roundings (two_sum), where holding all of K in pairs spent a pair addition (11
+//     operations) on each of 18 entries at every stage; the Hermitian part
+//     gives the quaternion's scalar part, which FP32 rounds anyway.  Against an
+//     all-FP64 polish of the same field the sweeps end 0.86 times as far off as with
+//     all of K in pairs (rms over 40 fields of 8^3 x 6 to 34^4, both gauges, 6 to 20
+//     sweeps; A in plain FP32 with the terms of T rounded at their own size: 1.29
+//     times) and take 67 us per 32^4 half-sweep against 83 (plain FP32: 64);
 //   * each SU(2) element in FP32 near-identity form (unit to ~|r|^2 2^-24) and
 //     delta = g - 1 in FP32 from the small quantities (error ~|delta| 2^-24);
 //   * D <- D + delta + delta D accumulated as an FP32 pair, so G stays unitary
@@ -51,18 +56,18 @@ __device__ __forceinline__ void small_row2(float d[18]) {
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     const int a = (k + 1) % 3, b = (k + 2) % 3;
-    float re = k == 0 ? -d[LGT_RE(0, 2)] : (k == 1 ? -d[LGT_RE(1, 2)] : d[LGT_RE(0, 0)] + d[LGT_RE(1, 1)]);
-    float im = k == 0 ? d[LGT_IM(0, 2)] : (k == 1 ? d[LGT_IM(1, 2)] : -d[LGT_IM(0, 0)] - d[LGT_IM(1, 1)]);
-    re = fmaf(d[LGT_RE(0, a)], d[LGT_RE(1, b)], re);
-    im = fmaf(-d[LGT_RE(0, a)], d[LGT_IM(1, b)], im);
+    const float lre = k == 0 ? -d[LGT_RE(0, 2)] : (k == 1 ? -d[LGT_RE(1, 2)] : d[LGT_RE(0, 0)] + d[LGT_RE(1, 1)]);
+    const float lim = k == 0 ? d[LGT_IM(0, 2)] : (k == 1 ? d[LGT_IM(1, 2)] : -d[LGT_IM(0, 0)] - d[LGT_IM(1, 1)]);
+    float re = d[LGT_RE(0, a)] * d[LGT_RE(1, b)];
+    float im = -d[LGT_RE(0, a)] * d[LGT_IM(1, b)];
     re = fmaf(-d[LGT_IM(0, a)], d[LGT_IM(1, b)], re);
     im = fmaf(-d[LGT_IM(0, a)], d[LGT_RE(1, b)], im);
     re = fmaf(-d[LGT_RE(0, b)], d[LGT_RE(1, a)], re);
     im = fmaf(d[LGT_RE(0, b)], d[LGT_IM(1, a)], im);
     re = fmaf(d[LGT_IM(0, b)], d[LGT_IM(1, a)], re);
     im = fmaf(d[LGT_IM(0, b)], d[LGT_RE(1, a)], im);
-    d[LGT_RE(2, k)] = re;
-    d[LGT_IM(2, k)] = im;
+    d[LGT_RE(2, k)] = lre + re;
+    d[LGT_IM(2, k)] = lim + im;
   }
 }
 
@@ -119,19 +124,22 @@ struct DIO {
 
 // K0(x) as its Hermitian part H (FP32) and its anti-Hermitian part A (FP32 pairs),
 // 28 floats in 7 float4 chunks (chunk c of parity p at (p * 7 + c) * vh + i):
-//   0: H_00 H_11 H_22 and Im A_00     1: Im A_11 Im A_22 H_01    2: H_02 H_12
+//   0: H_00 H_11 H_22 (less anchor_diag) and Im A_00     1: Im A_11 Im A_22 H_01    2: H_02 H_12
 //   3: A_01 A_02                      4: A_12, low Im A_00 Im A_11
 //   5: low Im A_22, low A_01, low Re A_02   6: low Im A_02, low A_12, tau
 // A is the traceless part: Im tr K0, which is not small, drops out of theta and of
 // every rotation; tau = Im tr K0 / 3 is kept for the products with K0.
 struct AnchorK0 {
-  float h[3];     // H_aa
+  float h[3];     // H_aa - anchor_diag
   float ho[6];    // H_01, H_02, H_12 (re, im)
   float ad[3];    // Im A_aa
   float ao[6];    // A_01, A_02, A_12 (re, im)
   float adl[3], aol[6];  // low parts
   float tau;             // Im tr K0 / 3
 };
+// H_aa is stored less this constant, near which it lies on a field near its maximum
+// (8 or 6 links of Re tr U / 3 ~ 0.8 to 0.95): 2 bits or more for its rounding.
+__host__ __device__ constexpr float anchor_diag(int gauge) { return gauge == GAUGE_COULOMB ? 5.0f : 6.5f; }
 struct K0IO {
   // EARLY: before the wait for the launch before (relaxed at GPU scope, as ld_early)
   template <bool EARLY>
@@ -156,7 +164,7 @@ struct K0IO {
     k.aol[3] = v[6].x, k.aol[4] = v[6].y, k.aol[5] = v[6].z, k.tau = v[6].w;
   }
   // from K0 in FP64
-  static __device__ __forceinline__ void store(void *base, int vh, int p, int i, const double K[18]) {
+  static __device__ __forceinline__ void store(void *base, int vh, int p, int i, const double K[18], float h0) {
     float4 *b = reinterpret_cast<float4 *>(base) + (size_t)(p * 7) * vh + i;
     float f[28];
     auto pair = [&](int hi, int lo, double v) {
@@ -167,7 +175,7 @@ struct K0IO {
     const double tau = (K[LGT_IM(0, 0)] + K[LGT_IM(1, 1)] + K[LGT_IM(2, 2)]) * (1.0 / 3.0);
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-      f[a] = __double2float_rn(K[LGT_RE(a, a)]);
+      f[a] = __double2float_rn(K[LGT_RE(a, a)] - (double)h0);
       pair(ad[a], adl[a], K[LGT_IM(a, a)] - tau);
     }
 #pragma unroll
@@ -190,14 +198,16 @@ __device__ __forceinline__ void acc_mul_dag(const float a[18], const float b[18]
   for (int i = 0; i < 3; i++)
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-      float re = c[LGT_RE(i, j)], im = c[LGT_IM(i, j)];
+      float re = 0.0f, im = 0.0f;
 #pragma unroll
       for (int k = 0; k < 3; k++) {  // a_ik conj(b_jk)
-        re += a[LGT_RE(i, k)] * b[LGT_RE(j, k)] + a[LGT_IM(i, k)] * b[LGT_IM(j, k)];
-        im += a[LGT_IM(i, k)] * b[LGT_RE(j, k)] - a[LGT_RE(i, k)] * b[LGT_IM(j, k)];
+        re = k ? fmaf(a[LGT_RE(i, k)], b[LGT_RE(j, k)], re) : a[LGT_RE(i, k)] * b[LGT_RE(j, k)];
+        im = k ? fmaf(a[LGT_IM(i, k)], b[LGT_RE(j, k)], im) : a[LGT_IM(i, k)] * b[LGT_RE(j, k)];
+        re = fmaf(a[LGT_IM(i, k)], b[LGT_IM(j, k)], re);
+        im = fmaf(-a[LGT_RE(i, k)], b[LGT_IM(j, k)], im);
       }
-      c[LGT_RE(i, j)] = re;
-      c[LGT_IM(i, j)] = im;
+      c[LGT_RE(i, j)] += re;
+      c[LGT_IM(i, j)] += im;
     }
 }
 
@@ -207,77 +217,122 @@ __device__ __forceinline__ void acc_dag_mul_dag(const float a[18], const float b
   for (int i = 0; i < 3; i++)
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-      float re = c[LGT_RE(i, j)], im = c[LGT_IM(i, j)];
+      float re = 0.0f, im = 0.0f;
 #pragma unroll
-      for (int k = 0; k < 3; k++) {  // conj(a_ki) conj(b_jk) = conj(b_jk a_ki)
-        re += b[LGT_RE(j, k)] * a[LGT_RE(k, i)] - b[LGT_IM(j, k)] * a[LGT_IM(k, i)];
-        im -= b[LGT_RE(j, k)] * a[LGT_IM(k, i)] + b[LGT_IM(j, k)] * a[LGT_RE(k, i)];
+      for (int k = 0; k < 3; k++) {  // b_jk a_ki
+        re = k ? fmaf(b[LGT_RE(j, k)], a[LGT_RE(k, i)], re) : b[LGT_RE(j, k)] * a[LGT_RE(k, i)];
+        im = k ? fmaf(b[LGT_RE(j, k)], a[LGT_IM(k, i)], im) : b[LGT_RE(j, k)] * a[LGT_IM(k, i)];
+        re = fmaf(-b[LGT_IM(j, k)], a[LGT_IM(k, i)], re);
+        im = fmaf(b[LGT_IM(j, k)], a[LGT_RE(k, i)], im);
       }
-      c[LGT_RE(i, j)] = re;
-      c[LGT_IM(i, j)] = im;
+      c[LGT_RE(i, j)] += re;
+      c[LGT_IM(i, j)] -= im;
     }
+}
+
+// x <- x + t, the rounding kept in x.lo (not renormalised: x is hi + lo)
+__device__ __forceinline__ void small_add(f2 &x, float t) {
+  const f2 s = two_sum(x.hi, t);
+  x = {s.hi, __fadd_rn(x.lo, s.lo)};
+}
+// x - y in one float
+__device__ __forceinline__ float small_diff(f2 x, f2 y) {
+  const f2 s = two_sum(x.hi, -y.hi);
+  return __fadd_rn(s.hi, __fadd_rn(s.lo, __fsub_rn(x.lo, y.lo)));
 }
 
 // K(x) = M + D M of the anchored polish, M = K0 + C: all of it as floats (W), and
 // its anti-Hermitian part apart (see above).
 struct AnchorK {
   float W[18];
-  float ad[3], ao[6];  // Im A_aa (less tau); A_01, A_02, A_12
+  float wd[3];      // Re W_aa - anchor_diag
+  f2 ad[3], ao[6];  // Im A_aa (less tau); A_01, A_02, A_12
 };
-__device__ __forceinline__ void anchor_K(const AnchorK0 &k0, const float C[18], const float dh[18], AnchorK &K) {
+// h0: anchor_diag
+__device__ __forceinline__ void anchor_K(const AnchorK0 &k0, float h0, const float C[18], const float dh[18], AnchorK &K) {
+  // K0 + X as floats: the small parts are summed first, so that each entry takes one
+  // rounding at its size
+  auto add_k0 = [&](const float X[18], float Y[18]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      Y[LGT_RE(a, a)] = h0 + (k0.h[a] + X[LGT_RE(a, a)]);
+      Y[LGT_IM(a, a)] = k0.tau + (k0.ad[a] + X[LGT_IM(a, a)]);
+    }
+#pragma unroll
+    for (int n = 0; n < 3; n++) {
+      const int a = n == 2 ? 1 : 0, c = n == 0 ? 1 : 2;
+      Y[LGT_RE(a, c)] = k0.ho[2 * n] + (k0.ao[2 * n] + X[LGT_RE(a, c)]);
+      Y[LGT_IM(a, c)] = k0.ho[2 * n + 1] + (k0.ao[2 * n + 1] + X[LGT_IM(a, c)]);
+      Y[LGT_RE(c, a)] = k0.ho[2 * n] + (X[LGT_RE(c, a)] - k0.ao[2 * n]);
+      Y[LGT_IM(c, a)] = (k0.ao[2 * n + 1] + X[LGT_IM(c, a)]) - k0.ho[2 * n + 1];
+    }
+  };
   float M[18], T[18];
+  add_k0(C, M);
+  // T = C + D M = K - K0.  The large entries of M are its diagonal's real parts, and
+  // D times them nearly cancels C where D is smooth: that product is added to C in one
+  // rounding of their sum, and the other products, small, are summed apart, with D
+  // times what the diagonal's rounding left (low).
+  float low[3];
 #pragma unroll
-  for (int a = 0; a < 3; a++) {
-    M[LGT_RE(a, a)] = k0.h[a] + C[LGT_RE(a, a)];
-    M[LGT_IM(a, a)] = (k0.ad[a] + k0.tau) + C[LGT_IM(a, a)];
-  }
+  for (int a = 0; a < 3; a++) low[a] = (k0.h[a] + C[LGT_RE(a, a)]) - (M[LGT_RE(a, a)] - h0);
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      float re = dh[LGT_RE(a, c)] * low[c], im = dh[LGT_IM(a, c)] * low[c];
+      re = fmaf(-dh[LGT_IM(a, c)], M[LGT_IM(c, c)], re);
+      im = fmaf(dh[LGT_RE(a, c)], M[LGT_IM(c, c)], im);
+#pragma unroll
+      for (int d = 1; d < 3; d++) {
+        const int k = (c + d) % 3;
+        re = fmaf(dh[LGT_RE(a, k)], M[LGT_RE(k, c)], re);
+        im = fmaf(dh[LGT_RE(a, k)], M[LGT_IM(k, c)], im);
+        re = fmaf(-dh[LGT_IM(a, k)], M[LGT_IM(k, c)], re);
+        im = fmaf(dh[LGT_IM(a, k)], M[LGT_RE(k, c)], im);
+      }
+      T[LGT_RE(a, c)] = fmaf(dh[LGT_RE(a, c)], M[LGT_RE(c, c)], C[LGT_RE(a, c)]) + re;
+      T[LGT_IM(a, c)] = fmaf(dh[LGT_IM(a, c)], M[LGT_RE(c, c)], C[LGT_IM(a, c)]) + im;
+    }
+  add_k0(T, K.W);
+#pragma unroll
+  for (int a = 0; a < 3; a++) K.wd[a] = k0.h[a] + T[LGT_RE(a, a)];
+#pragma unroll
+  for (int a = 0; a < 3; a++) K.ad[a] = {k0.ad[a], k0.adl[a]}, small_add(K.ad[a], T[LGT_IM(a, a)]);
 #pragma unroll
   for (int n = 0; n < 3; n++) {
     const int a = n == 2 ? 1 : 0, c = n == 0 ? 1 : 2;
-    M[LGT_RE(a, c)] = (k0.ho[2 * n] + k0.ao[2 * n]) + C[LGT_RE(a, c)];
-    M[LGT_IM(a, c)] = (k0.ho[2 * n + 1] + k0.ao[2 * n + 1]) + C[LGT_IM(a, c)];
-    M[LGT_RE(c, a)] = (k0.ho[2 * n] - k0.ao[2 * n]) + C[LGT_RE(c, a)];
-    M[LGT_IM(c, a)] = (k0.ao[2 * n + 1] - k0.ho[2 * n + 1]) + C[LGT_IM(c, a)];
-  }
-  mat_mul(dh, M, T);
-#pragma unroll
-  for (int e = 0; e < 18; e++) {
-    K.W[e] = M[e] + T[e];
-    T[e] += C[e];  // K = K0 + T
-  }
-#pragma unroll
-  for (int a = 0; a < 3; a++) K.ad[a] = k0.ad[a] + (k0.adl[a] + T[LGT_IM(a, a)]);
-#pragma unroll
-  for (int n = 0; n < 3; n++) {
-    const int a = n == 2 ? 1 : 0, c = n == 0 ? 1 : 2;
-    K.ao[2 * n] = k0.ao[2 * n] + fmaf(0.5f, T[LGT_RE(a, c)] - T[LGT_RE(c, a)], k0.aol[2 * n]);
-    K.ao[2 * n + 1] = k0.ao[2 * n + 1] + fmaf(0.5f, T[LGT_IM(a, c)] + T[LGT_IM(c, a)], k0.aol[2 * n + 1]);
+    K.ao[2 * n] = {k0.ao[2 * n], k0.aol[2 * n]};
+    K.ao[2 * n + 1] = {k0.ao[2 * n + 1], k0.aol[2 * n + 1]};
+    small_add(K.ao[2 * n], 0.5f * T[LGT_RE(a, c)]), small_add(K.ao[2 * n], -0.5f * T[LGT_RE(c, a)]);
+    small_add(K.ao[2 * n + 1], 0.5f * T[LGT_IM(a, c)]), small_add(K.ao[2 * n + 1], 0.5f * T[LGT_IM(c, a)]);
   }
 }
 
 // Re tr K and tr[Delta Delta^dagger], Delta the traceless part of (K - K^+)/(2i)
 __device__ __forceinline__ void anchor_violation(const AnchorK &K, float &retr, float &delta2) {
   retr = K.W[LGT_RE(0, 0)] + K.W[LGT_RE(1, 1)] + K.W[LGT_RE(2, 2)];
-  const float tr3 = (K.ad[0] + K.ad[1] + K.ad[2]) * (1.0f / 3.0f);
+  const float ad[3] = {pair_to_float(K.ad[0]), pair_to_float(K.ad[1]), pair_to_float(K.ad[2])};
+  const float tr3 = (ad[0] + ad[1] + ad[2]) * (1.0f / 3.0f);
   float s = 0.0f, t = 0.0f;
 #pragma unroll
-  for (int a = 0; a < 3; a++) s = fmaf(K.ad[a] - tr3, K.ad[a] - tr3, s);
+  for (int a = 0; a < 3; a++) s = fmaf(ad[a] - tr3, ad[a] - tr3, s);
 #pragma unroll
-  for (int e = 0; e < 6; e++) t = fmaf(K.ao[e], K.ao[e], t);
+  for (int e = 0; e < 6; e++) t = fmaf(pair_to_float(K.ao[e]), pair_to_float(K.ao[e]), t);
   delta2 = fmaf(2.0f, t, s);
 }
 
 // Sec. 3 local update for the anchored polish: the quaternions' scalar parts from
-// W, their vector parts from the anti-Hermitian part; each subgroup element in
-// FP32 near-identity form (1 + e0, r), unit to ~|r|^2 2^-24, i.e. ~1e-15 for the
-// |r| <~ 1e-4 of polishing (only G's unitarity depends on it, and G is
-// orthonormalised in FP64 when the field is formed).  W <- W + rho W between the
-// subgroups, as far as the later ones see it.
-__device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], float omega) {
+// the diagonal, in one rounding of their size, their vector parts from the
+// anti-Hermitian part; each subgroup element in FP32 near-identity form (1 + e0, r),
+// unit to ~|r|^2 2^-24, i.e. ~1e-15 for the |r| <~ 1e-4 of polishing (only G's
+// unitarity depends on it, and G is orthonormalised in FP64 when the field is
+// formed).  W <- W + rho W between the subgroups, as far as the later ones see it.
+__device__ __forceinline__ void anchor_local_update(AnchorK &K, float h0, RotF rf[3], float omega) {
   float *W = K.W;
   // (0,1)
-  RotF r = rf[0] = subgroup_rotation<ALGO_OR>(W[LGT_RE(0, 0)] + W[LGT_RE(1, 1)], 2.0f * K.ao[1], 2.0f * K.ao[0],
-                                           K.ad[0] - K.ad[1], omega, false);
+  RotF r = rf[0] = subgroup_rotation<ALGO_OR>(2.0f * h0 + (K.wd[0] + K.wd[1]), 2.0f * pair_to_float(K.ao[1]), 2.0f * pair_to_float(K.ao[0]),
+                                           small_diff(K.ad[0], K.ad[1]), omega, false);
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     const float xi = W[LGT_RE(0, c)], yi = W[LGT_IM(0, c)];
@@ -285,28 +340,28 @@ __device__ __forceinline__ void anchor_local_update(AnchorK &K, RotF rf[3], floa
     const float t0r = r.e0 * xi - r.r3 * yi + r.r2 * xj - r.r1 * yj, t0i = r.e0 * yi + r.r3 * xi + r.r2 * yj + r.r1 * xj;
     W[LGT_RE(0, c)] += t0r;
     W[LGT_IM(0, c)] += t0i;
-    if (c == 0) K.ad[0] += t0i;
-    if (c == 2) K.ao[2] = fmaf(0.5f, t0r, K.ao[2]), K.ao[3] = fmaf(0.5f, t0i, K.ao[3]);
+    if (c == 0) K.wd[0] += t0r, small_add(K.ad[0], t0i);
+    if (c == 2) small_add(K.ao[2], 0.5f * t0r), small_add(K.ao[3], 0.5f * t0i);
     if (c > 0) {
       const float t1r = -r.r2 * xi - r.r1 * yi + r.e0 * xj + r.r3 * yj, t1i = -r.r2 * yi + r.r1 * xi + r.e0 * yj - r.r3 * xj;
-      if (c == 1) W[LGT_RE(1, 1)] += t1r, K.ad[1] += t1i;
-      else K.ao[4] = fmaf(0.5f, t1r, K.ao[4]), K.ao[5] = fmaf(0.5f, t1i, K.ao[5]);
+      if (c == 1) K.wd[1] += t1r, small_add(K.ad[1], t1i);
+      else small_add(K.ao[4], 0.5f * t1r), small_add(K.ao[5], 0.5f * t1i);
     }
   }
   // (0,2)
-  r = rf[1] = subgroup_rotation<ALGO_OR>(W[LGT_RE(0, 0)] + W[LGT_RE(2, 2)], 2.0f * K.ao[3], 2.0f * K.ao[2],
-                                      K.ad[0] - K.ad[2], omega, false);
+  r = rf[1] = subgroup_rotation<ALGO_OR>(2.0f * h0 + (K.wd[0] + K.wd[2]), 2.0f * pair_to_float(K.ao[3]), 2.0f * pair_to_float(K.ao[2]),
+                                      small_diff(K.ad[0], K.ad[2]), omega, false);
 #pragma unroll
   for (int c = 1; c < 3; c++) {
     const float xi = W[LGT_RE(0, c)], yi = W[LGT_IM(0, c)];
     const float xj = W[LGT_RE(2, c)], yj = W[LGT_IM(2, c)];
     const float tr = -r.r2 * xi - r.r1 * yi + r.e0 * xj + r.r3 * yj, ti = -r.r2 * yi + r.r1 * xi + r.e0 * yj - r.r3 * xj;
-    if (c == 1) K.ao[4] = fmaf(-0.5f, tr, K.ao[4]), K.ao[5] = fmaf(0.5f, ti, K.ao[5]);  // A_12 -= conj(t_21) / 2
-    else W[LGT_RE(2, 2)] += tr, K.ad[2] += ti;
+    if (c == 1) small_add(K.ao[4], -0.5f * tr), small_add(K.ao[5], 0.5f * ti);  // A_12 -= conj(t_21) / 2
+    else K.wd[2] += tr, small_add(K.ad[2], ti);
   }
   // (1,2)
-  rf[2] = subgroup_rotation<ALGO_OR>(W[LGT_RE(1, 1)] + W[LGT_RE(2, 2)], 2.0f * K.ao[5], 2.0f * K.ao[4],
-                                  K.ad[1] - K.ad[2], omega, false);
+  rf[2] = subgroup_rotation<ALGO_OR>(2.0f * h0 + (K.wd[1] + K.wd[2]), 2.0f * pair_to_float(K.ao[5]), 2.0f * pair_to_float(K.ao[4]),
+                                  small_diff(K.ad[1], K.ad[2]), omega, false);
 }
 
 // delta = g - 1 for g = R2 R1 R0 from FP32 near-identity elements, written with

@@ -8,7 +8,7 @@
 // distance.  The body with the anti-Hermitian part apart is no further from 64 bits
 // and 20% faster, but it is not this one's result: the sweeps that users have run
 // keep theirs.  Overrelaxation contracts rounding (1e-10) and takes the faster body.
-// Issue-bound: 84 us per 32^4 half-sweep (configuration 11).
+// Issue-bound: 83 us per 32^4 half-sweep (configuration 11).
 #pragma once
 
 #include "lgt_anchor.cuh"
@@ -84,7 +84,7 @@ struct K0IO {
   }
 };
 
-// c += a b^+
+// c += a b^+, each product added as it comes (lgt_anchor.cuh forms the entry first)
 __device__ __forceinline__ void acc_mul_dag(const float a[18], const float b[18], float c[18]) {
 #pragma unroll
   for (int i = 0; i < 3; i++)

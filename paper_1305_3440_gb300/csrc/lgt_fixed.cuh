@@ -572,10 +572,10 @@ __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, in
     {
       if (NU < N) K0IO::load<false>(a.aux, a.g.vh, p, i, k0);
       AnchorK K;
-      anchor_K(k0, C, dh, K);
+      anchor_K(k0, anchor_diag(GAUGE), C, dh, K);
       anchor_violation(K, acc[0], acc[1]);
       RotF rf[3];
-      anchor_local_update(K, rf, (float)a.omega);
+      anchor_local_update(K, anchor_diag(GAUGE), rf, (float)a.omega);
       float_delta(rf, d);
     }
     f2 D[12];
@@ -657,7 +657,7 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
   for (int e = 0; e < 18; e++) C[e] += __shfl_xor_sync(0xffffffffu, C[e], 2);
   small_row2(dh);
   AnchorK K;
-  anchor_K(k0, C, dh, K);
+  anchor_K(k0, anchor_diag(GAUGE), C, dh, K);
   float acc[2] = {0.0f, 0.0f};
   {
     float vr, vd;
@@ -665,7 +665,7 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
     if (valid && m == 0) acc[0] = vr, acc[1] = vd;
   }
   RotF rf[3];
-  anchor_local_update(K, rf, (float)a.omega);
+  anchor_local_update(K, anchor_diag(GAUGE), rf, (float)a.omega);
   float d[18];
   float_delta(rf, d);
   f2 D[12];

@@ -391,7 +391,7 @@ __global__ void k_anchor_setup(Geom g, const void *u64, void *u32, void *K0, voi
 #pragma unroll
   for (int k = 0; k < 18; k++) z[k] = {0.0f, 0.0f};
   if constexpr (FMT == FMT_ANCHOR) {
-    K0IO::store(K0, g.vh, p, i, K);
+    K0IO::store(K0, g.vh, p, i, K, anchor_diag(mu0 ? GAUGE_COULOMB : GAUGE_LANDAU));
   } else {
     f2 k2[18];
 #pragma unroll
