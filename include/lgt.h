@@ -226,10 +226,14 @@ typedef struct {
  * tuned over the thread and register budgets of 3, 8 and 9 and, four threads
  * per site, 4.  The working links
  * are then G U G^+ formed in FP32 when they are asked for or measured.  FP32
- * rounding leaves such a field at theta ~ 6e-13 (rewritten links: 3e-14) but the
- * input transformed by G there too (rewritten links: 1e-8, G and the links
+ * rounding of G leaves such a field at theta ~ 6e-13 (rewritten links: 1e-14) but the
+ * input transformed by G there too (rewritten links: 1e-10 to 1e-8, G and the links
  * drifting apart), so the bulk phase of lgt_fix and of served jobs ends at theta <
- * max(theta_switch, 2e-12).
+ * max(theta_switch, 2e-12).  A driver of its own, on lgt_sweep or lgt_half_sweep,
+ * gets further: once lgt_estimate, lgt_measure or lgt_measure_slices has found theta
+ * < 1e-10, the next sweep first forms the field anew in FP64 (once per loaded field;
+ * G starts again from 1 and the sweeps end at theta ~ 1e-14, working links and
+ * transformed input alike).
  * The anchored polish (the default after promotion) runs in 0-3, in 4 (four
  * threads per site) and in 11 (<= 80 registers, 24 warps per SM).  A
  * configuration that a phase's kernel lacks (4-15 after promotion, except 4 and 11 for the anchored polish; 7, 10 and

@@ -222,6 +222,7 @@ struct lgt_ctx {
   void *G;        // accumulated transformation of the bulk phase; D = G - 1 of the anchored polish
   int fixed;      // the bulk sweeps keep the links in u32 as loaded and update G alone (lgt_fixed_links)
   int g_dirty;    // bulk sweeps have run since the load: G != 1 (fixed: the working links are G u32 G^+)
+  int rebase;     // fixed: 1 a theta under LGT_REBASE_THETA has been read, 2 the field has been formed anew since
   void *k0;       // anchored polish: K0 (AnchorK0)
   int anchored;   // anchored polish: K0, the FP32-12 copy in u32 and D refer to the field in u64
   int d_dirty;    // anchored polish: D != 0 (sweeps since the field in u64 was last formed)
@@ -384,7 +385,7 @@ static lgt_status load_field(lgt_ctx *c, const double *links, int links_on_devic
     return LGT_EINVAL;
   }
   c->phase = c->prm.bulk == LGT_FP64 ? 1 : 0;
-  c->anchored = c->d_dirty = c->g_dirty = 0;
+  c->anchored = c->d_dirty = c->g_dirty = c->rebase = 0;
   c->sa_pending = c->prm.sa_sweeps > 0;
   c->active_slices = g.nt;
   c->cfg.omega = c->prm.omega;  // omega_late may take over (omega schedule), omega_polish at promotion
@@ -641,6 +642,24 @@ static lgt_status run_halves(lgt_ctx *c, int first_parity, int n_half, int use_m
   return LGT_OK;
 }
 
+// Fixed-link bulk: a theta that the caller has read (LGT_REBASE_THETA), and the field
+// formed anew before the next sweep.  lgt_fix's own checks stay out of it: its bulk
+// ends at LGT_FIXED_FLOOR.
+static void read_theta(lgt_ctx *c, double theta) {
+  if (c->phase == 0 && c->fixed && c->g_dirty && c->rebase == 0 && theta < LGT_REBASE_THETA) c->rebase = 1;
+}
+static lgt_status rebase_due(lgt_ctx *c) {
+  if (c->phase != 0 || c->rebase != 1) return LGT_OK;
+  // (the links are spent and lend their memory to the orthonormal G)
+  LGT_CUDA(launch_apply_G(c->g, c->G, c->u64, c->u64, nullptr, skip_temporal(c), c->u32, c->stream));
+  LGT_CUDA(launch_copy_f32(c->bulk_fmt, c->g, c->u64, c->u32, c->stream));
+  LGT_CUDA(launch_g_identity(c->g, c->G, c->stream));
+  c->stats.launches += 4;
+  c->rebase = 2;
+  c->g_dirty = 0;
+  return LGT_OK;
+}
+
 static lgt_status run_sweeps(lgt_ctx *c, int n, int use_mask) { return run_halves(c, 0, 2 * n, use_mask); }
 
 extern "C" lgt_status lgt_half_sweep(lgt_ctx *ctx, int32_t parity) {
@@ -652,7 +671,8 @@ extern "C" lgt_status lgt_half_sweep(lgt_ctx *ctx, int32_t parity) {
     lgt_set_error("lgt_half_sweep: bad arguments");
     return LGT_EINVAL;
   }
-  lgt_status st = run_halves(ctx, parity, 1, 0);
+  lgt_status st = rebase_due(ctx);
+  if (st == LGT_OK) st = run_halves(ctx, parity, 1, 0);
   if (st != LGT_OK) return st;
   return sync_stream(ctx);
 }
@@ -666,7 +686,8 @@ extern "C" lgt_status lgt_sweep(lgt_ctx *ctx, int32_t n) {
     lgt_set_error("lgt_sweep: bad arguments");
     return LGT_EINVAL;
   }
-  lgt_status st = run_sweeps(ctx, n, 0);
+  lgt_status st = n > 0 ? rebase_due(ctx) : LGT_OK;
+  if (st == LGT_OK) st = run_sweeps(ctx, n, 0);
   if (st != LGT_OK) return st;
   return sync_stream(ctx);
 }
@@ -744,6 +765,7 @@ extern "C" lgt_status lgt_measure(lgt_ctx *ctx, double *F, double *theta, double
   Meas m;
   lgt_status st = measure(ctx, plaq != nullptr, -1.0, &m);
   if (st != LGT_OK) return st;
+  read_theta(ctx, m.theta);
   if (F) *F = m.F;
   if (theta) *theta = m.theta;
   if (plaq) *plaq = m.plaq;
@@ -762,6 +784,7 @@ extern "C" lgt_status lgt_measure_slices(lgt_ctx *ctx, double *F_t, double *thet
   Meas m;
   lgt_status st = measure(ctx, 0, -1.0, &m);
   if (st != LGT_OK) return st;
+  read_theta(ctx, m.theta);
   const size_t nb = sizeof(double) * (size_t)ctx->g.nt;
   if (F_t) {
     LGT_CUDA(cudaMemcpyAsync(F_t, ctx->ws.slice_F, nb, cudaMemcpyDeviceToHost, ctx->stream));
@@ -810,6 +833,7 @@ extern "C" lgt_status lgt_estimate(lgt_ctx *ctx, double *F, double *theta, doubl
   Meas m;
   lgt_status st = estimate(ctx, -1.0, &m);
   if (st != LGT_OK) return st;
+  read_theta(ctx, m.theta);
   if (F) *F = m.F;
   if (theta) *theta = m.theta;
   if (F_t || theta_t) {
@@ -1372,7 +1396,7 @@ static lgt_status to_output(lgt_ctx *c, double *out, int out_on_device, int work
   if (c->phase == 3 && c->d_dirty) {
     // through the memory of the anchor's FP32 copy, which is made anew after
     e = launch_apply_D(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->u32, c->stream);
-    if (e == cudaSuccess) e = launch_copy_f32_12(g, c->u64, c->u32, c->stream);
+    if (e == cudaSuccess) e = launch_copy_f32(FMT_F32_12, g, c->u64, c->u32, c->stream);
     c->stats.launches += 2;
   } else if (c->phase >= 1) e = launch_egress(work_fmt(c), g, c->u64, dst, c->stream);
   else if (working) e = launch_egress(read_fmt(c), g, c->u32, dst, c->stream, c->G, skip_temporal(c));

@@ -379,6 +379,12 @@ constexpr double LGT_FIXED_FLOOR = 2e-12;
 inline double lgt_bulk_target(bool fixed, double theta_switch) {
   return fixed && theta_switch < LGT_FIXED_FLOOR ? LGT_FIXED_FLOOR : theta_switch;
 }
+// A driver of its own that sweeps on with fixed links, reading theta, gets below that
+// floor all the same: once it has read a theta under this, the next sweep starts from
+// the field formed anew (u64 <- G u64 G^+ in FP64, the links from it, G = 1).  G is
+// then 1 plus entries of 1e-4 or so, whose roundings are that much smaller: theta ~
+// 1e-14, where rewritten links end too.  Once per loaded field (2 ms at 32^4).
+constexpr double LGT_REBASE_THETA = 1e-10;
 inline int lgt_fixed_fmt(int bulk_fmt) { return bulk_fmt == FMT_F32_18 ? FMT_FIX_18 : FMT_FIX_12; }
 
 // One half-sweep of parity p on a field of format fmt with launch
@@ -443,8 +449,8 @@ cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st);
 // ends: 3.5 instead of 1.6 ms at 32^4).
 cudaError_t launch_apply_G(const Geom &g, const void *G, const void *u64_in, void *u64_out, double *aos_out,
                            int skip_temporal, void *scratch, cudaStream_t st);
-// FP32-12 copy of FP64 links
-cudaError_t launch_copy_f32_12(const Geom &g, const void *u64, void *u32, cudaStream_t st);
+// copy of FP64 links in an FP32 storage format, rounded as by launch_ingest
+cudaError_t launch_copy_f32(int fmt, const Geom &g, const void *u64, void *u32, cudaStream_t st);
 
 // Temporal slabs: active[t] = (lo <= t < hi) for the nt slices.
 cudaError_t launch_slice_mask(uint8_t *active, int nt, int lo, int hi, cudaStream_t st);

@@ -399,20 +399,21 @@ cudaError_t apply_with(const Geom &g, const void *G, const void *u64_in, void *u
   return e != cudaSuccess ? e : apply<2>(g, scratch, u64_in, u64_out, aos_out, skip_temporal, st);
 }
 
-// FP32-12 copy of the FP64 links (each thread one link)
-__global__ void __launch_bounds__(256) k_copy_f32_12(Geom g, const void *u64, void *u32) {
+// FP32 copy of the FP64 links (each thread one link)
+template <int FMT>
+__global__ void __launch_bounds__(256) k_copy_f32(Geom g, const void *u64, void *u32) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= (long long)g.vh * 8) return;
   const int i = (int)(gid % g.vh), pm = (int)(gid / g.vh);
   const double2 *b = reinterpret_cast<const double2 *>(u64) + (size_t)(pm * 9) * g.vh + i;
   float r[18];
 #pragma unroll
-  for (int c = 0; c < 6; c++) {
+  for (int c = 0; c < (FMT == FMT_F32_12 ? 6 : 9); c++) {
     const double2 v = __ldg(b + (size_t)c * g.vh);
     r[2 * c] = __double2float_rn(v.x);
     r[2 * c + 1] = __double2float_rn(v.y);
   }
-  LinkIO<FMT_F32_12>::store(u32, g.vh, pm >> 2, pm & 3, i, r);
+  LinkIO<FMT>::store(u32, g.vh, pm >> 2, pm & 3, i, r);
 }
 
 }  // namespace
@@ -427,9 +428,11 @@ cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, voi
   return apply_with<1>(g, D, u64_in, u64_out, aos_out, skip_temporal, scratch, st);
 }
 
-cudaError_t launch_copy_f32_12(const Geom &g, const void *u64, void *u32, cudaStream_t st) {
-  const long long n = (long long)g.vh * 8;
-  k_copy_f32_12<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, u64, u32);
+cudaError_t launch_copy_f32(int fmt, const Geom &g, const void *u64, void *u32, cudaStream_t st) {
+  const unsigned grid = (unsigned)(((long long)g.vh * 8 + 255) / 256);
+  if (fmt == FMT_F32_12) k_copy_f32<FMT_F32_12><<<grid, 256, 0, st>>>(g, u64, u32);
+  else if (fmt == FMT_F32_18) k_copy_f32<FMT_F32_18><<<grid, 256, 0, st>>>(g, u64, u32);
+  else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
