@@ -183,21 +183,26 @@ class ClockSampler:
 
 
 def algorithmic_bytes_per_site(kind: str) -> int:
-    """Bytes one site update must move.  Bulk (the links stay as loaded): its 8 links
-    in (FP32-12 48 B, FP32-18 72 B; Coulomb gauge 6), G(x) in and out (2 rows: 48
-    B) and the other parity's G (48 B per site: each is read by 8 neighbours,
-    compulsory once).  FP32-pair and FP64 polish: 8 links of 144 B in and out.
-    Anchored polish: K0(x) (112 B) and the 8 links' FP32-12 copies (384 B) in, its
-    own D (96 B: rows 0, 1 as pairs) in and out, and the other parity's D high parts
-    (48 B per site)."""
+    """Bytes one site update must move.  Bulk by overrelaxation (the links stay as
+    loaded): its 8 links in (FP32-12 48 B, FP32-18 72 B; Coulomb gauge 6), G(x) in and
+    out (2 rows: 48 B) and the other parity's G (48 B per site: each is read by 8
+    neighbours, compulsory once).  Bulk with rewritten links (stochastic relaxation,
+    maximally Abelian gauge): 8 links and G(x) in and out.  FP32-pair and FP64 polish:
+    8 links of 144 B in and out.  Anchored polish: K0(x) (112 B; by stochastic
+    relaxation 144 B) and the 8 links' FP32-12 copies (384 B) in, its own D (96 B: rows
+    0, 1 as pairs) in and out, and the other parity's D high parts (48 B per site)."""
     if kind == "fp32_12":
         return 8 * 48 + 3 * 48
+    if kind == "fp32_12_rewritten":
+        return 16 * 48 + 2 * 48
     if kind == "fp32_12_coulomb":
         return 6 * 48 + 3 * 48
     if kind == "fp32_18":
         return 8 * 72 + 3 * 48
     if kind == "anchor":
         return 112 + 8 * 48 + 48 + 2 * 96
+    if kind == "anchor_sr":
+        return 144 + 8 * 48 + 48 + 2 * 96
     if kind == "anchor_coulomb":  # spatial directions only
         return 112 + 6 * 48 + 48 + 2 * 96
     return 16 * 144
@@ -556,6 +561,13 @@ def _timed_fix(lgt, ctx, src, stream):
     return e0.elapsed_time(e1) / 1e3, st, res, lgt.lgt_get_stats(ctx)
 
 
+def ladder_kinds(algo: str, polish_algo: str = "same"):
+    """The kernels of a Landau-gauge FP32-12 job's bulk and polish sweeps, as
+    algorithmic_bytes_per_site names them."""
+    return ("fp32_12" if algo == "or" else "fp32_12_rewritten",
+            "anchor" if algo == "or" or polish_algo == "or" else "anchor_sr")
+
+
 def _kernel_summary(stats, bytes_bulk, bytes_polish, vol):
     """Per sweep kernel: mean launch time and achieved GB/s from the site updates it
     actually did (converged Coulomb slices are skipped)."""
@@ -621,15 +633,17 @@ def run_landau64(args):
     dev = torch.from_numpy(U).cuda()
     stream = torch.cuda.Stream()
     out = {}
-    for name, kw in [("or_1.8", dict(algo=lgt.LGT_OR, omega=1.8)), ("sr_0.9", dict(algo=lgt.LGT_SR, p=0.9, seed=5)),
-                     ("sr_0.9_or_polish", dict(algo=lgt.LGT_SR, p=0.9, seed=5, polish_algo=lgt.LGT_POLISH_OR))]:
+    for name, kinds, kw in [("or_1.8", ladder_kinds("or"), dict(algo=lgt.LGT_OR, omega=1.8)),
+                            ("sr_0.9", ladder_kinds("sr"), dict(algo=lgt.LGT_SR, p=0.9, seed=5)),
+                            ("sr_0.9_or_polish", ladder_kinds("sr", "or"),
+                             dict(algo=lgt.LGT_SR, p=0.9, seed=5, polish_algo=lgt.LGT_POLISH_OR))]:
         p = lgt.lgt_params_default(dims=dims, bulk=lgt.LGT_FP32_12, max_sweeps=100000, **kw)
         ctx = lgt.lgt_create(p, dev, stream=stream)
         t, st, res, stats = _timed_fix(lgt, ctx, dev, stream)
         lgt.lgt_destroy(ctx)
         out[name] = {"status": st, "seconds": t, "sweeps_bulk": res.sweeps_bulk, "sweeps_polish": res.sweeps_fp64,
                      "F": res.F, "theta": res.theta, "site_updates_per_s": (res.sweeps_bulk + res.sweeps_fp64) * vol / t,
-                     "kernels": _kernel_summary(stats, algorithmic_bytes_per_site("fp32_12"), algorithmic_bytes_per_site("anchor"), vol)}
+                     "kernels": _kernel_summary(stats, *map(algorithmic_bytes_per_site, kinds), vol)}
     p = lgt.lgt_params_default(dims=dims, bulk=lgt.LGT_FP64, omega=1.8)
     ctx = lgt.lgt_create(p, dev, stream=stream)
     lgt.lgt_sweep(ctx, 2)
@@ -677,7 +691,7 @@ def run_mag(args):
     dims = (32, 32, 32, 32)
     vol = int(np.prod(dims))
     dev = torch.from_numpy(synth.field(dims, 0.5, 2)).cuda()
-    for name, bulk, bytes_per_site in [("bulk_fp32_12", lgt.LGT_FP32_12, 16 * 48 + 2 * 48),
+    for name, bulk, bytes_per_site in [("bulk_fp32_12", lgt.LGT_FP32_12, algorithmic_bytes_per_site("fp32_12_rewritten")),
                                        ("fp64", lgt.LGT_FP64, 2304)]:
         p = lgt.lgt_params_default(dims=dims, gauge=lgt.LGT_MAG, bulk=bulk, omega=1.7)
         ctx = lgt.lgt_create(p, dev, stream=stream)
