@@ -46,17 +46,9 @@ __global__ void __launch_bounds__(lgt_cfg_threads(CFG), lgt_cfg_minblocks(CFG)) 
   anchor_sr::sweep_body_anchor_sr<GAUGE>(a, p, t, bx);
 }
 
+// FP64 and FP32-pair sweeps
 template <int CFG>
-static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
-  if (fmt == FMT_ANCHOR || fmt == FMT_ANCHOR_SR) {
-    if (gauge == GAUGE_MAG || algo != (fmt == FMT_ANCHOR ? ALGO_OR : ALGO_SR)) return nullptr;
-    if (fmt == FMT_ANCHOR) return gauge == GAUGE_LANDAU ? k_sweep_anchor<GAUGE_LANDAU, CFG> : k_sweep_anchor<GAUGE_COULOMB, CFG>;
-    if constexpr (lgt_cfg_supported(FMT_ANCHOR_SR, CFG))
-      return gauge == GAUGE_LANDAU ? k_sweep_anchor_sr<GAUGE_LANDAU, CFG> : k_sweep_anchor_sr<GAUGE_COULOMB, CFG>;
-    return nullptr;
-  }
-  // four threads per site; 24 warps per SM at <= 80 registers: the anchored polish only
-  if constexpr (CFG == 4 || CFG == 11) return nullptr;
+static sweep_fn pick_links(int fmt, int gauge, int algo) {
   if (gauge == GAUGE_MAG) {  // maximally Abelian gauge: FP64 only here, configurations 0-3
     if constexpr (lgt_cfg_mag(CFG)) {
       if (fmt == FMT_F64 && algo == ALGO_OR) return k_sweep_f64<GAUGE_MAG, ALGO_OR, CFG>;
@@ -74,11 +66,27 @@ static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
     return algo == ALGO_SR ? k_sweep_f64<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_f64<GAUGE_COULOMB, ALGO_OR, CFG>;
   }
   if (algo == ALGO_SA) return nullptr;
-  if constexpr (CFG != 16) if (fmt == FMT_PAIR) {
-    if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_pair<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_pair<GAUGE_LANDAU, ALGO_OR, CFG>;
-    return algo == ALGO_SR ? k_sweep_pair<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_pair<GAUGE_COULOMB, ALGO_OR, CFG>;
+  if constexpr (lgt_cfg_supported(FMT_PAIR, CFG)) {
+    if (fmt == FMT_PAIR) {
+      if (gauge == GAUGE_LANDAU) return algo == ALGO_SR ? k_sweep_pair<GAUGE_LANDAU, ALGO_SR, CFG> : k_sweep_pair<GAUGE_LANDAU, ALGO_OR, CFG>;
+      return algo == ALGO_SR ? k_sweep_pair<GAUGE_COULOMB, ALGO_SR, CFG> : k_sweep_pair<GAUGE_COULOMB, ALGO_OR, CFG>;
+    }
   }
   return nullptr;
+}
+
+template <int CFG>
+static sweep_fn pick_cfg(int fmt, int gauge, int algo) {
+  if (fmt == FMT_ANCHOR || fmt == FMT_ANCHOR_SR) {
+    if (gauge == GAUGE_MAG || algo != (fmt == FMT_ANCHOR ? ALGO_OR : ALGO_SR)) return nullptr;
+    if (fmt == FMT_ANCHOR) return gauge == GAUGE_LANDAU ? k_sweep_anchor<GAUGE_LANDAU, CFG> : k_sweep_anchor<GAUGE_COULOMB, CFG>;
+    if constexpr (lgt_cfg_supported(FMT_ANCHOR_SR, CFG))
+      return gauge == GAUGE_LANDAU ? k_sweep_anchor_sr<GAUGE_LANDAU, CFG> : k_sweep_anchor_sr<GAUGE_COULOMB, CFG>;
+    return nullptr;
+  }
+  // (4, four threads per site, and 11, 24 warps per SM at <= 80 registers: the anchored polish only)
+  if constexpr (lgt_cfg_supported(FMT_F64, CFG)) return pick_links<CFG>(fmt, gauge, algo);
+  else return nullptr;
 }
 
 sweep_fn pick_sweep_hi(int fmt, int gauge, int algo, int cfg) {

@@ -16,3 +16,13 @@ def test_supported_configurations_are_the_documented_ones(tmp_path):
                            os.path.join(ROOT, "tests", "launch_table_check.cu"), "-o", str(exe)])
     out = subprocess.run([str(exe)], capture_output=True, text=True)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
+
+
+def test_no_sweep_kernel_is_compiled_that_no_dispatch_reaches():
+    """FP64 and FP32-pair sweep kernels exist in their configurations and in no other
+    (an early return under `if constexpr` discards nothing after it)."""
+    import re
+    from paper_1305_3440_gb300 import build
+    names = subprocess.run(["nm", "-C", build.build()], capture_output=True, text=True, check=True).stdout
+    for kernel, want in (("k_sweep_f64", {0, 1, 2, 3, 16}), ("k_sweep_pair", {0, 1, 2, 3})):
+        assert {int(c) for c in re.findall(kernel + r"<\d+, \d+, (\d+)>", names)} == want, kernel
