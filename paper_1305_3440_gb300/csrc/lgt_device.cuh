@@ -67,8 +67,8 @@ __host__ __device__ __forceinline__ int cb_index(const Geom &g, int x1, int x2, 
   return ((t * g.n3 + x3) * g.n2 + x2) * g.half1 + (x1 >> 1);
 }
 
-// within-parity index of x + dir * mu-hat (dir = +-1)
-__host__ __device__ __forceinline__ int cb_shift(const Geom &g, const Coords &c, int mu, int dir) {
+// x + dir * mu-hat (dir = +-1), and its within-parity index
+__host__ __device__ __forceinline__ Coords coords_shift(const Geom &g, const Coords &c, int mu, int dir) {
   int x1 = c.x1, x2 = c.x2, x3 = c.x3, t = c.t;
   if (mu == 0) {
     t += dir;
@@ -83,7 +83,11 @@ __host__ __device__ __forceinline__ int cb_shift(const Geom &g, const Coords &c,
     x3 += dir;
     x3 = x3 < 0 ? x3 + g.n3 : (x3 >= g.n3 ? x3 - g.n3 : x3);
   }
-  return cb_index(g, x1, x2, x3, t);
+  return Coords{x1, x2, x3, t};
+}
+__host__ __device__ __forceinline__ int cb_index(const Geom &g, const Coords &c) { return cb_index(g, c.x1, c.x2, c.x3, c.t); }
+__host__ __device__ __forceinline__ int cb_shift(const Geom &g, const Coords &c, int mu, int dir) {
+  return cb_index(g, coords_shift(g, c, mu, dir));
 }
 
 // Index arithmetic without integer division, for the kernels that count

@@ -692,27 +692,40 @@ __device__ __forceinline__ void sweep_body_anchor_quad(const SweepArgs &in, int 
 // The bulk's working link U_mu(x) -> G(x) U_mu(x) G(x+mu)^+ in FP32 (12-real
 // storage: rows 0, 1 formed and row 2 rebuilt, as a stored working link; 18-real:
 // all three rows), for measurements and output between sweeps.
+// G(x) with its row 2
+__device__ __forceinline__ void load_G_full(const void *G, int vh, int p, int i, float g[18]) {
+  load_G_rows(G, vh, p, i, g);
+  fma_row2(g);
+}
+// w: the stored link in, the working link out; gx, gy: G at its two ends
 template <int LFMT>
-__device__ __forceinline__ void load_working(const Geom &g, const void *links, const void *G, int skip_temporal, int p,
-                                             int mu, int i, float w[18]) {
-  LinkIO<LFMT>::load_raw(links, g.vh, p, mu, i, w);
-  if (LFMT == FMT_F32_12) fma_row2(w);
-  if (skip_temporal && mu == 0) return;
-  const int t = i / g.vs_half;
-  const Coords c = coords_in_slice(g, p, t, i - t * g.vs_half);
-  float gx[18], gy[18], r[18];
-  load_G_rows(G, g.vh, p, i, gx);
-  load_G_rows(G, g.vh, p ^ 1, cb_shift(g, c, mu, +1), gy);
-  fma_row2(gy);
+__device__ __forceinline__ void form_working(const float gx[18], const float gy[18], float w[18]) {
+  float r[18];
   if (LFMT == FMT_F32_12) {
     rows_mul(gx, w, r);
     rows_mul_dag(r, gy, w);
     fma_row2(w);
   } else {
-    fma_row2(gx);
     mat_mul(gx, w, r);
     mat_mul_dag(r, gy, w);
   }
+}
+template <int LFMT>
+__device__ __forceinline__ void load_stored(const void *links, int vh, int p, int mu, int i, float w[18]) {
+  LinkIO<LFMT>::load_raw(links, vh, p, mu, i, w);
+  if (LFMT == FMT_F32_12) fma_row2(w);
+}
+template <int LFMT>
+__device__ __forceinline__ void load_working(const Geom &g, const void *links, const void *G, int skip_temporal, int p,
+                                             int mu, int i, float w[18]) {
+  load_stored<LFMT>(links, g.vh, p, mu, i, w);
+  if (skip_temporal && mu == 0) return;
+  const int t = i / g.vs_half;
+  const Coords c = coords_in_slice(g, p, t, i - t * g.vs_half);
+  float gx[18], gy[18];
+  load_G_full(G, g.vh, p, i, gx);
+  load_G_full(G, g.vh, p ^ 1, cb_shift(g, c, mu, +1), gy);
+  form_working<LFMT>(gx, gy, w);
 }
 
 }  // namespace lgt

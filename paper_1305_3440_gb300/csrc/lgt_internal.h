@@ -151,6 +151,7 @@ struct MeasArgs {
   int mag;  // maximally Abelian gauge: slot 0 sums |U_aa|^2, slot 2 tr Delta_MAG^2
   const void *G;      // FMT_FIX_*: the links are formed as G U G^+
   int skip_temporal;  // FMT_FIX_*: except the temporal ones
+  int split;          // FMT_FIX_*: two threads per site
 };
 
 // Arguments of the fused estimate's finishing reduction (one block per slice).

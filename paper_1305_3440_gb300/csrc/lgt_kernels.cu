@@ -320,7 +320,7 @@ void fill_meas_args(MeasArgs *a, const Geom &g, const void *links, const Workspa
   a->coulomb_target = coulomb_target;
   a->with_plaq = with_plaq;
   a->G = nullptr;
-  a->skip_temporal = 0;
+  a->skip_temporal = a->split = 0;
   a->mag = 0;  // the maximally Abelian gauge's measurement is asked for explicitly (launch_measure)
 }
 
@@ -333,6 +333,16 @@ cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Work
   a.G = G;
   a.skip_temporal = skip_temporal;
   dim3 grid(ceil_div(g.vs_half, block), g.nt, 2);
+  // A link formed from U and G where it is read adds two G and two products to its
+  // chain.  The FP64 pipe hides that where warps are many; on a lattice whose blocks
+  // leave SMs idle, two threads take a site's plaquettes instead (64 sites per block:
+  // what the workspace holds partial sums for).  8^4 with plaquette: 108 -> 67 us (98
+  // by one thread per site, stored links 94); 10^4, where the blocks of 64 just fill the
+  // SMs: 109 -> 97 (101, 95).
+  if ((fmt == FMT_FIX_18 || fmt == FMT_FIX_12) && with_plaq && block == 128 && (int)(grid.x * grid.y * 2) < device_sms()) {
+    a.split = 1;
+    grid.x = ceil_div(g.vs_half, 64);
+  }
   if (fmt == FMT_F64) k_measure<FMT_F64><<<grid, block, 0, st>>>(a);
   else if (fmt == FMT_F32_18) k_measure<FMT_F32_18><<<grid, block, 0, st>>>(a);
   else if (fmt == FMT_F32_12) k_measure<FMT_F32_12><<<grid, block, 0, st>>>(a);
