@@ -503,7 +503,7 @@ __host__ __device__ constexpr int anchor_depth(int cfg) { return cfg == 16 ? 4 :
 // Anchored polishing sweep (lgt_anchor.cuh): a.links = FP32-12 copy of the anchor
 // field U', a.G = D = G - 1 (pairs), a.aux = K0.  One thread per site; only D(x) is
 // written.  Loads, indices and the unrolled terms as sweep_body_fixed's.  Against
-// the looped body with K in pairs at 80 registers: 32^4 half-sweep 84 -> 67 us (5.8
+// the looped body with K in pairs at 80 registers: 32^4 half-sweep 83 -> 67 us (5.8
 // TB/s in compulsory bytes), 8^4 8.0 -> 6.3 us.
 template <int GAUGE, int DEPTH>
 __device__ __forceinline__ void sweep_body_anchor(const SweepArgs &in, int p, int t, int bx) {

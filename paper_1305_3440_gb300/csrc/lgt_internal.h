@@ -363,9 +363,9 @@ constexpr int LGT_OFFSET32_SITES = 1 << 28;  // 16-byte chunks that 32-bit byte 
 // parity; the FP64 field of a larger lattice would not fit the device anyway).
 // Stochastic relaxation keeps rewriting its links: its squared steps are nearly
 // microcanonical, so the norm drift of rewritten links (1.3e-5 in 40 sweeps) stays
-// in the trajectory and theta of the two differs by up to 1e-4 there, more than a
-// change of kernel may (overrelaxation: 2e-5), although the fixed links have the
-// smaller error against FP64 (5e-7 against 1.3e-5 on 64^4).
+// in the trajectory, and with fixed links theta of the same job would differ by up
+// to 1e-4 from what these sweeps give (overrelaxation: 2e-5), although the fixed
+// links have the smaller error against FP64 (5e-7 against 1.3e-5 on 64^4).
 inline bool lgt_fixed_links(int bulk_fmt, int gauge, int algo, const Geom &g) {
   return (bulk_fmt == FMT_F32_18 || bulk_fmt == FMT_F32_12) && gauge != GAUGE_MAG && algo == ALGO_OR &&
          g.vh < LGT_OFFSET32_SITES;
@@ -474,10 +474,11 @@ cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, voi
 // in u32, D = 0.
 cudaError_t launch_anchor_setup(const Geom &g, const void *u64, void *u32, void *K0, void *D, int gauge, int algo,
                                 cudaStream_t st);
-// bytes of K0 (112 B per site; 144 where the bulk phase keeps the orthonormal FP64 G
-// there, see launch_apply_G) and of D (hi and lo arrays) for vh sites per parity
-// the anchored polish's sweeps: by algorithm
+// sweep format of the anchored polish: by algorithm
 constexpr int lgt_anchor_fmt(int algo) { return algo == ALGO_SR ? (int)FMT_ANCHOR_SR : (int)FMT_ANCHOR; }
+// bytes of K0's memory (144 B per site: K0 in pairs, or the orthonormal FP64 G that the
+// bulk phase keeps there, see launch_apply_G; AnchorK0 fills 112 of them) and of D (hi
+// and lo arrays) for vh sites per parity
 inline size_t k0_bytes(int vh) { return (size_t)vh * 2 * 144; }
 inline size_t d_bytes(int vh) { return (size_t)vh * 2 * 96; }
 cudaError_t launch_convert_pair(const Geom &g, void *u, int to_pair, cudaStream_t st);
