@@ -1395,9 +1395,10 @@ static lgt_status to_output(lgt_ctx *c, double *out, int out_on_device, int work
   cudaError_t e;
   if (c->phase == 3 && c->d_dirty) {
     // through the memory of the anchor's FP32 copy, which is made anew after
-    e = launch_apply_D(g, c->G, c->u64, nullptr, dst, skip_temporal(c), c->u32, c->stream);
-    if (e == cudaSuccess) e = launch_copy_f32(FMT_F32_12, g, c->u64, c->u32, c->stream);
-    c->stats.launches += 2;
+    void *const scratch = lgt_gauge_in_one_launch(g) ? nullptr : c->u32;
+    e = launch_apply_D(g, c->G, c->u64, nullptr, dst, skip_temporal(c), scratch, c->stream);
+    if (e == cudaSuccess && scratch) e = launch_copy_f32(FMT_F32_12, g, c->u64, c->u32, c->stream);
+    c->stats.launches += scratch ? 2 : 0;
   } else if (c->phase >= 1) e = launch_egress(work_fmt(c), g, c->u64, dst, c->stream);
   else if (working) e = launch_egress(read_fmt(c), g, c->u32, dst, c->stream, c->G, skip_temporal(c));
   else if (!c->g_dirty) e = launch_egress(FMT_F64, g, c->u64, dst, c->stream);  // G = 1

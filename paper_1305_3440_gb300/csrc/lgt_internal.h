@@ -450,6 +450,11 @@ cudaError_t launch_g_identity(const Geom &g, void *G, cudaStream_t st);
 // ends: 3.5 instead of 1.6 ms at 32^4).
 cudaError_t launch_apply_G(const Geom &g, const void *G, const void *u64_in, void *u64_out, double *aos_out,
                            int skip_temporal, void *scratch, cudaStream_t st);
+// whether scratch is better left out (one launch at one warp per scheduler), where
+// what the scratch held has to be made again
+bool lgt_gauge_in_one_launch(const Geom &g);
+// SMs of the current device
+int lgt_device_sms();
 // copy of FP64 links in an FP32 storage format, rounded as by launch_ingest
 cudaError_t launch_copy_f32(int fmt, const Geom &g, const void *u64, void *u32, cudaStream_t st);
 

@@ -38,12 +38,13 @@ unsigned tile_blocks(const Geom &g) { return (unsigned)((g.vh + kPairs - 1) / kP
 struct TileLink {
   int p, mu, i, pair, odd;
   bool valid;
-  __device__ __forceinline__ explicit TileLink(const Geom &g) {
-    const int w = (int)threadIdx.x >> 5;
+  __device__ __forceinline__ explicit TileLink(const Geom &g) : TileLink(g, (int)threadIdx.x >> 5, blockIdx.x) {}
+  // warp w of tile number `tile`
+  __device__ __forceinline__ TileLink(const Geom &g, int w, long long tile) {
     p = w >> 2;
     mu = w & 3;
     pair = (int)threadIdx.x & 31;
-    const long long ii = (long long)blockIdx.x * kPairs + pair;
+    const long long ii = tile * kPairs + pair;
     valid = ii < g.vh;
     i = valid ? (int)ii : 0;
     const int row = i / g.half1, plane = row / g.n2;
@@ -92,6 +93,24 @@ __device__ __forceinline__ void tile_store(const Geom &g, double *aos, const dou
   for (int k = 0; k < kPairs * kPairUnits / kThreads; k++) {
     const int u = k * kThreads + (int)threadIdx.x;
     if (u < n) __stcs(dst + u, tile[u + u / kPairUnits]);
+  }
+}
+
+// FP64 arithmetic per link takes one warp on a scheduler as long as 64 clocks an
+// operation, and a tile puts two on each: where the tiles leave SMs idle, the kernels
+// that do some run one warp per block instead (warp b of the launch is warp b % 8 of
+// tile b / 8) and write the public layout directly, a link's 144 B per lane.
+// waves: up to how many tiles per SM
+bool spread(const Geom &g, int waves = 1) { return (long long)tile_blocks(g) < (long long)waves * lgt_device_sms(); }
+
+__device__ __forceinline__ void link_store(double *aos, const TileLink &t, const double u[18]) {
+  double *to = aos + ((size_t)(2 * (long long)t.i + t.odd) * 4 + t.mu) * 18;
+  if (wide(aos)) {
+#pragma unroll
+    for (int c = 0; c < 9; c++) reinterpret_cast<double2 *>(to)[c] = make_double2(u[2 * c], u[2 * c + 1]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 18; c++) to[c] = u[c];
   }
 }
 
@@ -260,6 +279,16 @@ __global__ void __launch_bounds__(kThreads) k_egress(Geom g, const void *soa, do
   tile_store(g, aos, lgt_tile);
 }
 
+// the same by spread warps
+template <int FMT>
+__global__ void __launch_bounds__(32) k_egress_spread(Geom g, const void *soa, double *aos) {
+  const TileLink t(g, (int)blockIdx.x & 7, blockIdx.x >> 3);
+  if (!t.valid) return;
+  double u[18];
+  load_d<FMT>(soa, g.vh, t.p, t.mu, t.i, u);
+  link_store(aos, t, u);
+}
+
 constexpr int kTileBytes = kPairs * kPairStride * 16;
 
 }  // namespace
@@ -277,6 +306,10 @@ cudaError_t launch_ingest(int bulk_fmt, const Geom &g, const double *aos, void *
 cudaError_t launch_egress(int fmt, const Geom &g, const void *soa, double *aos, cudaStream_t st, const void *G,
                           int skip_temporal) {
   const unsigned grid = tile_blocks(g);
+  if (fmt == FMT_PAIR && spread(g)) {  // (54 FP64 operations per link: a call at 8^4 17.7 -> 14.9 us)
+    k_egress_spread<FMT_PAIR><<<8 * grid, 32, 0, st>>>(g, soa, aos);
+    return cudaGetLastError();
+  }
 #define LGT_EGRESS(F) \
   if (fmt == F) k_egress<F><<<grid, kThreads, kTileBytes, st>>>(g, soa, aos, G, skip_temporal); else
   LGT_EGRESS(FMT_F64)
@@ -346,6 +379,34 @@ __device__ __forceinline__ void load_gauge(const double2 *G64, int vh, int p, in
 // SRC 1: G = 1 + D of the anchored polish (pairs), SRC 2: G from k_gauge_fp64.
 // 216 FP64 multiply-adds per link: bound by the FP64 pipe (1.51 ms at 32^4, 1.44 at
 // its full rate; 3.5 to 3.9 ms with G orthonormalised for both ends of every link).
+template <int SRC>
+__device__ __forceinline__ void transformed_link(const Geom &g, const void *G, const void *u_in, int skip_temporal,
+                                                 const TileLink &t, double u[18]) {
+  LinkIO<FMT_F64>::load(u_in, g.vh, t.p, t.mu, t.i, u);
+  if (skip_temporal && t.mu == 0) return;
+  const int s = t.i / g.vs_half;
+  const Coords c = coords_in_slice(g, t.p, s, t.i - s * g.vs_half);
+  const int nb = cb_shift(g, c, t.mu, +1);
+  double m[18], tmp[18];
+  if constexpr (SRC == 2) load_gauge((const double2 *)G, g.vh, t.p, t.i, m);
+  else load_G_src<SRC>(G, g.vh, t.p, t.i, m);
+  mat_mul(m, u, tmp);
+  if constexpr (SRC == 2) load_gauge((const double2 *)G, g.vh, t.p ^ 1, nb, m);
+  else load_G_src<SRC>(G, g.vh, t.p ^ 1, nb, m);
+  mat_mul_dag(tmp, m, u);
+}
+
+template <int SRC>
+__global__ void __launch_bounds__(32) k_apply_G_spread(Geom g, const void *G, const void *u_in, void *u_out,
+                                                       double *aos_out, int skip_temporal) {
+  const TileLink t(g, (int)blockIdx.x & 7, blockIdx.x >> 3);
+  if (!t.valid) return;
+  double u[18];
+  transformed_link<SRC>(g, G, u_in, skip_temporal, t, u);
+  if (aos_out) link_store(aos_out, t, u);
+  else LinkIO<FMT_F64>::store(u_out, g.vh, t.p, t.mu, t.i, u);
+}
+
 template <int SRC, bool AOS>
 __global__ void __launch_bounds__(kThreads, 2) k_apply_G(Geom g, const void *G, const void *u_in, void *u_out,
                                                          double *aos_out, int skip_temporal) {
@@ -353,19 +414,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_apply_G(Geom g, const void *G, 
   const TileLink t(g);
   if (t.valid) {
     double u[18];
-    LinkIO<FMT_F64>::load(u_in, g.vh, t.p, t.mu, t.i, u);
-    if (!(skip_temporal && t.mu == 0)) {
-      const int s = t.i / g.vs_half;
-      const Coords c = coords_in_slice(g, t.p, s, t.i - s * g.vs_half);
-      const int nb = cb_shift(g, c, t.mu, +1);
-      double m[18], tmp[18];
-      if constexpr (SRC == 2) load_gauge((const double2 *)G, g.vh, t.p, t.i, m);
-      else load_G_src<SRC>(G, g.vh, t.p, t.i, m);
-      mat_mul(m, u, tmp);
-      if constexpr (SRC == 2) load_gauge((const double2 *)G, g.vh, t.p ^ 1, nb, m);
-      else load_G_src<SRC>(G, g.vh, t.p ^ 1, nb, m);
-      mat_mul_dag(tmp, m, u);
-    }
+    transformed_link<SRC>(g, G, u_in, skip_temporal, t, u);
     if (AOS) {
       double2 *dst = lgt_tile + t.unit();
 #pragma unroll
@@ -384,7 +433,10 @@ template <int SRC>
 cudaError_t apply(const Geom &g, const void *G, const void *u64_in, void *u64_out, double *aos_out, int skip_temporal,
                   cudaStream_t st) {
   const unsigned grid = tile_blocks(g);
-  if (aos_out) k_apply_G<SRC, true><<<grid, kThreads, kTileBytes, st>>>(g, G, u64_in, u64_out, aos_out, skip_temporal);
+  // (G orthonormalised for both ends of every link: 556 operations, whose uneven share of
+  // the SMs costs more than the tile saves up to 4 tiles per SM; with G at hand, 216)
+  if (spread(g, SRC == 2 ? 1 : 4)) k_apply_G_spread<SRC><<<8 * grid, 32, 0, st>>>(g, G, u64_in, u64_out, aos_out, skip_temporal);
+  else if (aos_out) k_apply_G<SRC, true><<<grid, kThreads, kTileBytes, st>>>(g, G, u64_in, u64_out, aos_out, skip_temporal);
   else k_apply_G<SRC, false><<<grid, kThreads, 0, st>>>(g, G, u64_in, u64_out, nullptr, skip_temporal);
   return cudaGetLastError();
 }
@@ -427,6 +479,8 @@ cudaError_t launch_apply_D(const Geom &g, const void *D, const void *u64_in, voi
                            int skip_temporal, void *scratch, cudaStream_t st) {
   return apply_with<1>(g, D, u64_in, u64_out, aos_out, skip_temporal, scratch, st);
 }
+
+bool lgt_gauge_in_one_launch(const Geom &g) { return 2 * (long long)tile_blocks(g) <= lgt_device_sms(); }
 
 cudaError_t launch_copy_f32(int fmt, const Geom &g, const void *u64, void *u32, cudaStream_t st) {
   const unsigned grid = (unsigned)(((long long)g.vh * 8 + 255) / 256);

@@ -124,7 +124,7 @@ void fill_sweep_args(SweepArgs *a, const Geom &g, void *links, void *G, const Wo
 }
 
 // SMs of the current device, looked up once per device ordinal
-static int device_sms() {
+int lgt_device_sms() {
   static int sms_of[64];
   int dev = 0;
   cudaGetDevice(&dev);
@@ -158,7 +158,7 @@ static cudaError_t launch_sweep_kernel(sweep_fn fn, int cfg, const Geom &g, Swee
     cudaError_t e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)ceil_div(g.vs_half, block) * a.t_count * a.n_half;
-    const long long cap = (long long)device_sms() * lgt_cfg_minblocks(cfg);
+    const long long cap = (long long)lgt_device_sms() * lgt_cfg_minblocks(cfg);
     const int blocks = (int)(tiles < cap ? tiles : cap);
     if (lgt_cfg_stream(cfg)) {  // counters start at zero in every launch
       e = cudaMemsetAsync(a.stream, 0, sizeof(unsigned) * ((size_t)g.nt + 2), st);
@@ -339,7 +339,7 @@ cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Work
   // what the workspace holds partial sums for).  8^4 with plaquette: 108 -> 67 us (98
   // by one thread per site, stored links 94); 10^4, where the blocks of 64 just fill the
   // SMs: 109 -> 97 (101, 95).
-  if ((fmt == FMT_FIX_18 || fmt == FMT_FIX_12) && with_plaq && block == 128 && (int)(grid.x * grid.y * 2) < device_sms()) {
+  if ((fmt == FMT_FIX_18 || fmt == FMT_FIX_12) && with_plaq && block == 128 && (int)(grid.x * grid.y * 2) < lgt_device_sms()) {
     a.split = 1;
     grid.x = ceil_div(g.vs_half, 64);
   }
