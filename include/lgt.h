@@ -130,7 +130,8 @@ typedef struct {
   uint64_t seed;              /* key of the SR random stream */
   uint64_t sweep_offset;      /* index of the first sweep (RNG counter; resume) */
   double theta_tol;           /* requested precision, e.g. 1e-14 */
-  double theta_switch;        /* bulk FP32 -> FP64 switch threshold (ignored for FP64) */
+  double theta_switch;        /* bulk FP32 -> FP64 switch threshold (ignored for FP64; with fixed
+                                 links, see below, 2e-12 at least) */
   int32_t max_sweeps;         /* cap on sweeps of one lgt_fix call (all phases) */
   int32_t check_every;        /* exact theta check every k sweeps */
   int32_t reunit_every;       /* reunitarise FP32 links / G every n sweeps (0: never) */
