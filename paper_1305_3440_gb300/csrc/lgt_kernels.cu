@@ -337,8 +337,8 @@ cudaError_t launch_measure(int fmt, const Geom &g, const void *links, const Work
   // chain.  The FP64 pipe hides that where warps are many; on a lattice whose blocks
   // leave SMs idle, two threads take a site's plaquettes instead (64 sites per block:
   // what the workspace holds partial sums for).  8^4 with plaquette: 108 -> 67 us (98
-  // by one thread per site, stored links 94); 10^4, where the blocks of 64 just fill the
-  // SMs: 109 -> 97 (101, 95).
+  // by one thread per site, stored links 94); 10^4, where the blocks of 64 are a
+  // few more than the SMs: 109 -> 97 to 99 (101, 95).
   if ((fmt == FMT_FIX_18 || fmt == FMT_FIX_12) && with_plaq && block == 128 && (int)(grid.x * grid.y * 2) < lgt_device_sms()) {
     a.split = 1;
     grid.x = ceil_div(g.vs_half, 64);

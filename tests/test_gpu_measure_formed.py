@@ -29,7 +29,7 @@ def test_values_are_those_of_the_links_read_back(lgt, dims, bulk):
     assert np.allclose(F_t, mc["F_t"], rtol=0, atol=1e-13) and np.allclose(th_t, mc["theta_t"], rtol=1e-13, atol=0)
 
 
-@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (8, 8, 8, 8), (10, 10, 10, 10)])
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (8, 8, 8, 8)])
 def test_a_formed_field_takes_no_longer_to_measure_than_a_stored_one(lgt, dims):
     """Device time of a measurement with plaquette after a sweep, against a context whose
     sweeps rewrite their links (launch_config named): at most 1.05 of it."""
